@@ -170,6 +170,10 @@ struct kvc_ctx {
   // Last append (queries of the following attention calls).
   bool attn_valid = false;
   int last_n_seq = 0, last_total = 0, last_max_t = 0;
+  // Estimates of its sessions' resident pages (largest, sum): what was fed, capped at what the
+  // eviction policy is to keep.  They guide the choice of the attention's split only.
+  int est_pages_max = 0;
+  int64_t est_pages_sum = 0;
   int attn_since_append = 0;  // attention launches since the last append (or layer write)
   uint64_t layers_written = 0;  // layers whose K/V of the last append are in the pool
   bool last_single = false;
@@ -372,6 +376,17 @@ int kvc_append_chunk(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, const i
     ctx->tail_mod[sid] = (ctx->tail_mod[sid] + t) % PS;
     ctx->pos_next[sid] += t;
   }
+  const int64_t keep = ctx->cfg.policy == KVC_POLICY_SINK_RECENT
+                           ? (int64_t)ctx->cfg.sink + ctx->cfg.recent
+                           : (ctx->cfg.budget >= 0 ? ctx->cfg.budget : INT64_MAX / 2);
+  ctx->est_pages_max = 0;
+  ctx->est_pages_sum = 0;
+  for (int i = 0; i < n_seq; ++i) {
+    const int64_t fed = ctx->pos_next[h_sessions[i]], t = h_cu_tokens[i + 1] - h_cu_tokens[i];
+    const int pages = (int)(std::min(fed, keep + t) / PS + 1);
+    ctx->est_pages_max = std::max(ctx->est_pages_max, pages);
+    ctx->est_pages_sum += pages;
+  }
   ctx->used_ub += need;
   ctx->delta_since_readback += need;
   ctx->attn_valid = true;
@@ -516,6 +531,7 @@ int kvc_attn_prefill_chunk(kvc_ctx* ctx, int layer, const void* d_q, void* d_out
   if (ctx->last_max_t > PF_MAX_TOKENS)
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
   KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
+                               ctx->est_pages_max, ctx->est_pages_sum,
                                ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream)));
   ++ctx->attn_since_append;
   return KVC_OK;
@@ -537,11 +553,13 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
     // copied only after its rows are written, and the previous launch writes
     // another layer's rows only.
     KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
+                               ctx->est_pages_max, ctx->est_pages_sum,
                                  ctx->attn_since_append > 0, s, d_k, d_v));
   } else {
     // Binary32 (CUDA-core prefill): the rows first, then the attention, unoverlapped.
     KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, s));
     KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
+                               ctx->est_pages_max, ctx->est_pages_sum,
                                  false, s));
   }
   ctx->layers_written |= 1ull << layer;

@@ -1,294 +1,287 @@
 // Chunked-prefill GQA attention on the 5th-generation tensor cores (tcgen05 +
 // TMEM), bfloat16 K/V/q, fp32 softmax and accumulation.
 //
-// The call's (session, KV head, page) units are cut into equal contiguous
-// ranges, one per CTA (stream-K); per segment (the part of one (session, KV
-// head) pair in a range) the T*G query rows (T <= 32 tokens, G = 4 heads) form
-// the M = 128 rows of an MMA tile, the rows past T*G being zero padding.  A
-// pair split over several CTAs is merged by the last of them (log-sum-exp).
-// Warp roles in one CTA:
-//   warps 0, 6 producers: 2-D TMA loads (128-byte swizzle) of the K (warp 0)
-//             and V (warp 6) tiles of 4 pages (64 keys) per stage into a
-//             shared-memory ring whose K and V halves are released separately;
-//   warps 1, 7 MMA issuers: one elected thread each issues tcgen05.mma, warp
-//             1 S = Q K^T (N = 64, Q from TMEM, K from shared memory) into a
-//             double-buffered TMEM tile, warp 7 O += P V (N = 128, P from
-//             TMEM, V from shared memory) into TMEM; completion is signalled
-//             with tcgen05.commit on mbarriers;
-//   warps 2-5 softmax: each thread owns one TMEM lane (= one query row):
-//             it builds its rotated, scaled query row in shared memory,
-//             reads its row of S from TMEM, masks (resident slots, causal
-//             inside the chunk), keeps the running max/sum, writes P as
-//             bfloat16 to a swizzled shared buffer, rescales O in TMEM when
-//             the row maximum grows by more than 2^8, and finally reads O.
+// A segment is a run of pages of one (session, KV head) pair; the pair's T*G query rows
+// (T <= 32 tokens, G = 4 heads) form the M = 128 rows of an MMA tile, the rows past T*G
+// being zero padding.  Two ways to cut a call into segments:
+//   - pair split (CLUSTER): each pair's pages are cut into k slices, one CTA each.  The k
+//     CTAs of a pair are a thread-block cluster: every CTA sends its partial rows (O, max,
+//     sum) to the CTAs that own them through distributed shared memory, and each merges
+//     and writes its share of the rows;
+//   - stream-K: the call's (session, KV head, page) units are cut into equal contiguous
+//     ranges, one per CTA; a pair split over several CTAs is merged by the last of them to
+//     finish (log-sum-exp over partial states in global memory).
+// Warp roles in one CTA (384 threads, one CTA per SM):
+//   warps 0, 1 producers: 2-D TMA loads (128-byte swizzle) of the K (warp 0) and V (warp 1)
+//              tiles of 4 pages (64 keys) per stage, one box per lane, into a ring whose K
+//              and V halves are released separately;
+//   warps 2, 3 MMA issuers: one elected thread each, warp 2 S = Q K^T (N = 64, Q from
+//              TMEM, K from shared memory), warp 3 O += P V (N = 128, P from TMEM, V from
+//              shared memory); completion is signalled with tcgen05.commit on mbarriers;
+//   warps 4-7, 8-11 two softmax groups that take the stages in turn: a thread owns one
+//              TMEM lane (= one query row); it reads its row of S, masks (resident slots,
+//              causal inside the chunk), keeps a running max/sum and writes P as bfloat16.
+//              Each group has its own S and P tiles, its own output accumulator and its own
+//              running state, so that the groups never wait for one another inside a
+//              segment; the two states are merged when it ends.  O is rescaled in TMEM when
+//              a row's maximum grows by more than 2^8.
 // All waits are bounded; a timeout records KVC_DERR_WAIT and the CTA stops.
+//
+// What bounds it: from about 18 sessions of 8 KV heads on HBM (64 sessions of 4,100
+// positions: 167 us per launch, 6.55 TB/s of K/V, q and output bytes; one softmax group with
+// a stage's boxes issued by one lane and a thread per row for q, partial states and outputs
+// took 193); below that, a stage of a lone CTA takes 0.6 us, the issue of S = Q K^T (10
+// instructions of about 70 cycles; one softmax group: 0.8 us), and a launch about 7 us beside
+// its stages (1 session: 48.1 -> 12.7 us, most of it the merge of 16 parts by one CTA;
+// 9 sessions: 48.6 -> 31 us).  Under load every access that misses L2 waits behind the K/V
+// bytes in flight (about 4 us with a full ring on every SM).  So the queries and rotary rows
+// of the next segment are copied while the current one runs, K and V carry an evict-first
+// hint that keeps them, the rotary table and the partial states in L2, and in the stream-K
+// split nothing waits for the arrival of a range's first partial segment.
 #include <cuda.h>
 
-#include "kvc_launch.cuh"
-#include "kvc_rope.cuh"
+#include "kvc_prefill_tc.cuh"
 
 namespace kvc {
 
 namespace {
 
-constexpr int G = 4;
-constexpr int D = 128;
-constexpr int M = 128;                       // MMA rows (query rows, padded)
-constexpr int NK = 64;                       // keys per stage (4 pages)
-constexpr int TC_STAGES = 6;                 // K/V stages of the ring (a 7-stage ring measured slower)
-constexpr int KV_PANEL = NK * 128;           // 64 rows x 128 B = 8 KiB
-constexpr int STAGE = 4 * KV_PANEL;          // K lo, K hi, V lo, V hi = 32 KiB
-// Tensor memory (512 columns x 128 lanes of 32 bits; lane = query row):
-//   S0 [0,64) S1 [64,128)  fp32 scores of two stages
-//   O  [128,256)           fp32 output accumulator
-//   P0 [256,288) P1 [288,320)  bfloat16 probabilities (2 per column), MMA A operand
-//   Q  [320,384)           bfloat16 rotated, scaled query rows, MMA A operand
+// Tensor memory (512 columns x 128 lanes of 32 bits; lane = query row), group g:
+//   S_g [64 g, +64)        fp32 scores of a stage
+//   O_g [128 + 128 g, +128) fp32 output accumulator
+//   P_g [384 + 32 g, +32)  bfloat16 probabilities (2 per column), MMA A operand
+//   Q   [448, 512)         bfloat16 rotated, scaled query rows, MMA A operand
 constexpr int TMEM_COLS = 512;
-constexpr int S_COL = 0, O_COL = 128, P_COL = 256, Q_COL = 320;
-constexpr float LOG2E = 1.4426950408889634f;
-constexpr float RESCALE_LOG2 = 8.f;          // rescale O only when the max grows by > 2^8
-constexpr int THREADS = 8 * 32;
-constexpr int PF_MIN_UNITS = 16;              // pages per CTA of the stream-K split, at least
+constexpr int S_COL = 0, O_COL = 128, P_COL = 384, Q_COL = 448;
+constexpr int THREADS = 12 * 32;
+constexpr int SM_THREADS = 8 * 32;           // softmax threads
+constexpr int PF_MIN_UNITS = 16;             // pages per CTA of the stream-K split, at least
 constexpr int PF_MAX_PARTS = 1 << 16;        // no limit on CTAs per pair (merged row by row)
-constexpr unsigned FULL = 0xFFFFFFFFu;
+constexpr int MAX_RING = 6;                  // K/V stages of the ring, at most
+constexpr int MAX_K = 8;                     // slices of a pair (cluster size), at most
 
-// Shared memory map (offsets from a 1024-aligned base): the K/V ring, barriers.
-constexpr int OFF_KV = 0;
-constexpr int OFF_BAR = OFF_KV + TC_STAGES * STAGE;
+// Shared memory map (offsets from a 1024-aligned base): barriers and (max, sum) pairs
+// first, then the K/V ring, then (CLUSTER) the partial rows sent to this CTA.
 enum {
-  B_K_FULL = 0,                          // [TC_STAGES] K half of a stage loaded
-  B_K_EMPTY = B_K_FULL + TC_STAGES,      // [TC_STAGES] ... and read by S = Q K^T
-  B_V_FULL = B_K_EMPTY + TC_STAGES,      // [TC_STAGES] V half loaded
-  B_V_EMPTY = B_V_FULL + TC_STAGES,      // [TC_STAGES] ... and read by O += P V
-  B_S_FULL = B_V_EMPTY + TC_STAGES,      // [2]
-  B_S_EMPTY = B_S_FULL + 2,              // [2]
-  B_P_FULL = B_S_EMPTY + 2,              // [2]
-  B_P_EMPTY = B_P_FULL + 2,              // [2]
-  // [2] P V product j complete: barrier j % 2, phase j / 2.  One barrier per P
-  // buffer keeps every waiter at most one phase behind (P V products j - 3 and
-  // earlier are known complete when j is waited for), so parity waits are exact.
-  B_O = B_P_EMPTY + 2,
-  B_Q = B_O + 2,                         // one phase per segment (query tile ready)
-  B_FINAL = B_Q + 1,                     // every MMA of the CTA complete (both issuers)
+  B_K_FULL = 0,                          // [MAX_RING] K half of a stage loaded
+  B_K_EMPTY = B_K_FULL + MAX_RING,       // [MAX_RING] ... and read by S = Q K^T
+  B_V_FULL = B_K_EMPTY + MAX_RING,       // [MAX_RING] V half loaded
+  B_V_EMPTY = B_V_FULL + MAX_RING,       // [MAX_RING] ... and read by O += P V
+  // Per group, one phase per stage of the group (its j-th stage is stage 2 j + g of the
+  // CTA).  Every waiter has seen the phase before the one it waits for, so parity waits are
+  // exact.
+  B_S_FULL = B_V_EMPTY + MAX_RING,       // [2] scores complete
+  B_S_EMPTY = B_S_FULL + 2,              // [2] scores read by the group's warps
+  B_P_FULL = B_S_EMPTY + 2,              // [2] probabilities written
+  B_PV = B_P_FULL + 2,                   // [2] O += P V complete
+  B_Q = B_PV + 2,                        // one phase per segment (query tile ready)
   // Fused layer write: one phase per segment holding chunk slots, completed when the
   // softmax warps have written those rows into the pool.
-  B_ROWS = B_FINAL + 1,
-  N_BARS = B_ROWS + 1
+  B_ROWS = B_Q + 1,
+  B_FINAL = B_ROWS + 1,                  // every MMA of the CTA complete (both issuers)
+  B_RECV = B_FINAL + 1,                  // CLUSTER: every part of this CTA's rows received
+  // Stream-K: the first segment's partial state is in global memory (warp 1 arrives for the
+  // pair then); warp 1 has looked whether the last segment's other parts are all there.
+  B_PUB = B_RECV + 1,
+  B_PEEK = B_PUB + 1,
+  N_BARS = B_PEEK + 1
 };
+constexpr int OFF_ML = 0;                              // [2][M] (max, sum) of the groups
+constexpr int OFF_BAR = OFF_ML + 2 * M * 8;
 constexpr int OFF_TMEM_ADDR = OFF_BAR + N_BARS * 8;
-constexpr int TC_SMEM = OFF_TMEM_ADDR + 16 + 1024;  // + alignment slack
-static_assert(TC_SMEM <= 227 * 1024, "shared memory per CTA");
+constexpr int OFF_SEQ = OFF_TMEM_ADDR + 16;            // [SEQ_CACHE] sessions of the range
+constexpr int SEQ_CACHE = 8;
+constexpr int OFF_KV = 3 * 1024;
+static_assert(OFF_SEQ % 16 == 0 && OFF_SEQ + SEQ_CACHE * sizeof(SeqInfo) <= OFF_KV &&
+                  OFF_KV % 1024 == 0, "header fits");
+// A partial row sent to its owner: D binary32 values, then (max, sum) in the padding that
+// keeps the rows apart in the banks.
+constexpr int ROW_PITCH = (D + 4) * 4;
+// Staged rows, padded likewise: query and rotary rows on their way to tensor memory, output
+// rows on their way out.  With a thread per row a warp's global accesses would touch 32 lines
+// each.
+constexpr int ST_PITCH = D * 2 + 16, ROPE_PITCH = D * 4 + 16;
+constexpr int SMEM_MAX = 227 * 1024 - 256;   // (the rest: static shared memory)
 
-// -- tcgen05 helpers ------------------------------------------------------------------
-__device__ inline void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                   smem_u32(smem_dst)),
-               "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+// After the ring of `ring` stages: the query rows of max_t tokens, their rotary rows, then
+// the output rows or (CLUSTER, k > 1) the `recv` received rows.
+__host__ __device__ constexpr int off_q(int ring) { return OFF_KV + ring * STAGE; }
+__host__ __device__ constexpr int off_rope(int ring, int max_t) {
+  return off_q(ring) + max_t * G * ST_PITCH;
 }
-__device__ inline void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-               : "memory");
+__host__ __device__ constexpr int off_out(int ring, int max_t) {
+  return off_rope(ring, max_t) + max_t * ROPE_PITCH;
 }
-__device__ inline void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+constexpr int tc_smem(int ring, int max_t, int recv) {
+  return 1024 + off_out(ring, max_t) + (recv > 0 ? recv * ROW_PITCH : max_t * G * ST_PITCH);
 }
-__device__ inline void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+static_assert(M * ROW_PITCH <= 3 * STAGE, "a CTA's partial rows fit a ring of three stages");
+
+__device__ inline void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ inline void tc_commit(uint64_t* bar) {
+__device__ inline void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Address of this CTA's shared address `saddr` in CTA `rank` of the cluster.
+__device__ inline uint32_t cluster_map(uint32_t saddr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+// Bulk copy of `bytes` (a multiple of 16) to shared address `dst` of a CTA of the cluster,
+// completing on `bar` (an address in that CTA too).
+__device__ inline void bulk_s2cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(dst),
+      "r"(src), "r"(bytes), "r"(bar)
       : "memory");
-}
-// D (TMEM) (+)= A B with A read from tensor memory (M lanes, K/2 columns of
-// bfloat16 pairs) and B from shared memory.
-__device__ inline void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                 uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Each thread of the warp reads 32 consecutive fp32 columns of its TMEM lane.
-__device__ inline void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-        "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ inline void tmem_st32(uint32_t taddr, const uint32_t* w) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-      "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(
-          taddr),
-      "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]),
-      "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]),
-      "r"(w[15]), "r"(w[16]), "r"(w[17]), "r"(w[18]), "r"(w[19]), "r"(w[20]), "r"(w[21]),
-      "r"(w[22]), "r"(w[23]), "r"(w[24]), "r"(w[25]), "r"(w[26]), "r"(w[27]), "r"(w[28]),
-      "r"(w[29]), "r"(w[30]), "r"(w[31])
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-__device__ inline void tmem_st32(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-      "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(
-          taddr),
-      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-      "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-      "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-      "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-      "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-      "r"(__float_as_uint(v[15])), "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])),
-      "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])), "r"(__float_as_uint(v[20])),
-      "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-      "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])),
-      "r"(__float_as_uint(v[27])), "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])),
-      "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle: `sbo` bytes between 8-row
-// groups; `lbo` bytes between 64-element groups of the contiguous dimension
-// (MN-major operands only).
-__device__ inline uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;  // 128-byte swizzle
-  return d;
+__device__ inline void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// A segment: units [u, end) of the pair (session seq of the call, KV head) whose units are
+// [pair_start, pair_end); nb pages per pair of the session.
+struct PSeg {
+  int seq, head, nb, pair_start, pair_end, u, end;
+  __device__ int blk() const { return u - pair_start; }
+  __device__ int n_blk() const { return end - u; }
+  __device__ int n_st() const { return (end - u + 3) / 4; }
+  __device__ bool whole() const { return u == pair_start && end == pair_end; }
+};
+
+// Session of the call that holds unit u (one warp; one round trip for 32 sessions each).
+__device__ inline int session_of_unit(const Dev& d, int u, int lane) {
+  const int n_seq = d.g->n_seq;
+  int n = 0;
+  for (int i = lane; i < n_seq + lane; i += 32)
+    n += __popc(__ballot_sync(FULL, i < n_seq && d.seq[i].unit_base <= u));
+  return n - 1;
 }
 
-// The per-layer write of the chunk rows of tokens [t0, t1) of a session (its call
-// row q_row0, positions from pos_first) for KV head `head`, by the 128 softmax
-// threads (thread index ts): V rows copied, K rows rotated at their positions, in
-// 16-byte chunks, every load of an item issued before its stores.  Each thread then
-// orders its writes before later tensor copies (async proxy).
-__device__ inline void write_chunk_rows(const Dev& d, int layer, const SeqInfo& si, int head,
-                                        const __nv_bfloat16* new_k, const __nv_bfloat16* new_v,
-                                        int t0, int t1, int ts) {
-  // Item (token, c): 16-byte chunk c of the first half of the K row with its
-  // rotate-half partner, and chunks c and c + 8 of the V row.
-  constexpr int VEC = 8, HALF = D / 2, KC = HALF / VEC;
-  __nv_bfloat16* pool = reinterpret_cast<__nv_bfloat16*>(d.pool);
-  const int H = d.kv_heads;
-  const int n = (t1 - t0) * KC;
-  for (int idx = ts; idx < n; idx += 128) {
-    const int t = t0 + idx / KC, c = idx % KC;
-    const size_t in_row = ((size_t)(si.q_row0 + t) * H + head) * D + c * VEC;
-    const uint4 ka = *reinterpret_cast<const uint4*>(new_k + in_row);
-    const uint4 kb = *reinterpret_cast<const uint4*>(new_k + in_row + HALF);
-    const uint4 va = *reinterpret_cast<const uint4*>(new_v + in_row);
-    const uint4 vb = *reinterpret_cast<const uint4*>(new_v + in_row + HALF);
-    const float2* t2 = d.rope + (size_t)(si.pos_first + t) * HALF + c * VEC;
-    float2 cs[VEC];
+// The segment that starts at unit u of a range ending at u_end, in session seq.
+__device__ inline PSeg segment_at(const SeqInfo& si, int seq, int u, int u_end) {
+  PSeg s;
+  s.seq = seq;
+  s.nb = si.n_blocks;
+  s.head = (u - si.unit_base) / s.nb;
+  s.pair_start = si.unit_base + s.head * s.nb;
+  s.pair_end = s.pair_start + s.nb;
+  s.u = u;
+  s.end = min(u_end, s.pair_end);
+  return s;
+}
+
+// The only segment of a CTA of the pair split: stages (groups of 4 pages) of slice
+// blockIdx.x % k of pair blockIdx.x / k; empty if the pair has fewer stages than slices.
+__device__ inline PSeg slice_segment(const Dev& d, int k) {
+  const int pair = blockIdx.x / k, slice = blockIdx.x % k;
+  PSeg s;
+  s.seq = pair / d.kv_heads;
+  s.head = pair % d.kv_heads;
+  const int nb = d.seq[s.seq].n_blocks, n_all = (nb + 3) / 4;
+  s.nb = nb;
+  s.pair_start = d.seq[s.seq].unit_base + s.head * nb;
+  s.pair_end = s.pair_start + nb;
+  s.u = s.pair_start + min(nb, 4 * (int)((int64_t)slice * n_all / k));
+  s.end = s.pair_start + min(nb, 4 * (int)((int64_t)(slice + 1) * n_all / k));
+  return s;
+}
+
+// Rows of partial slot `slot`: [D / 4 chunks][M rows] of 16 bytes, so that the threads of a
+// warp, a row each, access them side by side.
+__device__ inline float4* part_rows(const Dev& d, int slot) {
+  return reinterpret_cast<float4*>(d.pf_part_o + (size_t)slot * (M * D));
+}
+
+__device__ inline int us_first_part(const UnitSplit& us, const PSeg& s) {
+  return us.U > 0 ? us.owner(s.pair_start) : 0;
+}
+
+// Log-sum-exp merge of the nch parts of segment s's pair (CTAs cf .. cf + nch - 1) by the
+// softmax threads, columns [64 grp, +64) of row r each; columns [64 grp + 32 c, +32) go to
+// store(c, .).  Part own_ch (this CTA's, of maximum Mr and sum Lr) comes from own(c, scale,
+// .); own_ch < 0: every part from its slot.  The first other part's columns are loaded
+// together with its (max, sum), so a pair of two parts costs one round trip.
+template <typename OwnFn, typename StoreFn>
+__device__ inline void merge_parts(const Dev& d, const UnitSplit& us, const PSeg& s, int cf,
+                                   int nch, int own_ch, bool write, int r, int grp, float Mr,
+                                   float Lr, OwnFn own, StoreFn store) {
+  const int first_slot = us.slot_of(cf, cf, s.pair_start);
+  auto slot_of = [&](int ch) { return ch ? 2 * (cf + ch) : first_slot; };
+  auto part4 = [&](int ch, int i) {  // 16-byte chunk i of the half row
+    return write ? __ldcg(part_rows(d, slot_of(ch)) + (16 * grp + i) * M + r)
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  auto part_ml = [&](int ch) {
+    return write && ch != own_ch ? __ldcg(&d.pf_part_ml[(size_t)slot_of(ch) * M + r])
+                                 : make_float2(-INFINITY, 0.f);
+  };
+  const int f0 = own_ch == 0 ? 1 : 0;  // first other part
+  float4 v[16];
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) cs[e] = t2[e];
-    const int gs = d.tok_slot[si.q_row0 + t];
-    float xa[VEC], xb[VEC], ya[VEC], yb[VEC];
-    Chunk16<__nv_bfloat16>::unpack(ka, xa);
-    Chunk16<__nv_bfloat16>::unpack(kb, xb);
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) rope_pair(xa[e], xb[e], cs[e], ya[e], yb[e]);
-    __nv_bfloat16* kd = pool + pool_offset_elems(d, gs / PS, layer, 0, head, gs % PS) + c * VEC;
-    __nv_bfloat16* vd = pool + pool_offset_elems(d, gs / PS, layer, 1, head, gs % PS) + c * VEC;
-    *reinterpret_cast<uint4*>(kd) = Chunk16<__nv_bfloat16>::pack(ya);
-    *reinterpret_cast<uint4*>(kd + HALF) = Chunk16<__nv_bfloat16>::pack(yb);
-    *reinterpret_cast<uint4*>(vd) = va;
-    *reinterpret_cast<uint4*>(vd + HALF) = vb;
+  for (int i = 0; i < 16; ++i) v[i] = part4(f0, i);
+  const float2 mlf = part_ml(f0);
+  const float m_own = write ? Mr : -INFINITY;
+  float Mx = fmaxf(m_own, mlf.x);
+  for (int ch = f0 + 1; ch < nch; ++ch) Mx = fmaxf(Mx, part_ml(ch).x);
+  const float s_own = exp2_safe(m_own, Mx), s_f = exp2_safe(mlf.x, Mx);
+  float Ls = Lr * s_own + mlf.y * s_f;
+  for (int ch = f0 + 1; ch < nch; ++ch) {
+    const float2 ml = part_ml(ch);
+    Ls += ml.y * exp2_safe(ml.x, Mx);
   }
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
-// Chunk tokens [t0, t1) of a session whose slots lie in its blocks [b_lo, b_hi).
-__device__ inline void chunk_tokens_in(const SeqInfo& si, int b_lo, int b_hi, int& t0, int& t1) {
-  const int sl_first = si.live_head + si.n_live - si.t;  // live slot of the first token
-  const int lo = (b_lo - si.n_hist_pages) * PS, hi = (b_hi - si.n_hist_pages) * PS;
-  t0 = max(0, lo - sl_first);
-  t1 = min(si.t, hi - sl_first);
-}
-
-// Instruction descriptor, kind::f16: D fp32, A and B bf16, A K-major, B K- or MN-major.
-__host__ __device__ constexpr uint32_t instr_desc(int n, int m, bool b_mn_major) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) |
-         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-__device__ inline uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-
-__device__ inline float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// The segment after `s` in a range ending at u_end, given s.end < u_end: s then ends
-// at its pair's end, and the next segment is the next pair from its first unit, the
-// session's next KV head or the next session's first one.  Unlike unit_segment, no
-// search over the sessions (a chain of dependent loads) is needed.
-__device__ inline UnitSeg next_segment(const Dev& d, const UnitSeg& s, int u_end) {
-  UnitSeg n;
-  if (s.head + 1 < d.kv_heads) {
-    n.seq = s.seq;
-    n.si = s.si;
-    n.head = s.head + 1;
-  } else {
-    n.seq = s.seq + 1;
-    n.si = d.seq[n.seq];
-    n.head = 0;
+  const float inv = 1.f / Ls;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    float o[32];
+    own(c, s_own * inv, o);
+    auto add = [&](int i, const float4& w, float sc) {
+      o[4 * i] = fmaf(w.x, sc, o[4 * i]);
+      o[4 * i + 1] = fmaf(w.y, sc, o[4 * i + 1]);
+      o[4 * i + 2] = fmaf(w.z, sc, o[4 * i + 2]);
+      o[4 * i + 3] = fmaf(w.w, sc, o[4 * i + 3]);
+    };
+#pragma unroll
+    for (int i = 0; i < 8; ++i) add(i, v[8 * c + i], s_f * inv);
+    for (int ch = f0 + 1; ch < nch; ++ch) {  // pairs over three or more CTAs
+      if (ch == own_ch) continue;
+      const float sc = exp2_safe(part_ml(ch).x, Mx) * inv;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) add(i, part4(ch, 8 * c + i), sc);
+    }
+    store(c, o);
   }
-  const int nb = n.si.n_blocks;
-  n.pair_start = n.si.unit_base + n.head * nb;
-  n.pair_end = n.pair_start + nb;
-  n.u = s.end;
-  n.end = min(u_end, n.pair_end);
-  return n;
 }
 
 // FUSED (the per-layer order): the chunk's K (rotated at each token's position) and
 // V of this layer are not in the pool yet; new_k / new_v hold them ([total][Hkv][D],
-// the append's token order).  The producer warp that loads a stage holding chunk
-// slots of its (session, head) first writes those rows into the pool (the CTA
-// owning a (session, head, page) unit is the only reader of that unit in the
-// launch), then orders the writes before its tensor copy of the stage.
-template <bool FUSED>
+// the append's token order).  The softmax warps write the rows of a segment's chunk
+// slots into the pool when the segment starts (the CTA owning a (session, head, page)
+// unit is the only reader of that unit in the launch), and the producers copy a stage
+// holding such slots only after that.
+template <bool FUSED, bool CLUSTER>
 __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     Dev d, int layer, const __grid_constant__ CUtensorMap map_lo,
     const __grid_constant__ CUtensorMap map_hi, const __nv_bfloat16* __restrict__ q,
-    __nv_bfloat16* __restrict__ out, float qk_scale, const __nv_bfloat16* __restrict__ new_k,
-    const __nv_bfloat16* __restrict__ new_v) {
+    __nv_bfloat16* __restrict__ out, float qk_scale, int ring, int max_t, int k_slices,
+    const __nv_bfloat16* __restrict__ new_k, const __nv_bfloat16* __restrict__ new_v) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  // (The same offset in every CTA, so that cluster_map() of an address finds the peer's.)
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_TMEM_ADDR);
-  __shared__ int s_abort_flag, s_last;
+  __shared__ int s_abort_flag, s_last, s_peek, s_first_last;
   volatile int& s_abort = s_abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
+  const int H = d.kv_heads, L = d.layers;
+  if (CLUSTER && d.g->n_units == 0) return;  // the append failed: nothing to do for any CTA
   if (tid == 0) {
-    for (int s = 0; s < TC_STAGES; ++s) {
+    for (int s = 0; s < ring; ++s) {
       mbar_init(&bars[B_K_FULL + s], 1);
       mbar_init(&bars[B_K_EMPTY + s], 1);
       mbar_init(&bars[B_V_FULL + s], 1);
@@ -298,22 +291,64 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       mbar_init(&bars[B_S_FULL + s], 1);
       mbar_init(&bars[B_S_EMPTY + s], 4);
       mbar_init(&bars[B_P_FULL + s], 4);
-      mbar_init(&bars[B_P_EMPTY + s], 1);
+      mbar_init(&bars[B_PV + s], 1);
     }
-    mbar_init(&bars[B_O + 0], 1);
-    mbar_init(&bars[B_O + 1], 1);
-    mbar_init(&bars[B_Q], 4);
+    mbar_init(&bars[B_Q], 8);
+    mbar_init(&bars[B_ROWS], 8);
     mbar_init(&bars[B_FINAL], 2);
-    mbar_init(&bars[B_ROWS], 4);
+    mbar_init(&bars[B_RECV], 1);
+    mbar_init(&bars[B_PUB], 1);
+    mbar_init(&bars[B_PEEK], 1);
     fence_mbar_init();
     s_abort = 0;
+    s_first_last = 0;
   }
-  // Zero the K/V ring once: the keys of partly filled stages only ever hold finite
-  // values (their weights are 0, and 0 times a stale NaN would not be 0).
-  for (int i = tid; i < OFF_BAR / 16; i += THREADS)
-    reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  fence_proxy_async_smem();
-  if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
+  // This CTA's range of units.
+  UnitSplit us = {};
+  PSeg seg = {};
+  int u_begin, u_end;
+  const int cta = blockIdx.x;
+  SeqInfo* s_seq = reinterpret_cast<SeqInfo*>(smem + OFF_SEQ);
+  if constexpr (CLUSTER) {
+    seg = slice_segment(d, k_slices);
+    u_begin = seg.u;
+    u_end = seg.end;
+  } else {
+    us = unit_split(d, gridDim.x, PF_MIN_UNITS, PF_MAX_PARTS);
+    const bool active = cta < us.n_cta;
+    u_begin = active ? us.start_of(cta) : 0;
+    u_end = active ? us.start_of(cta + 1) : 0;
+    if (u_begin < u_end) seg.seq = session_of_unit(d, u_begin, lane);
+  }
+  // The sessions that the range can touch first, for every role (info()).
+  const int seq0 = seg.seq;
+  if (tid < SEQ_CACHE * 16 && seq0 + tid / 16 < d.g->n_seq)
+    reinterpret_cast<int*>(s_seq)[tid] = reinterpret_cast<const int*>(d.seq + seq0)[tid];
+  auto info = [&](int seq) -> const SeqInfo& {
+    return seq - seq0 < SEQ_CACHE ? s_seq[seq - seq0] : d.seq[seq];
+  };
+  if (CLUSTER && k_slices > 1) {
+    // Rows [rank R / k, (rank + 1) R / k) of the pair are CTA rank's to merge and write: it
+    // receives k parts of each.  Arrival: this CTA has started and its barrier expects them.
+    if (tid == 0) {
+      const int R = d.seq[seg.seq].t * G, k = k_slices, slice = cta % k;
+      mbar_arrive_expect_tx(&bars[B_RECV], k * ((slice + 1) * R / k - slice * R / k) * ROW_PITCH);
+    }
+    __syncwarp();
+    cluster_arrive();
+  }
+  // The V rows that a partly filled stage leaves unwritten in the ring's first pass have to
+  // be finite (their weights are 0, and 0 times a NaN would not be 0); later passes find
+  // pool values there.
+  {
+    const int n_v = CLUSTER ? min(ring, (u_end - u_begin + 3) / 4) : ring;
+    for (int s = CLUSTER ? max(0, n_v - 1) : 0; s < n_v; ++s) {
+      uint4* v = reinterpret_cast<uint4*>(smem + OFF_KV + s * STAGE + 2 * KV_PANEL);
+      for (int i = tid; i < 2 * KV_PANEL / 16; i += THREADS) v[i] = make_uint4(0, 0, 0, 0);
+    }
+    fence_proxy_async_smem();
+  }
+  if (warp == 2) tmem_alloc(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -321,41 +356,58 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
   // Before pdl_wait() only the append's data is read (work list, page tables, K/V
   // pages); the softmax warps wait before reading q or writing any result.
   pdl_launch_dependents();
-
-  const int H = d.kv_heads, L = d.layers;
-  // Stream-K: this CTA's contiguous range of the call's units (UnitSplit); the three
-  // roles walk the same segments of it.
-  const UnitSplit us = unit_split(d, gridDim.x, PF_MIN_UNITS, PF_MAX_PARTS);
-  const int cta = blockIdx.x;
-  const bool active = cta < us.n_cta;
-  const int u_begin = active ? us.start_of(cta) : 0, u_end = active ? us.start_of(cta + 1) : 0;
   const uint32_t sKV = smem_u32(smem + OFF_KV);
+  if (!CLUSTER && u_begin < u_end) seg = segment_at(info(seq0), seq0, u_begin, u_end);
+  // The segment that starts where `s` ends, given s.end < u_end: s then ends at its pair's
+  // end, and the next segment is the next pair from its first unit, the session's next KV
+  // head or the next session's first one.
+  auto step = [&](PSeg& s) {
+    if (++s.head == H) {
+      s.head = 0;
+      s.nb = info(++s.seq).n_blocks;
+    }
+    s.pair_start = s.u = s.end;
+    s.pair_end = s.pair_start + s.nb;
+    s.end = min(u_end, s.pair_end);
+  };
+  // Stream-K: a pair's CTAs arrive at its counter.  The first segment's partial state (of a
+  // pair that ends inside the range) is published when its segment ends but nothing waits
+  // for the arrival; the last one's is not even published when every other part is there.
+  const bool early = !CLUSTER && u_begin < u_end && seg.u != seg.pair_start && seg.end < u_end;
 
-  if (warp == 0 || warp == 6) {
+  if (warp < 2) {
     // ---------------- producers ----------------
-    // Warp 0 loads the K halves of the stages, warp 6 the V halves, each with its
-    // own full/empty barriers: a K half is free again once S = Q K^T of its stage
-    // is complete, a V half once O += P V is, so the K loads run ahead of the V
-    // loads by up to the ring depth.  The whole warp walks the segments; lane j
-    // fetches the page id of block (window + j) so that one round trip serves 32
-    // blocks, and lane 0 issues the TMA loads with the ids shuffled to it.
-    const bool is_v = warp == 6;
-    const int b_full = is_v ? B_V_FULL : B_K_FULL, b_empty = is_v ? B_V_EMPTY : B_K_EMPTY;
-    uint32_t n = 0;  // stages produced
+    // A K half is free again once S = Q K^T of its stage is complete, a V half once O += P V
+    // is, so the K loads run ahead of the V loads by up to the ring depth.  Page ids come 32
+    // at a time (lane i holds the id of the window's page i); lane 2 pg + h issues half h
+    // (columns 0-63, 64-127) of page pg of a stage: one lane issuing all of a stage's boxes
+    // is bound by the issue itself (about 50 ns a box).
+    const bool is_v = warp == 1;
+    uint64_t* full = bars + (is_v ? B_V_FULL : B_K_FULL);
+    uint64_t* empty = bars + (is_v ? B_V_EMPTY : B_K_EMPTY);
+    const int pg = (lane >> 1) & 3;
+    const CUtensorMap* map = (lane & 1) ? &map_hi : &map_lo;
+    uint8_t* dst = smem + OFF_KV + (is_v ? 2 * KV_PANEL : 0) + (lane & 1) * KV_PANEL + pg * 2048;
+    const uint64_t policy = evict_first_policy();
+    bool arrive_first = is_v && early;  // (lane 0) the first pair's arrival is still to come
+    const int first_cf = us_first_part(us, seg), first_pair = seg.seq * H + seg.head;
+    const int first_nch = cta - first_cf + 1;
+    uint32_t n = 0;          // stages produced
+    int st = 0;              // ring slot and pass of the next stage
+    uint32_t pass = 0;
     bool stop = false;
     uint32_t rows_seen = 0;  // segments holding chunk slots, before this one
     (void)rows_seen;
-    UnitSeg seg;
     for (int u = u_begin; u < u_end && !stop;) {
-      seg = u == u_begin ? unit_segment(d, u, u_end) : next_segment(d, seg, u_end);
+      if (u != u_begin) step(seg);
       u = seg.end;
       const int head = seg.head;
-      const SeqInfo& si = seg.si;
+      const SeqInfo& si = info(seg.seq);
       const int32_t* hrow = d.hist_pt + (size_t)si.sid * d.max_pages_per_session;
       const int32_t* lrow = d.live_pt + (size_t)si.sid * d.max_pages_per_session;
-      const int blk0 = seg.blk_begin(), nblk = seg.end - seg.u;
-      const int n_st = (nblk + 3) / 4;
-      int pid = 0;
+      const int blk0 = seg.blk(), nblk = seg.n_blk(), n_st = seg.n_st();
+      auto page_at = [&](int b) { return b < nblk ? block_page(si, hrow, lrow, blk0 + b) : 0; };
+      int pid = page_at(lane), pid_next = page_at(32 + lane);
       if (is_v) {
         // The segment's query rows (T tokens x G heads, 1 KiB per token) and rotary
         // rows (512 B per token) into L2 ahead of the softmax warps, which read them
@@ -371,48 +423,40 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
         }
       }
       for (int k = 0; k < n_st; ++k, ++n) {
-        const int b0 = 4 * k;
-        if ((b0 & 31) == 0) {
-          const int bj = b0 + lane;
-          pid = bj < nblk ? block_page(si, hrow, lrow, blk0 + bj) : 0;
+        if (k > 0 && (k & 7) == 0) {
+          pid = pid_next;
+          pid_next = page_at(4 * k + 32 + lane);
         }
-        const int st = n % TC_STAGES;
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait(d, &bars[b_empty + st], ((n / TC_STAGES) & 1) ^ 1);
-        ok = __shfl_sync(FULL, ok, 0);
-        if (!ok) {
-          if (lane == 0) s_abort = 1;
-          stop = true;
-          break;
+        const int page = __shfl_sync(FULL, pid, 4 * (k & 7) + pg);
+        if (arrive_first && lane == 0 && mbar_try_wait(&bars[B_PUB], 0)) {
+          s_first_last = arrive_acq_rel(&d.pf_count[first_pair], first_nch);
+          arrive_first = false;
         }
-        const int npg = min(4, nblk - b0);
-        int pages[4];
-#pragma unroll
-        for (int pg = 0; pg < 4; ++pg) pages[pg] = __shfl_sync(FULL, pid, (b0 & 31) + pg);
+        __syncwarp();
+        const int npg = min(4, nblk - 4 * k);
+        bool ok = mbar_wait(d, &empty[st], (pass & 1) ^ 1);
         if constexpr (FUSED) {
           // A stage holding chunk slots is copied only once the softmax warps have
           // written the segment's rows (they do so when the segment starts).
           int t0, t1;
-          chunk_tokens_in(si, blk0 + b0, blk0 + b0 + npg, t0, t1);
-          if (t0 < t1) {
-            int ok = 1;
-            if (lane == 0) ok = mbar_wait(d, &bars[B_ROWS], rows_seen & 1);
-            if (!__shfl_sync(FULL, ok, 0)) {
-              if (lane == 0) s_abort = 1;
-              stop = true;
-              break;
-            }
-          }
+          chunk_tokens_in(si, blk0 + 4 * k, blk0 + 4 * k + npg, t0, t1);
+          if (t0 < t1) ok = ok && mbar_wait(d, &bars[B_ROWS], rows_seen & 1);
         }
-        if (lane == 0) {
-          mbar_arrive_expect_tx(&bars[b_full + st], npg * 2 * 2048);
-          uint8_t* base = smem + OFF_KV + st * STAGE + (is_v ? 2 * KV_PANEL : 0);
-          for (int pg = 0; pg < npg; ++pg) {
-            // Pool rows of this page's K (kv = 0) or V (kv = 1) tile of `head`.
-            const int row = (((pages[pg] * L + layer) * 2 + (is_v ? 1 : 0)) * H + head) * PS;
-            tma_load_2d(base + pg * 2048, &map_lo, 0, row, &bars[b_full + st]);
-            tma_load_2d(base + KV_PANEL + pg * 2048, &map_hi, 0, row, &bars[b_full + st]);
-          }
+        if (!__all_sync(FULL, ok)) {
+          if (lane == 0) s_abort = 1;
+          stop = true;
+          break;
+        }
+        if (lane == 0) mbar_arrive_expect_tx(&full[st], npg * 2 * 2048);
+        __syncwarp();
+        if (lane < 8 && pg < npg) {
+          // Pool rows of this page's K (kv = 0) or V (kv = 1) tile of `head`.
+          const int row = (((page * L + layer) * 2 + (is_v ? 1 : 0)) * H + head) * PS;
+          tma_load_2d_hint(dst + st * STAGE, map, 0, row, &full[st], policy);
+        }
+        if (++st == ring) {
+          st = 0;
+          ++pass;
         }
       }
       if constexpr (FUSED) {
@@ -422,166 +466,228 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       }
       stop = stop || __any_sync(FULL, s_abort != 0);
     }
-  } else if (warp == 1 || warp == 7) {
+    if (stop) {
+      // No copy may still be in flight when the CTA ends.
+      for (uint32_t i = n > (uint32_t)ring ? n - ring : 0; i < n; ++i)
+        mbar_wait(d, &full[i % ring], (i / ring) & 1);
+    }
+    if (!CLUSTER && is_v && u_begin < u_end) {
+      pdl_wait();  // the counters may still be the previous launch's until then
+      if (arrive_first && lane == 0 && mbar_wait(d, &bars[B_PUB], 0))
+        s_first_last = arrive_acq_rel(&d.pf_count[first_pair], first_nch);
+      __syncwarp();
+      if (!seg.whole() && !stop) {
+        const int cf = us.owner(seg.pair_start), nch = us.owner(seg.pair_end - 1) - cf + 1;
+        int there = 0;
+        if (lane == 0) {
+          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(there)
+                       : "l"(&d.pf_count[seg.seq * H + seg.head]) : "memory");
+          s_peek = there == nch - 1;
+        }
+        there = __shfl_sync(FULL, there, 0);
+        if (there == nch - 1) {
+          // The first other part's rows into L2 (written long ago, perhaps).
+          const int ch = cta == cf ? 1 : 0;
+          const char* p = reinterpret_cast<const char*>(
+              d.pf_part_o + (size_t)(ch ? 2 * (cf + 1) : us.slot_of(cf, cf, seg.pair_start)) * (M * D));
+          const int lines = (info(seg.seq).t * G * 16 + 127) / 128;  // per 16-byte chunk column
+          for (int i = lane; i < lines * (D / 4); i += 32)
+            prefetch_l2(p + (size_t)(i / lines) * (M * 16) + (i % lines) * 128);
+        }
+      } else if (lane == 0) {
+        s_peek = 0;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_PEEK]);
+    }
+  } else if (warp < 4) {
     // ---------------- MMA issuers ----------------
-    // One elected thread each: warp 1 issues S = Q K^T of every stage, warp 7
-    // O += P V.  Their products use different accumulators, and each thread's
-    // tcgen05.commit tracks only its own MMAs, so the two streams interleave in
-    // the tensor pipe and neither waits behind the other's issue cost.
+    // One elected thread each: their products use different accumulators, and each
+    // thread's tcgen05.commit tracks only its own MMAs, so the two streams interleave in
+    // the tensor pipe and neither waits behind the other's issue cost (about 60 cycles per
+    // instruction, 8 + 2 for a stage's S).
     if (lane == 0) {
-      uint32_t n = 0;  // K/V stages of the earlier segments
-      if (warp == 1) {
+      uint32_t n = 0;  // stage
+      int st = 0;
+      uint32_t pass = 0;
+      bool ok = true;
+      if (warp == 2) {
         constexpr uint32_t ID_S = instr_desc(NK, M, false);
-        uint32_t sc = 0;     // S tiles issued
-        uint32_t segs = 0;   // segments started
-        UnitSeg seg;
-        for (int u = u_begin; u < u_end && !s_abort; ++segs) {
-          seg = u == u_begin ? unit_segment(d, u, u_end) : next_segment(d, seg, u_end);
+        uint32_t segs = 0;
+        for (int u = u_begin; u < u_end && ok && !s_abort; ++segs) {
+          if (u != u_begin) step(seg);
           u = seg.end;
-          const int n_st = (seg.end - seg.u + 3) / 4;
-          if (!mbar_wait(d, &bars[B_Q], segs & 1)) {
-            s_abort = 1;
-            break;
-          }
-          tc_fence_after();
-          for (int k = 0; k < n_st && !s_abort; ++k) {
-            const int st = (n + k) % TC_STAGES;
-            const int sb = sc % 2;
-            if (!mbar_wait(d, &bars[B_K_FULL + st], ((n + k) / TC_STAGES) & 1) ||
-                !mbar_wait(d, &bars[B_S_EMPTY + sb], ((sc / 2) & 1) ^ 1)) {
-              s_abort = 1;
-              break;
-            }
+          const int n_st = seg.n_st();
+          ok = mbar_wait(d, &bars[B_Q], segs & 1);
+          for (int k = 0; k < n_st && ok; ++k, ++n) {
+            const int g = n & 1;
+            ok = mbar_wait(d, &bars[B_K_FULL + st], pass & 1) &&
+                 mbar_wait(d, &bars[B_S_EMPTY + g], ((n >> 1) & 1) ^ 1);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t kbase = sKV + st * STAGE;
+            const uint64_t kdesc = smem_desc(sKV + st * STAGE, 0, 1024);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               // 16 dims per step: 8 TMEM columns of Q; 32 bytes of a swizzled K row.
-              const uint32_t kb = kbase + (kk >> 2) * KV_PANEL + (kk & 3) * 32;
-              tc_mma_ts(tmem + S_COL + sb * NK, tmem + Q_COL + kk * 8, smem_desc(kb, 0, 1024),
-                        ID_S, kk > 0 ? 1u : 0u);
+              tc_mma_ts(tmem + S_COL + g * NK, tmem + Q_COL + kk * 8,
+                        desc_at(kdesc, (kk >> 2) * KV_PANEL + (kk & 3) * 32), ID_S, kk > 0 ? 1u : 0u);
             }
-            tc_commit(&bars[B_S_FULL + sb]);
+            tc_commit(&bars[B_S_FULL + g]);
             tc_commit(&bars[B_K_EMPTY + st]);
-            ++sc;
+            if (++st == ring) {
+              st = 0;
+              ++pass;
+            }
           }
-          n += n_st;
         }
       } else {
         constexpr uint32_t ID_PV = instr_desc(D, M, true);
-        uint32_t pv = 0;  // P V products issued
-        UnitSeg seg;
-        for (int u = u_begin; u < u_end && !s_abort;) {
-          seg = u == u_begin ? unit_segment(d, u, u_end) : next_segment(d, seg, u_end);
+        for (int u = u_begin; u < u_end && ok && !s_abort;) {
+          if (u != u_begin) step(seg);
           u = seg.end;
-          const int n_st = (seg.end - seg.u + 3) / 4;
-          for (int k = 0; k < n_st && !s_abort; ++k) {
-            const int st = (n + k) % TC_STAGES;
-            const int pb = pv % 2;
-            if (!mbar_wait(d, &bars[B_V_FULL + st], ((n + k) / TC_STAGES) & 1) ||
-                !mbar_wait(d, &bars[B_P_FULL + pb], (pv / 2) & 1)) {
-              s_abort = 1;
-              break;
-            }
+          const int n_st = seg.n_st();
+          for (int k = 0; k < n_st && ok; ++k, ++n) {
+            const int g = n & 1;
+            ok = mbar_wait(d, &bars[B_V_FULL + st], pass & 1) &&
+                 mbar_wait(d, &bars[B_P_FULL + g], (n >> 1) & 1);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t vbase = sKV + st * STAGE + 2 * KV_PANEL;
+            const uint64_t vdesc = smem_desc(sKV + st * STAGE + 2 * KV_PANEL, KV_PANEL, 1024);
 #pragma unroll
             for (int kk = 0; kk < NK / 16; ++kk) {
-              // 16 keys per step: 8 TMEM columns of P; 16 rows of the V panels.  The
-              // first product of a segment overwrites O (its previous contents were
-              // read by the epilogue before this segment's first P was written).
-              const uint32_t vb = vbase + kk * 16 * 128;
-              tc_mma_ts(tmem + O_COL, tmem + P_COL + pb * (NK / 2) + kk * 8,
-                        smem_desc(vb, KV_PANEL, 1024), ID_PV, (k > 0 || kk > 0) ? 1u : 0u);
+              // 16 keys per step: 8 TMEM columns of P; 16 rows of the V panels.  A group's
+              // first product of a segment overwrites its O (both groups read the previous
+              // contents before they wrote any P of this segment).
+              tc_mma_ts(tmem + O_COL + g * D, tmem + P_COL + g * (NK / 2) + kk * 8,
+                        desc_at(vdesc, kk * 16 * 128), ID_PV, (k > 1 || kk > 0) ? 1u : 0u);
             }
+            tc_commit(&bars[B_PV + g]);
             tc_commit(&bars[B_V_EMPTY + st]);
-            tc_commit(&bars[B_P_EMPTY + pb]);
-            tc_commit(&bars[B_O + pb]);
-            ++pv;
+            if (++st == ring) {
+              st = 0;
+              ++pass;
+            }
           }
-          n += n_st;
         }
       }
+      if (!ok) s_abort = 1;
       // No MMA may still be running when the tensor memory is released.
       tc_commit(&bars[B_FINAL]);
       mbar_wait(d, &bars[B_FINAL], 0);
     }
+    __syncwarp();
   } else {
     // ---------------- softmax / epilogue ----------------
     // A failed (timed-out) wait makes the warp "dead": it then skips waits and
-    // work but still walks the same items, arrivals and named barriers, so the
-    // other softmax warps never wait for it.
+    // work but still walks the same segments and named barriers, so the other
+    // softmax warps never wait for it.
+    const int grp = (warp >> 2) - 1;           // group 0 (warps 4-7) or 1 (warps 8-11)
     const int quarter = warp & 3;              // TMEM lanes 32*quarter .. +31
     const int r = quarter * 32 + lane;         // this thread's query row
+    const int ts = tid - (THREADS - SM_THREADS);
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    uint32_t sc = 0, pv = 0;
+    float2* s_ml = reinterpret_cast<float2*>(smem + OFF_ML);
+    uint32_t n = 0;                            // stages of the earlier segments
     bool dead = false;
-    pdl_wait();
     auto wait = [&](uint64_t* bar, uint32_t parity) {
       if (dead) return;
       dead = !__all_sync(FULL, mbar_wait(d, bar, parity));
       if (dead && lane == 0) s_abort = 1;
     };
-    UnitSeg seg;
-    for (int u = u_begin; u < u_end;) {
-      seg = u == u_begin ? unit_segment(d, u, u_end) : next_segment(d, seg, u_end);
-      const int first = seg.u == u_begin;
-      u = seg.end;
-      const int head = seg.head;
-      const SeqInfo& si = seg.si;
-      const int blk0 = seg.blk_begin(), nblk = seg.end - seg.u;
-      const int n_st = (nblk + 3) / 4;
-      const int R = si.t * G;
-      const bool live = r < R;
-      const int t = r / G, g = r % G;
-      const int qlog = si.n_hist + si.n_live - si.t + t;
-      // The previous segment's products are complete (its epilogue waited for the
-      // last one), so the query tile in tensor memory can be overwritten.  Every
-      // lane writes its row: the query (bfloat16 pairs, dims 0..127 in columns
-      // 0..63), or zeros for padding rows.
-      if (!dead) {
-        uint32_t qw[D / 2];
-        if (live) {
-          // Chunk c (dims 8c..8c+7) of the first half pairs with chunk c of the second.
-          const uint4* qrow = reinterpret_cast<const uint4*>(
-              q + ((size_t)(si.q_row0 + t) * d.q_heads + head * G + g) * D);
-          const float4* cs =
-              reinterpret_cast<const float4*>(d.rope + (size_t)(si.pos_first + t) * (D / 2));
+    auto sync_groups = [] { asm volatile("bar.sync 1, %0;" ::"n"(SM_THREADS) : "memory"); };
+    uint8_t* st_q = smem + off_q(ring);
+    uint8_t* st_rope = smem + off_rope(ring, max_t);
+    uint8_t* st_out = smem + off_out(ring, max_t);
+    // Asynchronous copies of a segment's rotary and query rows into their staging rows.
+    auto copy_rope = [&](const PSeg& sg) {
+      const SeqInfo& si = info(sg.seq);
+      const uint4* src = reinterpret_cast<const uint4*>(d.rope + (size_t)si.pos_first * (D / 2));
+      const uint32_t dst = smem_u32(st_rope);
+      for (int i = ts; i < si.t * 32; i += SM_THREADS)
+        cp_async16(dst + (i >> 5) * ROPE_PITCH + (i & 31) * 16, src + i);
+    };
+    auto copy_q = [&](const PSeg& sg) {
+      const SeqInfo& si = info(sg.seq);
+      const uint4* src = reinterpret_cast<const uint4*>(
+          q + ((size_t)si.q_row0 * d.q_heads + sg.head * G) * D);
+      const uint32_t dst = smem_u32(st_q);
+      const size_t tok = (size_t)d.q_heads * D / 8;
+      for (int i = ts; i < si.t * 64; i += SM_THREADS)  // a token's G rows are contiguous
+        cp_async16(dst + (i >> 4) * ST_PITCH + (i & 15) * 16, src + (i >> 6) * tok + (i & 63));
+    };
+    // The staged query rows, rotated at their tokens' positions, scaled and rounded, into
+    // tensor memory: this thread's row, its group's 4 of the 8 pairs of 16-byte chunks (c,
+    // c + 8) that rotate together.  Padding rows: zero, and their P too.  Then, in the
+    // per-layer order, the segment's new rows into the pool.
+    auto start_segment = [&](const PSeg& sg) {
+      const SeqInfo& si = info(sg.seq);
+      uint32_t qw[32];
+      if (r < si.t * G) {
+        const uint4* qrow = reinterpret_cast<const uint4*>(st_q + r * ST_PITCH) + 4 * grp;
+        const float4* cs = reinterpret_cast<const float4*>(st_rope + (r / G) * ROPE_PITCH) + 16 * grp;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const uint4 wa = qrow[c], wb = qrow[c + 8];
-            const uint32_t ua[4] = {wa.x, wa.y, wa.z, wa.w}, ub[4] = {wb.x, wb.y, wb.z, wb.w};
+        for (int c = 0; c < 4; ++c) {
+          const uint4 wa = qrow[c], wb = qrow[c + 8];
+          const uint32_t ua[4] = {wa.x, wa.y, wa.z, wa.w}, ub[4] = {wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const float4 t4 = cs[c * 4 + h];  // (cos, sin) of dims 8c + 2h, 8c + 2h + 1
-              const float a0 = bf16lo(ua[h]), a1 = bf16hi(ua[h]);
-              const float b0 = bf16lo(ub[h]), b1 = bf16hi(ub[h]);
-              qw[4 * c + h] = pack_bf16(fmaf(a0, t4.x, -b0 * t4.y) * qk_scale,
-                                        fmaf(a1, t4.z, -b1 * t4.w) * qk_scale);
-              qw[D / 4 + 4 * c + h] = pack_bf16(fmaf(b0, t4.x, a0 * t4.y) * qk_scale,
-                                                fmaf(b1, t4.z, a1 * t4.w) * qk_scale);
-            }
+          for (int h = 0; h < 4; ++h) {
+            const float4 t4 = cs[c * 4 + h];  // (cos, sin) of dims 8c + 2h, 8c + 2h + 1
+            const float a0 = bf16lo(ua[h]), a1 = bf16hi(ua[h]);
+            const float b0 = bf16lo(ub[h]), b1 = bf16hi(ub[h]);
+            qw[4 * c + h] = pack_bf16(fmaf(a0, t4.x, -b0 * t4.y) * qk_scale,
+                                      fmaf(a1, t4.z, -b1 * t4.w) * qk_scale);
+            qw[16 + 4 * c + h] = pack_bf16(fmaf(b0, t4.x, a0 * t4.y) * qk_scale,
+                                           fmaf(b1, t4.z, a1 * t4.w) * qk_scale);
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < D / 2; ++j) qw[j] = 0u;
         }
-        tmem_st32(trow + Q_COL, qw);
-        tmem_st32(trow + Q_COL + 32, qw + 32);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) qw[i] = 0u;
       }
+      __syncwarp();
+      tmem_st16(trow + Q_COL + 16 * grp, qw);
+      tmem_st16(trow + Q_COL + 32 + 16 * grp, qw + 16);
+      if (quarter * 32 >= si.t * G) tmem_st32(trow + P_COL + grp * (NK / 2), qw);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_Q]);
       if constexpr (FUSED) {
         int t0, t1;
-        chunk_tokens_in(si, blk0, blk0 + nblk, t0, t1);
+        chunk_tokens_in(si, sg.blk(), sg.blk() + sg.n_blk(), t0, t1);
         if (t0 < t1) {
-          if (!dead) write_chunk_rows(d, layer, si, head, new_k, new_v, t0, t1, r);
+          if (!dead)
+            write_chunk_rows(d, layer, si, sg.head, new_k, new_v, t0, t1, ts, SM_THREADS);
           __syncwarp();
           if (lane == 0) mbar_arrive(&bars[B_ROWS]);
         }
       }
-
+    };
+    if (u_begin < u_end) copy_rope(seg);  // (the table is not written by any launch)
+    pdl_wait();
+    if (u_begin < u_end) {
+      copy_q(seg);
+      cp_async_wait_all();
+      sync_groups();
+      start_segment(seg);
+    }
+    for (int u = u_begin; u < u_end;) {
+      const bool first = u == u_begin;
+      u = seg.end;
+      const PSeg cur = seg;
+      const SeqInfo& si = info(cur.seq);
+      const int head = cur.head;
+      const int blk0 = cur.blk(), nblk = cur.n_blk(), n_st = cur.n_st();
+      const int R = si.t * G;
+      if (u < u_end) {
+        // The next segment's rows are copied while this one runs (every thread is done with
+        // the staged ones: the last segment's end synchronised them).
+        step(seg);
+        if (first) sync_groups();
+        copy_rope(seg);
+        copy_q(seg);
+      }
+      const bool live = r < R, idle = quarter * 32 >= R;
+      const int qlog = si.n_hist + si.n_live - si.t + r / G;
       // Blocks that may need a mask: the partly filled last history page, the
       // first live page when it starts mid-page, and every block from the one
       // holding the chunk's first query on (causal).  A stage of four pages that
@@ -592,17 +698,23 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       const int sl_first = si.live_head + si.n_live - si.t;  // live slot of the first query
       const int b_causal = nhp + sl_first / PS + ((sl_first % PS) == PS - 1 ? 1 : 0);
       float m_used = -INFINITY, l = 0.f;
-      for (int k = 0; k < n_st; ++k) {
-        const int sb = sc % 2, pb = pv % 2;
-        wait(&bars[B_S_FULL + sb], (sc / 2) & 1);
+      const int k_first = (grp ^ n) & 1;  // this group's stages: k_first, + 2, ...
+      for (int k = k_first; k < n_st; k += 2) {
+        const uint32_t j = (n + k) >> 1;
+        wait(&bars[B_S_FULL + grp], j & 1);
+        if (dead) break;
         tc_fence_after();
+        if (idle) {  // padding rows alone: their P is zero already
+          if (lane == 0) mbar_arrive(&bars[B_S_EMPTY + grp]);
+          if (j > 0) wait(&bars[B_PV + grp], (j - 1) & 1);
+          if (lane == 0 && !dead) mbar_arrive(&bars[B_P_FULL + grp]);
+          continue;
+        }
         float s[NK];
-        tmem_ld32(trow + S_COL + sb * NK, s);
-        tmem_ld32(trow + S_COL + sb * NK + 32, s + 32);
+        tmem_ld64(trow + S_COL + grp * NK, s);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bars[B_S_EMPTY + sb]);
-        ++sc;
+        if (lane == 0) mbar_arrive(&bars[B_S_EMPTY + grp]);
         // Mask the keys that are not resident slots or lie after the row's query.
         // Interior stages (four full pages, every key before the chunk's first
         // query) need no mask.  Padding rows (r >= T*G) are left unmasked: their
@@ -612,16 +724,13 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
         const bool interior = npg == 4 && b0 + 3 < b_causal &&
                               (unsigned)(b_hist_part - b0) > 3u && (unsigned)(b_live_part - b0) > 3u;
         if (!interior) {
-          BlockRange brs[4];
-#pragma unroll
-          for (int pg = 0; pg < 4; ++pg) brs[pg] = block_range(si, b0 + min(pg, npg - 1));
 #pragma unroll
           for (int pg = 0; pg < 4; ++pg) {
+            const BlockRange br = block_range(si, b0 + min(pg, npg - 1));
 #pragma unroll
-            for (int j = 0; j < PS; ++j) {
-              const bool v = pg < npg && j >= brs[pg].lo && j < brs[pg].hi &&
-                             brs[pg].base + j <= qlog;
-              float& x = s[pg * PS + j];
+            for (int i = 0; i < PS; ++i) {
+              const bool v = pg < npg && i >= br.lo && i < br.hi && br.base + i <= qlog;
+              float& x = s[pg * PS + i];
               x = (v || !live) ? x : -INFINITY;
             }
           }
@@ -631,233 +740,371 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
 #pragma unroll
         for (int i = 0; i < 8; ++i) m8[i] = s[i];
 #pragma unroll
-        for (int j = 8; j < NK; ++j) m8[j % 8] = fmaxf(m8[j % 8], s[j]);
+        for (int i = 8; i < NK; i += 16)
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            if (i + 8 + c < NK) m8[c] = fmaxf(fmaxf(m8[c], s[i + c]), s[i + 8 + c]);
+            else m8[c] = fmaxf(m8[c], s[i + c]);
+          }
         float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
                          fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
-        if (dead || !live) mx = -INFINITY;
-        // Rescale O (in TMEM) and l only when the row maximum grows by > 2^8; this
-        // waits for the previous P V product.  Every lane of the warp takes part
-        // in the TMEM accesses; lanes that need no rescale use factor 1.
+        if (!live) mx = -INFINITY;
+        // The group's previous product is complete: its O may be rescaled and its P
+        // overwritten.
+        if (j > 0) wait(&bars[B_PV + grp], (j - 1) & 1);
+        if (dead) break;
+        // Rescale O (in TMEM) and l only when the row maximum grows by > 2^8.  Every lane
+        // of the warp takes part in the TMEM accesses; lanes that need no rescale use
+        // factor 1.
         const bool need = mx > m_used + RESCALE_LOG2;
-        const bool have_o = pv > 0 && m_used != -INFINITY;
+        const bool have_o = k > k_first && m_used != -INFINITY;
         if (__any_sync(FULL, need && have_o)) {
-          wait(&bars[B_O + (pv - 1) % 2], ((pv - 1) / 2) & 1);
           tc_fence_after();
           const float f = (need && have_o) ? exp2f(m_used - mx) : 1.f;
+#pragma unroll 1
+          for (int c = 0; c < D / 16; ++c) {
+            float o[16];
+            tmem_ld16(trow + O_COL + grp * D + c * 16, o);
 #pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
-            float o[32];
-            tmem_ld32(trow + O_COL + c * 32, o);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] *= f;
-            tmem_st32(trow + O_COL + c * 32, o);
+            for (int i = 0; i < 16; ++i) o[i] *= f;
+            tmem_st16(trow + O_COL + grp * D + c * 16, o);
           }
-          tc_fence_before();
         }
         if (need) {
           if (have_o) l *= exp2f(m_used - mx);
           m_used = mx;
         }
-        // P = exp2(s - m_used) as bfloat16 pairs into TMEM buffer pb (row r, 32 columns).
-        wait(&bars[B_P_EMPTY + pb], ((pv / 2) & 1) ^ 1);
-        // Masked keys are -inf and give 0; a row with no finite key yet uses 0 as
-        // its reference so that no -inf - -inf appears; padding rows get weight 0.
+        // P = exp2(s - m_used) as bfloat16 pairs.  Masked keys are -inf and give 0; a row
+        // with no finite key yet uses 0 as its reference so that no -inf - -inf appears;
+        // padding rows get weight 0.
         const float mref = !live ? INFINITY : (m_used == -INFINITY ? 0.f : m_used);
-        float rs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const float2 nref = make_float2(-mref, -mref);
+        float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
+                        make_float2(0.f, 0.f)};
         uint32_t pw[NK / 2];
 #pragma unroll
-        for (int j = 0; j < NK; j += 2) {
-          const float p0 = ex2(s[j] - mref), p1 = ex2(s[j + 1] - mref);
-          rs[j % 8] += p0;
-          rs[j % 8 + 1] += p1;
-          pw[j / 2] = pack_bf16(p0, p1);
+        for (int i = 0; i < NK; i += 2) {
+          const float2 x = __fadd2_rn(make_float2(s[i], s[i + 1]), nref);
+          const float2 p = make_float2(ex2(x.x), ex2(x.y));
+          rs[(i / 2) & 3] = __fadd2_rn(rs[(i / 2) & 3], p);
+          pw[i / 2] = pack_bf16(p.x, p.y);
         }
-        l += ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
-        if (!dead) tmem_st32(trow + P_COL + pb * (NK / 2), pw);
+        const float2 r2 = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
+        l += r2.x + r2.y;
+        tmem_st32(trow + P_COL + grp * (NK / 2), pw);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bars[B_P_FULL + pb]);
-        ++pv;
+        if (lane == 0) mbar_arrive(&bars[B_P_FULL + grp]);
       }
-      // Epilogue: wait for the last P V, read O.
-      wait(&bars[B_O + (pv - 1) % 2], ((pv - 1) / 2) & 1);
-      tc_fence_after();
-      const bool single = seg.whole();
-      const int slot = 2 * cta + (first ? 0 : 1);
-      const size_t prow0 = (size_t)slot * (PF_MAX_TOKENS * G) + r;
-      const bool write = live && !dead;
-      const float inv = 1.f / l;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        float o[32];
-        tmem_ld32(trow + O_COL + c * 32, o);
-        if (write && single) {
-          __nv_bfloat16* orow =
-              out + ((size_t)(si.q_row0 + t) * d.q_heads + head * G + g) * D + c * 32;
-#pragma unroll
-          for (int i = 0; i < 32; i += 8)
-            *reinterpret_cast<uint4*>(orow + i) =
-                make_uint4(pack_bf16(o[i] * inv, o[i + 1] * inv),
-                           pack_bf16(o[i + 2] * inv, o[i + 3] * inv),
-                           pack_bf16(o[i + 4] * inv, o[i + 5] * inv),
-                           pack_bf16(o[i + 6] * inv, o[i + 7] * inv));
-        } else if (write) {
-          float* prow = d.pf_part_o + prow0 * D + c * 32;
-#pragma unroll
-          for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4*>(prow + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
-        }
+      // Epilogue: every product of the segment complete, both groups' (max, sum) known.
+      if (k_first < n_st) {
+        const uint32_t j = (n + ((n_st - 1 - k_first) & ~1) + k_first) >> 1;  // last own stage
+        wait(&bars[B_PV + grp], j & 1);
       }
+      n += n_st;
+      s_ml[grp * M + r] = make_float2(dead ? -INFINITY : m_used, l);
       tc_fence_before();
-      if (!single) {
+      cp_async_wait_all();
+      sync_groups();
+      tc_fence_after();
+      if (u < u_end) start_segment(seg);
+      const float2 ml0 = s_ml[r], ml1 = s_ml[M + r];
+      // A segment of one stage has the state of one group only.
+      const bool has0 = n_st > 1 || k_first == grp, has1 = n_st > 1 || k_first != grp;
+      const float Mr = fmaxf(has0 ? ml0.x : -INFINITY, has1 ? ml1.x : -INFINITY);
+      const float f0 = has0 ? exp2_safe(ml0.x, Mr) : 0.f, f1 = has1 ? exp2_safe(ml1.x, Mr) : 0.f;
+      const float Lr = (has0 ? ml0.y * f0 : 0.f) + (has1 ? ml1.y * f1 : 0.f);
+      // Columns [64 grp + 32 c, + 32) of this row, both groups' parts summed.
+      auto own = [&](int c, float sc, float (&o)[32]) {
+        const uint32_t col = trow + O_COL + 64 * grp + 32 * c;
+        const float a0 = f0 * sc, a1 = f1 * sc;
+        if (has0) {
+          tmem_ld32(col, o);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] *= a0;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] = 0.f;
+        }
+        if (has1) {
+#pragma unroll
+          for (int h = 0; h < 32; h += 16) {
+            float o1[16];
+            tmem_ld16(col + D + h, o1);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) o[h + i] = fmaf(o1[i], a1, o[h + i]);
+          }
+        }
+      };
+      const bool write = live && !dead;
+      // Output rows leave through the staging rows: store() puts 32 normalised columns of this
+      // thread's row there, flush() writes the rows out whole.
+      auto store = [&](int c, const float (&o)[32]) {
+        if (!live) return;
+#pragma unroll
+        for (int i = 0; i < 32; i += 8)
+          *reinterpret_cast<uint4*>(st_out + r * ST_PITCH + 128 * grp + 64 * c + 2 * i) =
+              make_uint4(pack_bf16(o[i], o[i + 1]), pack_bf16(o[i + 2], o[i + 3]),
+                         pack_bf16(o[i + 4], o[i + 5]), pack_bf16(o[i + 6], o[i + 7]));
+      };
+      auto flush = [&] {
+        sync_groups();
+        for (int i = ts; i < R * 16 && !dead; i += SM_THREADS) {
+          const int row = i >> 4, c = i & 15;
+          __nv_bfloat16* orow =
+              out + ((size_t)(si.q_row0 + row / G) * d.q_heads + head * G + row % G) * D;
+          reinterpret_cast<uint4*>(orow)[c] =
+              *reinterpret_cast<const uint4*>(st_out + row * ST_PITCH + c * 16);
+        }
+      };
+      if (CLUSTER ? k_slices == 1 : cur.whole()) {
+        const float inv = 1.f / Lr;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float o[32];
+          own(c, inv, o);
+          store(c, o);
+        }
+        flush();
+      } else if constexpr (CLUSTER) {
+        // The partial rows into the ring's place (every copy and product is complete); they
+        // are sent from there below.
+        float* prow = reinterpret_cast<float*>(smem + OFF_KV + r * ROW_PITCH);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float o[32];
+          own(c, 1.f, o);
+          if (write) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+              *reinterpret_cast<float4*>(prow + 64 * grp + 32 * c + i) =
+                  make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
+          }
+        }
+        if (live && grp == 0) *reinterpret_cast<float2*>(prow + D) = make_float2(Mr, Lr);
+      } else {
         // Split-K: publish this part's (O, max, sum); the last CTA to arrive for the
-        // (session, head) merges every part, one thread per query row.  All four
-        // softmax warps reach both named barriers on every such segment.
-        if (write) d.pf_part_ml[prow0] = make_float2(m_used, l);
-        const int cf = us.owner(seg.pair_start), nch = us.owner(seg.pair_end - 1) - cf + 1;
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (warp == 2 && lane == 0)
-          s_last = arrive_acq_rel(&d.pf_count[seg.seq * H + head], nch);
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (s_last) {
-          // The merge runs in tensor memory: this CTA's own part is still in the O
-          // columns (the next segment's first P V overwrites them only after this),
-          // and each other part's row is loaded whole, all its words at once, and
-          // added there.  The first other part's row is loaded together with every
-          // part's (max, sum), so a pair of two parts costs one round trip.  Every
-          // lane takes part in the tensor-memory accesses; rows that are padding (or
-          // of a warp whose wait gave up) weigh 0 and write nothing.
-          const int first_slot = us.slot_of(cf, cf, seg.pair_start);
-          const int own = cta - cf;
-          auto prow = [&](int ch) {
-            return (size_t)(ch ? 2 * (cf + ch) : first_slot) * (PF_MAX_TOKENS * G) + r;
-          };
-          auto load_row = [&](int ch, float4 (&v)[D / 4]) {
-            const float4* src = reinterpret_cast<const float4*>(d.pf_part_o + prow(ch) * D);
+        // (session, head) merges every part, half a query row per thread.  Every softmax
+        // warp reaches the same named barriers.
+        const bool first_early = first && early, last = u >= u_end;
+        if (last) wait(&bars[B_PEEK], 0);
+        const bool alone = last && !dead && s_peek;  // every other part is there
+        const int cf = us.owner(cur.pair_start), nch = us.owner(cur.pair_end - 1) - cf + 1;
+        if (!__any_sync(FULL, alone)) {
+          const int slot = 2 * cta + (first ? 0 : 1);
 #pragma unroll
-            for (int i = 0; i < D / 4; ++i)
-              v[i] = write ? __ldcg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-          };
-          const int f0 = own == 0 ? 1 : 0;  // first other part
-          float4 v[D / 4];
-          load_row(f0, v);
-          constexpr int MB = 8;
-          float2 ml[MB];
-          auto load_ml = [&](int c0) {
-#pragma unroll
-            for (int i = 0; i < MB; ++i)
-              ml[i] = (write && c0 + i < nch && c0 + i != own) ? __ldcg(&d.pf_part_ml[prow(c0 + i)])
-                                                               : make_float2(-INFINITY, 0.f);
-          };
-          float Mx = write ? m_used : -INFINITY;
-          load_ml(0);
-#pragma unroll
-          for (int i = 0; i < MB; ++i) Mx = fmaxf(Mx, ml[i].x);
-          const float ml_f0_x = f0 < MB ? (f0 == 0 ? ml[0].x : ml[1].x) : -INFINITY;
-          float Ls = 0.f;
-#pragma unroll
-          for (int i = 0; i < MB; ++i) Ls += ml[i].y * exp2_safe(ml[i].x, Mx);
-          for (int c0 = MB; c0 < nch; c0 += MB) {
-            load_ml(c0);
-#pragma unroll
-            for (int i = 0; i < MB; ++i) Mx = fmaxf(Mx, ml[i].x);
-          }
-          if (nch > MB) {  // the sum again, against the final maximum
-            Ls = 0.f;
-            for (int c0 = 0; c0 < nch; c0 += MB) {
-              load_ml(c0);
-#pragma unroll
-              for (int i = 0; i < MB; ++i) Ls += ml[i].y * exp2_safe(ml[i].x, Mx);
-            }
-          }
-          if (write) Ls += l * exp2_safe(m_used, Mx);
-          const float invL = write ? 1.f / Ls : 0.f;
-          const float s_own = write ? exp2_safe(m_used, Mx) : 0.f;
-          // Own part scaled, plus the first other part.
-          float s_f = write ? exp2_safe(ml_f0_x, Mx) : 0.f;
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
+          for (int c = 0; c < 2; ++c) {
             float o[32];
-            tmem_ld32(trow + O_COL + c * 32, o);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float4 w4 = v[c * 8 + i];
-              o[4 * i] = o[4 * i] * s_own + w4.x * s_f;
-              o[4 * i + 1] = o[4 * i + 1] * s_own + w4.y * s_f;
-              o[4 * i + 2] = o[4 * i + 2] * s_own + w4.z * s_f;
-              o[4 * i + 3] = o[4 * i + 3] * s_own + w4.w * s_f;
-            }
-            tmem_st32(trow + O_COL + c * 32, o);
-          }
-          // The remaining parts (pairs over three or more CTAs), one row at a time.
-          for (int ch = f0 + 1; ch < nch; ++ch) {
-            if (ch == own) continue;
-            load_row(ch, v);
-            s_f = write ? exp2_safe(__ldcg(&d.pf_part_ml[prow(ch)]).x, Mx) : 0.f;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              float o[32];
-              tmem_ld32(trow + O_COL + c * 32, o);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const float4 w4 = v[c * 8 + i];
-                o[4 * i] += w4.x * s_f;
-                o[4 * i + 1] += w4.y * s_f;
-                o[4 * i + 2] += w4.z * s_f;
-                o[4 * i + 3] += w4.w * s_f;
-              }
-              tmem_st32(trow + O_COL + c * 32, o);
-            }
-          }
-          __nv_bfloat16* orow = out + ((size_t)(si.q_row0 + t) * d.q_heads + head * G + g) * D;
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
-            float o[32];
-            tmem_ld32(trow + O_COL + c * 32, o);
+            own(c, 1.f, o);
             if (write) {
 #pragma unroll
-              for (int i = 0; i < 32; i += 8)
-                *reinterpret_cast<uint4*>(orow + c * 32 + i) = make_uint4(
-                    pack_bf16(o[i] * invL, o[i + 1] * invL), pack_bf16(o[i + 2] * invL, o[i + 3] * invL),
-                    pack_bf16(o[i + 4] * invL, o[i + 5] * invL),
-                    pack_bf16(o[i + 6] * invL, o[i + 7] * invL));
+              for (int i = 0; i < 8; ++i)
+                part_rows(d, slot)[(16 * grp + 8 * c + i) * M + r] =
+                    make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
             }
           }
-          tc_fence_before();
-          if (warp == 2 && lane == 0) d.pf_count[seg.seq * H + head] = 0;
+          if (write && grp == 0) d.pf_part_ml[(size_t)slot * M + r] = make_float2(Mr, Lr);
+        }
+        sync_groups();
+        if (first_early) {
+          if (ts == 0) mbar_arrive(&bars[B_PUB]);
+        } else {
+          if (ts == 0)
+            s_last = alone || arrive_acq_rel(&d.pf_count[cur.seq * H + head], nch);
+          sync_groups();
+        }
+        if (!first_early && s_last) {
+          // This CTA's own part is still in the O columns.  Every lane takes part in the
+          // tensor-memory accesses; rows that are padding (or of a warp whose wait gave up)
+          // write nothing.
+          merge_parts(d, us, cur, cf, nch, cta - cf, write, r, grp, Mr, Lr,
+                      [&](int c, float sc, float (&o)[32]) { own(c, sc, o); }, store);
+          flush();
+          if (ts == 0) d.pf_count[cur.seq * H + head] = 0;
         }
       }
+      // Both groups have read O and the (max, sum) pairs before either goes on.
+      tc_fence_before();
+      sync_groups();
     }
   }
 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+  if (warp == 2) tmem_dealloc(tmem, TMEM_COLS);
+  if (!CLUSTER && s_first_last && warp >= 4) {
+    // The first segment's pair was complete when this CTA arrived for it: every part,
+    // this CTA's own too, comes from its slot.
+    const int grp = (warp >> 2) - 1, r = (warp & 3) * 32 + lane, ts = tid - (THREADS - SM_THREADS);
+    const PSeg s = segment_at(info(seq0), seq0, u_begin, u_end);
+    const SeqInfo& si = info(seq0);
+    const int R = si.t * G, cf = us.owner(s.pair_start), nch = cta - cf + 1;
+    uint8_t* st_out = smem + off_out(ring, max_t);
+    merge_parts(
+        d, us, s, cf, nch, -1, r < R, r, grp, -INFINITY, 0.f,
+        [](int, float, float (&o)[32]) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] = 0.f;
+        },
+        [&](int c, const float (&o)[32]) {
+          if (r >= R) return;
+#pragma unroll
+          for (int i = 0; i < 32; i += 8)
+            *reinterpret_cast<uint4*>(st_out + r * ST_PITCH + 128 * grp + 64 * c + 2 * i) =
+                make_uint4(pack_bf16(o[i], o[i + 1]), pack_bf16(o[i + 2], o[i + 3]),
+                           pack_bf16(o[i + 4], o[i + 5]), pack_bf16(o[i + 6], o[i + 7]));
+        });
+    asm volatile("bar.sync 1, %0;" ::"n"(SM_THREADS) : "memory");
+    for (int i = ts; i < R * 16; i += SM_THREADS) {
+      const int row = i >> 4, c = i & 15;
+      __nv_bfloat16* orow =
+          out + ((size_t)(si.q_row0 + row / G) * d.q_heads + s.head * G + row % G) * D;
+      reinterpret_cast<uint4*>(orow)[c] =
+          *reinterpret_cast<const uint4*>(st_out + row * ST_PITCH + c * 16);
+    }
+    if (ts == 0) d.pf_count[seq0 * H + s.head] = 0;
+  }
+  if constexpr (CLUSTER) {
+    if (k_slices == 1) return;
+    const int k = k_slices, slice = cta % k;
+    const SeqInfo& si = info(seg.seq);
+    const int R = si.t * G, per = (R + k - 1) / k;
+    const int r0 = slice * R / k, n_rows = (slice + 1) * R / k - r0;
+    const uint32_t s_recv = smem_u32(smem + off_out(ring, max_t));
+    // Every part goes to slot `slice` of the owner's received rows.
+    for (int i = tid; u_begin == u_end && i < R; i += THREADS)  // no page: weighs nothing
+      *reinterpret_cast<float2*>(smem + OFF_KV + i * ROW_PITCH + D * 4) = make_float2(-INFINITY, 0.f);
+    fence_proxy_async_smem();
+    __syncthreads();
+    cluster_wait();  // every CTA of the cluster has started
+    if (tid < k) {
+      const int f = tid * R / k, nf = (tid + 1) * R / k - f;
+      if (nf > 0)
+        bulk_s2cluster(cluster_map(s_recv + slice * per * ROW_PITCH, tid), sKV + f * ROW_PITCH,
+                       nf * ROW_PITCH, cluster_map(smem_u32(&bars[B_RECV]), tid));
+    }
+    __syncwarp();
+    pdl_wait();
+    const bool got = mbar_wait(d, &bars[B_RECV], 0);
+    __syncwarp();
+    cluster_arrive();
+    // Merge and write this CTA's rows, a 4-element chunk per thread and pass.
+    const uint8_t* rows = smem + off_out(ring, max_t);
+    for (int i = tid; i < n_rows * (D / 4) && got; i += THREADS) {
+      const int rl = i / (D / 4), c = i % (D / 4), row = r0 + rl;
+      const uint8_t* p0 = rows + rl * ROW_PITCH;
+      float2 ml[MAX_K];
+      float4 o[MAX_K];
+#pragma unroll
+      for (int p = 0; p < MAX_K; ++p) {
+        const uint8_t* pr = p0 + min(p, k - 1) * per * ROW_PITCH;
+        ml[p] = p < k ? *reinterpret_cast<const float2*>(pr + D * 4) : make_float2(-INFINITY, 0.f);
+        o[p] = *reinterpret_cast<const float4*>(pr + c * 16);
+      }
+      float mx = -INFINITY;
+#pragma unroll
+      for (int p = 0; p < MAX_K; ++p) mx = fmaxf(mx, ml[p].x);
+      float Ls = 0.f;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int p = 0; p < MAX_K; ++p) {
+        if (ml[p].x == -INFINITY) continue;  // a part without a key of this row
+        const float w = exp2f(ml[p].x - mx);
+        Ls += ml[p].y * w;
+        a.x = fmaf(o[p].x, w, a.x);
+        a.y = fmaf(o[p].y, w, a.y);
+        a.z = fmaf(o[p].z, w, a.z);
+        a.w = fmaf(o[p].w, w, a.w);
+      }
+      const float inv = 1.f / Ls;
+      __nv_bfloat16* orow = out + ((size_t)(si.q_row0 + row / G) * d.q_heads + seg.head * G +
+                                   row % G) * D + c * 4;
+      *reinterpret_cast<uint2*>(orow) =
+          make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
+    }
+    __syncwarp();
+    cluster_wait();  // every part was received: no copy still reads this CTA's rows
+  }
+}
+
+using TcFn = void (*)(Dev, int, const CUtensorMap, const CUtensorMap, const __nv_bfloat16*,
+                      __nv_bfloat16*, float, int, int, int, const __nv_bfloat16*,
+                      const __nv_bfloat16*);
+TcFn tc_kernel(bool fused, bool cluster) {
+  return cluster ? (fused ? &attn_prefill_tc_kernel<true, true> : &attn_prefill_tc_kernel<false, true>)
+                 : (fused ? &attn_prefill_tc_kernel<true, false> : &attn_prefill_tc_kernel<false, false>);
+}
+
+cudaError_t set_attributes() {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(tc_kernel(i & 1, i & 2)),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+  return e;
 }
 
 }  // namespace
 
-const void* prefill_tc_kernel_ptr() {
-  return reinterpret_cast<const void*>(&attn_prefill_tc_kernel<false>);
-}
-int prefill_tc_smem() { return TC_SMEM; }
+const void* prefill_tc_kernel_ptr() { return reinterpret_cast<const void*>(tc_kernel(false, false)); }
+int prefill_tc_smem() { return SMEM_MAX; }
 int prefill_tc_threads() { return THREADS; }
+int prefill_tc_max_slices() { return MAX_K; }
+
+int prefill_tc_max_clusters(int k) {
+  if (set_attributes() != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(k);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM_MAX;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = k;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, tc_kernel(false, true), &cfg) == cudaSuccess ? n : 0;
+}
 
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
-                                   bool pdl, cudaStream_t s, const void* new_k, const void* new_v) {
+                                   int k, int max_t, bool pdl, cudaStream_t s, const void* new_k,
+                                   const void* new_v) {
+  static thread_local const cudaError_t attr_err = set_attributes();
+  if (attr_err != cudaSuccess) return attr_err;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
-  if (new_k != nullptr) {
-    static thread_local const cudaError_t attr = cudaFuncSetAttribute(
-        reinterpret_cast<const void*>(&attn_prefill_tc_kernel<true>),
-        cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-    if (attr != cudaSuccess) return attr;
+  // The deepest ring that leaves room for the rows sent to a CTA (k parts of its share).
+  const int recv = k > 1 ? (max_t * G + k - 1) / k * k : 0;
+  int ring = MAX_RING;
+  while (tc_smem(ring, max_t, recv) > SMEM_MAX) --ring;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = tc_smem(ring, max_t, recv);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (k > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = k;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    ++n;
   }
-  return launch_ex(new_k != nullptr ? &attn_prefill_tc_kernel<true> : &attn_prefill_tc_kernel<false>,
-                   dim3(grid), dim3(THREADS), TC_SMEM, s, pdl, d, layer, lo, hi,
-                   static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out), scale,
-                   static_cast<const __nv_bfloat16*>(new_k), static_cast<const __nv_bfloat16*>(new_v));
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, tc_kernel(new_k != nullptr, k > 0), d, layer, lo, hi,
+                            static_cast<const __nv_bfloat16*>(q),
+                            static_cast<__nv_bfloat16*>(out), scale, ring, max_t, k,
+                            static_cast<const __nv_bfloat16*>(new_k),
+                            static_cast<const __nv_bfloat16*>(new_v));
 }
 
 }  // namespace kvc

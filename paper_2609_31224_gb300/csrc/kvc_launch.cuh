@@ -57,12 +57,20 @@ cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const C
                                      const void* new_v, int n_pairs, bool pdl, cudaStream_t s);
 // new_k / new_v (optional, bfloat16 only): the chunk's rows of this layer, written
 // into the pool by the launch itself (the per-layer order).
+// pages_max, pages_sum: estimates of the sessions' resident pages (largest, sum over the
+// call), for the choice of the split only.
 cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                int max_t, bool pdl, cudaStream_t s, const void* new_k = nullptr,
+                                int max_t, int pages_max, int64_t pages_sum, bool pdl,
+                                cudaStream_t s, const void* new_k = nullptr,
                                 const void* new_v = nullptr);
+// k = 0: stream-K over `grid` CTAs; k >= 1: pair split, grid = pairs * k CTAs.
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
-                                   bool pdl, cudaStream_t s, const void* new_k, const void* new_v);
+                                   int k, int max_t, bool pdl, cudaStream_t s, const void* new_k,
+                                   const void* new_v);
+int prefill_tc_max_slices();
+// Clusters of k CTAs of the pair split that fit the current device at once.
+int prefill_tc_max_clusters(int k);
 const void* prefill_tc_kernel_ptr();
 // Two 2-D views of the bfloat16 pool as rows of 128 elements (columns 0-63 and
 // 64-127), 16-row boxes, 128-byte swizzle; cached per pool.  False if the driver
@@ -73,6 +81,7 @@ int prefill_tc_threads();
 int noalloc_max_pairs();
 cudaError_t launch_attn_decode_noalloc(const Dev& d, int layer, const void* q, void* out,
                                        int n_seq, cudaStream_t s);
+
 int prefill_grid_ctas(const Dev& d);
 
 }  // namespace kvc
