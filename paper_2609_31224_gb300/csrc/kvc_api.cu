@@ -177,7 +177,6 @@ struct kvc_ctx {
   int attn_since_append = 0;  // attention launches since the last append (or layer write)
   uint64_t layers_written = 0;  // layers whose K/V of the last append are in the pool
   bool last_single = false;
-  int pf_target = 0;
   uint32_t dec_epoch = 0;  // tag of the last decode launch's partial states
 };
 
@@ -310,7 +309,6 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
       launch_init(d, cfg->rope_base, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return cleanup(fail(KVC_ECUDA, "initialisation failed: %s",
                         cudaGetErrorString(cudaGetLastError())));
-  ctx->pf_target = 3 * prefill_grid_ctas(d);
   *out = ctx;
   return KVC_OK;
 }
@@ -363,9 +361,6 @@ int kvc_append_chunk(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, const i
   AppendArgs a;
   a.n_seq = n_seq;
   a.total = total;
-  // Only the binary32 prefill kernel reads the per-session chunk list.
-  a.pf_target = ctx->d.esz == 4 ? ctx->pf_target : 0;
-  a.pf_min_blocks = 4;
   for (int i = 0; i < n_seq; ++i) a.sessions[i] = h_sessions[i];
   for (int i = 0; i <= n_seq; ++i) a.cu[i] = h_cu_tokens[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -12,8 +12,6 @@ namespace kvc {
 struct AppendArgs {
   int32_t n_seq;
   int32_t total;
-  int32_t pf_target;       // desired item count of the binary32 prefill's chunk list
-  int32_t pf_min_blocks;
   int32_t sessions[MAX_SEQ];
   int32_t cu[MAX_SEQ + 1];
 };
@@ -71,6 +69,9 @@ cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& l
 int prefill_tc_max_slices();
 // Clusters of k CTAs of the pair split that fit the current device at once.
 int prefill_tc_max_clusters(int k);
+// binary32; pages_max as in launch_attn_prefill, sms: SMs of the device.
+cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void* out, int n_seq,
+                                    int max_t, int pages_max, int sms, bool pdl, cudaStream_t s);
 const void* prefill_tc_kernel_ptr();
 // Two 2-D views of the bfloat16 pool as rows of 128 elements (columns 0-63 and
 // 64-127), 16-row boxes, 128-byte swizzle; cached per pool.  False if the driver
@@ -81,7 +82,5 @@ int prefill_tc_threads();
 int noalloc_max_pairs();
 cudaError_t launch_attn_decode_noalloc(const Dev& d, int layer, const void* q, void* out,
                                        int n_seq, cudaStream_t s);
-
-int prefill_grid_ctas(const Dev& d);
 
 }  // namespace kvc

@@ -163,51 +163,20 @@ __global__ void init_rope_kernel(Dev d, double base) {
 // ---------------------------------------------------------------------------
 // Append, part 1 (one CTA): page demand, allocation, positions and units
 // (warp ballot over UNIT_BEGIN flags), slot tags, state update and the
-// split-K work lists of the attention calls that follow.
+// work split of the attention calls that follow.
 // ---------------------------------------------------------------------------
-__device__ void build_worklist(const Dev& d, int n_seq, int nb, int target, int min_blocks,
-                               int max_items, Item* items, int* s_warp, int* s_total_items) {
-  const int i = threadIdx.x;
-  int total_blocks;
-  (void)block_exclusive_scan(i < n_seq ? nb : 0, &total_blocks, s_warp);
-  int per = max(min_blocks, (int)(((int64_t)total_blocks * d.kv_heads + target - 1) / target));
-  int chunks = 0, base = 0, total_items = 0;
-  for (int iter = 0; iter < 32; ++iter) {
-    chunks = (i < n_seq) ? min(MAX_CHUNKS_PER_SEQ, (nb + per - 1) / per) : 0;
-    base = block_exclusive_scan(chunks, &total_items, s_warp);
-    if ((int64_t)total_items * d.kv_heads <= max_items) break;
-    per *= 2;
-  }
-  if (i < n_seq) {
-    SeqInfo& si = d.seq[i];
-    si.pf_chunks = chunks;
-    si.pf_base = base;
-    for (int c = 0; c < chunks; ++c) {
-      Item it;
-      it.seq = i;
-      it.chunk = c;
-      it.blk_begin = (int)((int64_t)c * nb / chunks);
-      it.blk_end = (int)((int64_t)(c + 1) * nb / chunks);
-      items[base + c] = it;
-    }
-  }
-  if (threadIdx.x == 0) *s_total_items = total_items;
-  __syncthreads();
-}
-
 // A failed append leaves the state as it was and gives the K/V writer and the
 // attention kernels nothing to do.
 __device__ void abandon_append(const Dev& d) {
   d.g->total_tokens = 0;
   d.g->n_units = 0;
-  d.g->n_pf_items = 0;
 }
 
 __global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, AppendArgs a,
                                                                    const uint8_t* types) {
   __shared__ int s_warp[33];
   __shared__ int s_bad;
-  __shared__ int s_total_dec, s_total_pf;
+  __shared__ int s_total_dec;
   const int i = threadIdx.x;
   const int n_seq = a.n_seq;
   if (i == 0) s_bad = 0;
@@ -307,10 +276,9 @@ __global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, Append
     d.seq[i] = si;
   }
   __syncthreads();
-  // 4. Split-K work for the attention calls.  The decode and bfloat16 prefill
-  // kernels split the call's (session, kv head, page) units evenly over their CTAs
-  // (stream-K): they need each session's first unit, the total and the largest
-  // session.  The binary32 prefill kernel takes the per-session chunk list.
+  // 4. Work of the attention calls: the stream-K splits cut the call's (session, kv head,
+  // page) units evenly over their CTAs; they need each session's first unit, the total
+  // and the largest session.
   {
     int total_units;
     const int ubase = block_exclusive_scan(i < n_seq ? nb * d.kv_heads : 0, &total_units, s_warp);
@@ -322,17 +290,10 @@ __global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, Append
     }
     __syncthreads();
   }
-  if (a.pf_target > 0) {
-    build_worklist(d, n_seq, nb, a.pf_target, a.pf_min_blocks, d.max_pf_items, d.pf_items,
-                   s_warp, &s_total_pf);
-  } else if (i == 0) {
-    s_total_pf = 0;
-  }
   if (i == 0) {
     d.g->n_seq = n_seq;
     d.g->total_tokens = a.total;
     d.g->n_units = s_total_dec;
-    d.g->n_pf_items = s_total_pf;
     d.g->pages_used += total_need;
   }
 }
@@ -385,7 +346,7 @@ __global__ void __launch_bounds__(META_THREADS) append_single_kernel(Dev d, Appe
                                                                      const uint8_t* types,
                                                                      const T* k, const T* v) {
   __shared__ int s_warp[33];
-  __shared__ int s_bad, s_total_pf;
+  __shared__ int s_bad;
   __shared__ int s_gs[MAX_SEQ], s_pos[MAX_SEQ];
   const int i = threadIdx.x;
   const int n_seq = a.n_seq;
@@ -468,16 +429,11 @@ __global__ void __launch_bounds__(META_THREADS) append_single_kernel(Dev d, Appe
     d.seq[i] = si;
   }
   __syncthreads();
-  s_total_pf = 0;
-  if (a.pf_target > 0)
-    build_worklist(d, n_seq, nb, a.pf_target, a.pf_min_blocks, d.max_pf_items, d.pf_items,
-                   s_warp, &s_total_pf);
   if (i == 0) {
     d.g->n_seq = n_seq;
     d.g->total_tokens = n_seq;
     d.g->n_units = total_units;
     d.g->nb_max = nb_max;
-    d.g->n_pf_items = s_total_pf;
     d.g->pages_used += total_need;
   }
   if (k == nullptr) return;

@@ -1,6 +1,7 @@
-"""The tcgen05 prefill kernel's two splits against the oracle at the sizes where they can go
-wrong: each number of slices per pair, fewer stages than slices, chunks of 1 to 32 tokens
-in one call, stream-K pairs over two and over many CTAs, with and without the fused write.
+"""The prefill kernels against the oracle at the sizes where their splits can go wrong: 1
+to 8 (binary32: 16) slices per pair, fewer pages than slices, chunks of 1 to 32 tokens in one
+call, the two row-block sizes of binary32, stream-K pairs over two and over many CTAs, with
+and without the fused write.
 """
 import numpy as np
 import pytest
@@ -16,7 +17,7 @@ from synth import values as V  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
-D, L = 128, 2
+L = 2
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -32,43 +33,45 @@ def _history(n):
     return np.array((unit * (n // 20 + 1))[:n], np.uint8)
 
 
-# (tokens of each session's chunk, positions of each session's history, budget).  Pairs are
-# 8 per session: 1, 2, 3, 4, 5 and 9 sessions take 8, 6, 5, 4, 3 and 2 slices, 16 sessions
-# one, 20 sessions stream-K.
+# (tokens of each session's chunk, positions of each session's history, budget); 8 KV heads.
 CASES = {
-    "8 slices, 32 tokens": ([32], [1500], 1200),
-    "8 slices, fewer stages than slices": ([5], [40], -1),
-    "8 slices, first chunk of a session": ([17], [0], -1),
-    "6 slices, 1 and 17 tokens": ([1, 17], [700, 333], 300),
-    "5 slices, 2 to 31 tokens": ([17, 31, 2], [640, 655, 1001], 500),
-    "4 slices": ([17] * 4, [500, 64, 65, 1024], 400),
-    "3 slices": ([17] * 5, [300, 301, 302, 303, 304], 250),
-    "2 slices": ([17, 16, 1, 32, 17, 17, 3, 17, 17], [150 + 37 * i for i in range(9)], 260),
-    "1 slice": ([17] * 16, [20 + 11 * i for i in range(16)], 100),
-    "stream-K, parts of two CTAs": ([17, 1, 32, 8] * 5, [330 + 16 * i for i in range(20)], 400),
-    "stream-K, parts of many CTAs": ([17] * 20, [5000] + [40] * 19, -1),
+    "1 session, 32 tokens": ([32], [1500], 1200),
+    "1 session, fewer stages than slices": ([5], [40], -1),
+    "first chunk of a session": ([17], [0], -1),
+    "1 session, 8 tokens": ([8], [700], 600),
+    "2 sessions, 1 and 17 tokens": ([1, 17], [1700, 1333], 1300),
+    "2 sessions, one with fewer pages than slices": ([17, 17], [1700, 5], 1300),
+    "3 sessions, 2 to 31 tokens": ([17, 31, 2], [1640, 1655, 2001], 1500),
+    "4 sessions": ([17] * 4, [1500, 1064, 1065, 1024], 900),
+    "5 sessions": ([17] * 5, [1300, 1301, 1302, 1303, 1304], 1250),
+    "9 sessions": ([17, 16, 1, 32, 17, 17, 3, 17, 17], [1150 + 37 * i for i in range(9)], 1260),
+    "16 sessions, short": ([17] * 16, [20 + 11 * i for i in range(16)], 100),
+    "20 sessions": ([17, 1, 32, 8] * 5, [330 + 16 * i for i in range(20)], 400),
+    "20 sessions, one much longer": ([17] * 20, [5000] + [40] * 19, -1),
 }
 
 
 @pytest.mark.parametrize("per_layer", [False, True], ids=["whole", "per_layer"])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("name", list(CASES))
-def test_prefill_split(name, per_layer):
+def test_prefill_split(name, dtype, per_layer):
     from paper_2609_31224_gb300 import KVCache
     tokens, hist, budget = CASES[name]
     n, heads, seed = len(tokens), 8, 5
+    D, tdtype = (128, torch.bfloat16) if dtype == "bf16" else (64, torch.float32)
     total = sum(h + t for h, t in zip(hist, tokens))
     pages = [2 * ((h + t) // 16 + 3) for h, t in zip(hist, tokens)]
     cache = KVCache(n_sessions=n, layers=L, q_heads=4 * heads, kv_heads=heads, head_dim=D,
-                    budget=budget, window=2, dtype="bf16", n_pages=sum(pages),
+                    budget=budget, window=2, dtype=dtype, n_pages=sum(pages),
                     max_pages_per_session=max(pages), max_positions=max(hist) + 64,
                     max_seq_per_call=n, max_tokens_per_call=total)
     orc = OracleCache(OracleConfig(n_sessions=n, layers=L, q_heads=4 * heads, kv_heads=heads,
                                    head_dim=D, page_size=16, budget=budget, window=2,
-                                   dtype="bf16", rope_base=10000.0, n_pages=sum(pages)))
+                                   dtype=dtype, rope_base=10000.0, n_pages=sum(pages)))
 
     def fill(tag, h, sess, pos):
-        x = torch.empty((L, len(pos), h, D), dtype=torch.bfloat16, device="cuda")
-        G.fill(x, "bf16", seed, tag, torch.tensor(sess, dtype=torch.int32, device="cuda"),
+        x = torch.empty((L, len(pos), h, D), dtype=tdtype, device="cuda")
+        G.fill(x, dtype, seed, tag, torch.tensor(sess, dtype=torch.int32, device="cuda"),
                torch.tensor(pos, dtype=torch.int32, device="cuda"))
         return x
 
@@ -89,7 +92,7 @@ def test_prefill_split(name, per_layer):
         orc.evict(who)
     chunk = [np.array([0x80] + [0] * (t - 1), np.uint8) for t in tokens]
     cu, k, v, q = append(list(range(n)), chunk, hist, not per_layer)
-    out = torch.full((L, int(cu[-1]), 4 * heads, D), float("nan"), dtype=torch.bfloat16,
+    out = torch.full((L, int(cu[-1]), 4 * heads, D), float("nan"), dtype=tdtype,
                      device="cuda")
     st = torch.cuda.current_stream().cuda_stream
     for _ in range(2):  # the second time overlaps the launches of the first
@@ -102,14 +105,14 @@ def test_prefill_split(name, per_layer):
     assert cache.device_status()[1] == 0
 
     def kv_source(s, layer, positions):
-        return tuple(V.layer_tensor(seed, tag, s, layer, positions, heads, D, "bf16")
+        return tuple(V.layer_tensor(seed, tag, s, layer, positions, heads, D, dtype)
                      .astype(np.float64) for tag in (V.TAG_K, V.TAG_V))
 
     got = out.float().cpu().numpy()
     layer = L - 1
     picked = sorted(set([0, n // 2, n - 1]))
     qs = [V.layer_tensor(seed, V.TAG_Q, s, layer, range(hist[s], hist[s] + tokens[s]), 4 * heads,
-                         D, "bf16") for s in picked]
+                         D, dtype) for s in picked]
     for s, ref in zip(picked, orc.attend(layer, qs, kv_source, sessions=picked)):
-        assert_close(got[layer, cu[s]:cu[s + 1]], ref, "bf16", f"{name}, session {s}")
+        assert_close(got[layer, cu[s]:cu[s + 1]], ref, dtype, f"{name}, session {s}")
     assert np.isfinite(got).all()
