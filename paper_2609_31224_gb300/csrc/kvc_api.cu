@@ -403,7 +403,7 @@ int kvc_append_kv_layer(kvc_ctx* ctx, int layer, const void* d_k, const void* d_
   if (!aligned16(d_k) || !aligned16(d_v)) return fail(KVC_EINVAL, "d_k / d_v must be 16-byte aligned");
   if (!ctx->attn_valid)
     return fail(KVC_ESTATE, "kvc_append_kv_layer needs a preceding kvc_append_chunk (no evict/release after it)");
-  KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v,
+  KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false,
                                 static_cast<cudaStream_t>(stream)));
   ctx->layers_written |= 1ull << layer;
   // The next attention launch must not start early: its prologue loads pages
@@ -552,7 +552,7 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
                                  ctx->attn_since_append > 0, s, d_k, d_v));
   } else {
     // Binary32 (CUDA-core prefill): the rows first, then the attention, unoverlapped.
-    KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, s));
+    KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false, s));
     KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
                                ctx->est_pages_max, ctx->est_pages_sum,
                                  false, s));
