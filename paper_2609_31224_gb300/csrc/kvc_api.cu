@@ -473,7 +473,7 @@ int kvc_attn_decode(kvc_ctx* ctx, int layer, const void* d_q, void* d_out, void*
   // new token's K/V, so it does not start early; later ones may.
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
-  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq,
+  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
                               ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream),
                               epoch));
   ++ctx->attn_since_append;
@@ -493,7 +493,7 @@ int kvc_attn_decode_kv(kvc_ctx* ctx, int layer, const void* d_k, const void* d_v
   // after their loads, and the previous launch writes another layer's rows only.
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
-  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq,
+  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
                               ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream),
                               epoch, d_k, d_v));
   ctx->layers_written |= 1ull << layer;

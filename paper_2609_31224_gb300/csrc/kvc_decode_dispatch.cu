@@ -1,10 +1,12 @@
 // Dispatch of a decode attention call (one token per session) between the three
-// kernel shapes, by the number of (session, KV head) pairs it has:
-//   - pair split, 16-warp CTAs (one per SM): every pair gets k >= 5 CTAs in one
-//     wave (at most 3 sessions of 8 KV heads on 152 SMs); for bfloat16 the pages run
-//     on the tensor cores;
+// kernel shapes, by the number of (session, KV head) pairs it has and the pages of its
+// longest session (estimated on the host):
+//   - pair split, 16-warp CTAs (one per SM): sessions of 100 pages or more when every
+//     pair gets k >= 5 CTAs in one wave (at most 3 sessions of 8 KV heads on 152 SMs); for
+//     bfloat16 the pages run on the tensor cores;
 //   - pair split, 4-warp CTAs (three per SM, tensor-core pages for bfloat16): every
-//     pair gets k >= 1 CTAs in one wave (with k = 1 a pair needs no merge);
+//     other call whose pairs each get k >= 1 CTAs in one wave (with k = 1 a pair needs no
+//     merge);
 //   - stream-K over (session, KV head, page) units, tensor-core pages for bfloat16:
 //     the rest (more pairs than the 4-warp shape's resident CTAs, e.g. the full-batch
 //     rounds of 64 sessions).
@@ -31,12 +33,38 @@ constexpr int DEC_MIN_UNITS = 12;
 // faster from 4 sessions on (15.4 against 16.7 us at 4, 26.4 against 28.1 at 9) and
 // slower below (11.7 against 8.1 at 1).
 constexpr int SPLIT_MIN_K = 5, SPLIT4_MIN_K = 1;
+// Below this many pages the 16-warp shape leaves most of its warps without one
+// (64 pages, 8 pairs: 6.8 us against 6.4-6.7 with 4 warps; 20 pages: 6.7 against 5.2).
+constexpr int WIDE_MIN_PAGES = 100;
+
+// Slices per pair of the 16-warp shape: no more than give each warp a page (257 pages, 8
+// pairs: 7.6 us at 17 slices, 7.9 at 19, 8.9 at 15; 4 pairs: 7.2 at 19, 8.4 at 38).
+int wide_slices(int slots, int n_pairs, int pages) {
+  return min(MAX_PARTS, min(slots / n_pairs, (pages + 15) / 16));
+}
+
+// ... and of the 4-warp shape: up to 5/6 of the slots for as long as that leaves 6 slices or
+// more, all of them beyond (257 pages: 14.5 us at 12 slices of 32 pairs, 15.0 at 14; 18.9 at 8
+// of 48, 19.6 at 9; but 26.0 at 6 of 72, 26.5 at 5), and about three pages per slice at least
+// (33 pages, one binary32 pair: 4.7 us at 12 slices, 9.9 at 64; 20 pages, 8 pairs: 5.2 at 8,
+// 6.1 at 12; 17 pages: 4.5 at 6, 9.3 at 64).  The CUDA-core pages of binary32 are bound by
+// the pages of a warp: there more slices are taken if they save a warp one (48 pairs of 130
+// pages: 12.0 us at 9 slices, 12.5 at 8).
+int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
+  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs;
+  int fit = five_sixths >= 6 ? five_sixths : slots / n_pairs;
+  // (Two more pages than estimated: the partly filled ones of both regions.)
+  auto warp_pages = [&](int k) { return ((pages + 2 + k - 1) / k + 3) / 4; };
+  for (int k = fit + 1; cuda_cores && k <= slots / n_pairs; ++k)
+    if (warp_pages(k) < warp_pages(fit)) fit = k;
+  return max(1, min(MAX_PARTS, min(fit, (pages + 2) / 3)));
+}
 
 }  // namespace
 
 cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               bool pdl, cudaStream_t s, uint32_t epoch, const void* new_k,
-                               const void* new_v) {
+                               int pages, bool pdl, cudaStream_t s, uint32_t epoch,
+                               const void* new_k, const void* new_v) {
   const int esz = d.esz;
   // Grid sizes of the three shapes, per element type (their CTA shapes differ), worked
   // out on a thread's first call with that type.
@@ -53,8 +81,9 @@ cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out
   const int grid = sh.grid, slots = sh.slots, slots4 = sh.slots4;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   const int n_pairs = n_seq * d.kv_heads;
-  const int k = n_pairs * SPLIT_MIN_K <= slots ? min(MAX_PARTS, slots / n_pairs) : 0;
-  const int k4 = k == 0 && n_pairs * SPLIT4_MIN_K <= slots4 ? min(MAX_PARTS, slots4 / n_pairs) : 0;
+  const int k = n_pairs * SPLIT_MIN_K <= slots && pages >= WIDE_MIN_PAGES
+                    ? wide_slices(slots, n_pairs, pages) : 0;
+  const int k4 = k == 0 && n_pairs * SPLIT4_MIN_K <= slots4 ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
   // Tensor maps of the pool for the tensor-core page loop (bfloat16).
   CUtensorMap map_lo, map_hi;
   memset(&map_lo, 0, sizeof(map_lo));

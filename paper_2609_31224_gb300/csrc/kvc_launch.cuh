@@ -36,8 +36,9 @@ cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_o
 // new_k / new_v (optional): the fused per-layer write of the new tokens' K/V.
 // epoch: tag of this launch's partial states (nonzero, never reused while tags
 // of it may remain in the slots); 0 selects the fenced arrival instead.
+// pages: estimate of the longest session's pages, for the choice of the split only.
 cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               bool pdl, cudaStream_t s, uint32_t epoch,
+                               int pages, bool pdl, cudaStream_t s, uint32_t epoch,
                                const void* new_k = nullptr, const void* new_v = nullptr);
 // Stream-K decode kernel (kvc_attn_decode.cu): its grid (resident CTAs, capped by
 // the partial slots) and its launch.
