@@ -39,15 +39,15 @@ UNIT = "audio-s/s"
 
 # DRAM bytes per algorithmic byte of the roofline kernel (reads + writes), from one
 # ncu capture of the stream-K kernel on the 64-session, two-layer case (the bench's
-# launch shape; smaller calls run the pair-split kernel): 1,088.57 MB of traffic
-# (1,084.41 MB read, 4.16 MB written) for a 1,077.10 MB launch.  Valid only while the
+# launch shape; smaller calls may run the pair-split kernel): 1,085.39 MB of traffic
+# (1,082.53 MB read, 2.86 MB written) for a 1,077.10 MB launch.  Valid only while the
 # decode sources hash to the version it was taken on; the roofline's traffic is null
 # otherwise.
-DECODE_TRAFFIC_RATIO = 1088.57 / 1077.10
+DECODE_TRAFFIC_RATIO = 1085.39 / 1077.10
 DECODE_TRAFFIC_SOURCES = ("paper_2609_31224_gb300/csrc/kvc_attn_decode.cu",
                           "paper_2609_31224_gb300/csrc/kvc_decode_common.cuh",
                           "paper_2609_31224_gb300/csrc/kvc_internal.cuh")
-DECODE_TRAFFIC_SHA256 = "1e7582c380f739e8b63919fc568b9687161723d1076652b086603f3e9759a8e7"
+DECODE_TRAFFIC_SHA256 = "3d10ae39fc6f95d5358d2fd8671f631631448302659143c429b91f1c8aff59d7"
 
 
 def code_only(text: str) -> str:
@@ -79,14 +79,14 @@ def decode_traffic(alg_bytes_per_launch):
 def decode_kernel_label(w) -> str:
     """Kernel that the library's dispatch gives a full-batch decode call of `w` (sessions
     at full budget): the 16-warp pair split while every (session, KV head) pair gets five
-    one-CTA-per-SM slices, the 4-warp pair split while it gets one of the three CTAs per
-    SM, else stream-K."""
+    one-CTA-per-SM slices, the 4-warp pair split while it gets two of the three CTAs per
+    SM, or one with at least 7/8 of them taken, else stream-K."""
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     pairs = w.n_sessions * w.kv_heads
     if 5 * pairs <= sms:
         return "attn_decode_split_kernel (16 warps)"
-    if pairs <= 3 * sms:
+    if 2 * pairs <= 3 * sms or 3 * sms * 7 // 8 < pairs <= 3 * sms:
         return "attn_decode_split_kernel (4 warps)"
     return "attn_decode_kernel"
 

@@ -35,7 +35,7 @@ int fail(int code, const char* fmt, ...) {
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Sizes {
-  int max_moves, max_alloc, dec_slots, dec_tag_slots, max_pf_items;
+  int max_moves, max_alloc, dec_slots, dec_tag_slots, pf_slots;
 };
 
 Sizes derive_sizes(const kvc_config& c) {
@@ -47,9 +47,8 @@ Sizes derive_sizes(const kvc_config& c) {
   s.dec_slots = 4096;
   // Tagged partial slots of the pair-split decode (one per CTA of its one-wave grid).
   s.dec_tag_slots = 2048;
-  // Prefill partial slots: the binary32 kernel's chunk list, and two per CTA of the
-  // bfloat16 kernel's stream-K split.
-  s.max_pf_items = (int)std::min<int64_t>(2048, std::max<int64_t>(512, (int64_t)c.max_seq_per_call * c.kv_heads * 4));
+  // Prefill partial slots: two per CTA of the bfloat16 kernel's stream-K split.
+  s.pf_slots = c.dtype == KVC_BF16 ? 512 : 0;
   return s;
 }
 
@@ -77,7 +76,6 @@ size_t layout_meta(const kvc_config& c, uint8_t* base, Dev* d) {
   uint8_t* glob = take(sizeof(DevGlobals));
   uint8_t* rope = take((size_t)c.max_positions * (c.head_dim / 2) * sizeof(float2));
   uint8_t* seq = take((size_t)c.max_seq_per_call * sizeof(SeqInfo));
-  uint8_t* pi = take((size_t)z.max_pf_items * sizeof(Item));
   uint8_t* ts = take((size_t)c.max_tokens_per_call * 4);
   uint8_t* tp = take((size_t)c.max_tokens_per_call * 4);
   uint8_t* mv = take((size_t)z.max_moves * sizeof(int2));
@@ -85,8 +83,8 @@ size_t layout_meta(const kvc_config& c, uint8_t* base, Dev* d) {
   uint8_t* dpo = take((size_t)z.dec_slots * G * c.head_dim * 4);
   uint8_t* dpm = take((size_t)z.dec_slots * G * sizeof(float2));
   uint8_t* dtg = take((size_t)z.dec_tag_slots * (G * c.head_dim + 2 * G) * 8);
-  uint8_t* ppo = take((size_t)z.max_pf_items * PF_MAX_TOKENS * G * 128 * 4);
-  uint8_t* ppm = take((size_t)z.max_pf_items * PF_MAX_TOKENS * G * sizeof(float2));
+  uint8_t* ppo = take((size_t)z.pf_slots * PF_MAX_TOKENS * G * 128 * 4);
+  uint8_t* ppm = take((size_t)z.pf_slots * PF_MAX_TOKENS * G * sizeof(float2));
   uint8_t* dc = take((size_t)c.max_seq_per_call * c.kv_heads * 4);
   uint8_t* pc = take((size_t)c.max_seq_per_call * c.kv_heads * 4);
   off = align_up(off, 256);
@@ -101,7 +99,6 @@ size_t layout_meta(const kvc_config& c, uint8_t* base, Dev* d) {
     d->g = reinterpret_cast<DevGlobals*>(glob);
     d->rope = reinterpret_cast<float2*>(rope);
     d->seq = reinterpret_cast<SeqInfo*>(seq);
-    d->pf_items = reinterpret_cast<Item*>(pi);
     d->tok_slot = reinterpret_cast<int32_t*>(ts);
     d->tok_pos = reinterpret_cast<int32_t*>(tp);
     d->moves = reinterpret_cast<int2*>(mv);
@@ -117,7 +114,7 @@ size_t layout_meta(const kvc_config& c, uint8_t* base, Dev* d) {
     d->max_moves = z.max_moves;
     d->max_alloc = z.max_alloc;
     d->dec_slots = z.dec_slots;
-    d->max_pf_items = z.max_pf_items;
+    d->pf_slots = z.pf_slots;
     d->bitmap_words = words;
   }
   return off;
@@ -469,8 +466,8 @@ int kvc_attn_decode(kvc_ctx* ctx, int layer, const void* d_q, void* d_out, void*
   if (rc) return rc;
   if (!ctx->last_single)
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
-  // The first attention launch after an append follows the kernel that wrote the
-  // new token's K/V, so it does not start early; later ones may.
+  // The first attention launch after an append follows the kernel that wrote the new
+  // token's K/V, so it reads nothing before that is complete; later ones may.
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
   KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,

@@ -38,7 +38,7 @@ template <typename T, int D, bool FUSED>
 __global__ void __launch_bounds__(SkCfg<T, D>::THREADS) attn_decode_kernel(
     Dev d, int layer, const __grid_constant__ CUtensorMap map_lo,
     const __grid_constant__ CUtensorMap map_hi, const T* __restrict__ q, T* __restrict__ out,
-    float qk_scale, int min_units, const T* new_k, const T* new_v) {
+    float qk_scale, int min_units, int early, const T* new_k, const T* new_v) {
   using C = SkCfg<T, D>;
   static_assert(C::WARPS == G, "the split-K merge maps one warp to one query row");
   extern __shared__ __align__(128) uint8_t smem[];
@@ -50,7 +50,9 @@ __global__ void __launch_bounds__(SkCfg<T, D>::THREADS) attn_decode_kernel(
   __syncthreads();
   // The next attention call may start its CTAs as soon as slots free up.  Before
   // pdl_wait() this kernel reads only what the append wrote (work list, page
-  // tables, K/V pages); q, outputs, partials and counters come after it.
+  // tables, K/V pages); q, outputs, partials and counters come after it.  The first call
+  // after an append (!early) waits for that append before it lets anything else start.
+  if (!early) pdl_wait();
   pdl_launch_dependents();
   bool waited = false;
 
@@ -177,22 +179,22 @@ int decode_stream_k_grid(const Dev& d) {
 cudaError_t launch_attn_decode_streamk(const Dev& d, int layer, const CUtensorMap& map_lo,
                                        const CUtensorMap& map_hi, const void* q, void* out,
                                        float scale, int grid, int min_units, const void* new_k,
-                                       const void* new_v, bool pdl, cudaStream_t s) {
+                                       const void* new_v, bool early, cudaStream_t s) {
   if (d.esz == 2) {
     using T = __nv_bfloat16;
     const T* nk = static_cast<const T*>(new_k);
     const T* nv = static_cast<const T*>(new_v);
     return launch_ex(nk ? &attn_decode_kernel<T, 128, true> : &attn_decode_kernel<T, 128, false>,
-                     dim3(grid), dim3(SkCfg<T, 128>::THREADS), SkCfg<T, 128>::SMEM, s, pdl, d,
+                     dim3(grid), dim3(SkCfg<T, 128>::THREADS), SkCfg<T, 128>::SMEM, s, true, d,
                      layer, map_lo, map_hi, static_cast<const T*>(q), static_cast<T*>(out), scale,
-                     min_units, nk, nv);
+                     min_units, (int)early, nk, nv);
   }
   const float* nk = static_cast<const float*>(new_k);
   const float* nv = static_cast<const float*>(new_v);
   return launch_ex(nk ? &attn_decode_kernel<float, 64, true> : &attn_decode_kernel<float, 64, false>,
-                   dim3(grid), dim3(SkCfg<float, 64>::THREADS), SkCfg<float, 64>::SMEM, s, pdl, d,
+                   dim3(grid), dim3(SkCfg<float, 64>::THREADS), SkCfg<float, 64>::SMEM, s, true, d,
                    layer, map_lo, map_hi, static_cast<const float*>(q), static_cast<float*>(out),
-                   scale, min_units, nk, nv);
+                   scale, min_units, (int)early, nk, nv);
 }
 
 }  // namespace kvc

@@ -165,7 +165,7 @@ template <typename T, int D, bool FUSED, class C>
 __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
     Dev d, int layer, const __grid_constant__ CUtensorMap map_lo,
     const __grid_constant__ CUtensorMap map_hi, const T* __restrict__ q, T* __restrict__ out,
-    float qk_scale, int k, uint32_t epoch, const T* new_k, const T* new_v) {
+    float qk_scale, int k, uint32_t epoch, int early, const T* new_k, const T* new_v) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Smem<C> sm(smem, warp);
@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
   const int seq = pair / d.kv_heads, head = pair % d.kv_heads;
   init_warp_barriers<C>(sm.wbars, lane);
   __syncthreads();
+  if (!early) pdl_wait();  // (as in the stream-K kernel)
   pdl_launch_dependents();
 
   const SeqInfo si = d.seq[seq];
@@ -271,12 +272,12 @@ template <typename T, int D, class C>
 cudaError_t launch_split(const Dev& d, int layer, const CUtensorMap& map_lo,
                          const CUtensorMap& map_hi, const void* q, void* out, float scale, int k,
                          uint32_t epoch, const void* new_k, const void* new_v, int n_pairs,
-                         bool pdl, cudaStream_t s) {
+                         bool early, cudaStream_t s) {
   const bool fused = new_k != nullptr;
   return launch_ex(fused ? &attn_decode_split_kernel<T, D, true, C>
                          : &attn_decode_split_kernel<T, D, false, C>,
-                   dim3(n_pairs * k), dim3(C::THREADS), C::SMEM, s, pdl, d, layer, map_lo, map_hi,
-                   static_cast<const T*>(q), static_cast<T*>(out), scale, k, epoch,
+                   dim3(n_pairs * k), dim3(C::THREADS), C::SMEM, s, true, d, layer, map_lo, map_hi,
+                   static_cast<const T*>(q), static_cast<T*>(out), scale, k, epoch, (int)early,
                    static_cast<const T*>(new_k), static_cast<const T*>(new_v));
 }
 
@@ -297,19 +298,19 @@ bool decode_split_uses_tma(int esz, bool wide) {
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
                                      float scale, int k, uint32_t epoch, const void* new_k,
-                                     const void* new_v, int n_pairs, bool pdl, cudaStream_t s) {
+                                     const void* new_v, int n_pairs, bool early, cudaStream_t s) {
   if (d.esz == 2) {
     if (wide)
       return launch_split<__nv_bfloat16, 128, SpCfg<__nv_bfloat16, 128>>(
-          d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, pdl, s);
+          d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, early, s);
     return launch_split<__nv_bfloat16, 128, Sp4Cfg<__nv_bfloat16, 128>>(
-        d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, pdl, s);
+        d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, early, s);
   }
   if (wide)
     return launch_split<float, 64, SpCfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k,
-                                                     epoch, new_k, new_v, n_pairs, pdl, s);
+                                                     epoch, new_k, new_v, n_pairs, early, s);
   return launch_split<float, 64, Sp4Cfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k,
-                                                    epoch, new_k, new_v, n_pairs, pdl, s);
+                                                    epoch, new_k, new_v, n_pairs, early, s);
 }
 
 }  // namespace kvc

@@ -148,7 +148,7 @@ int prefill_slices(const TcLimits& lim, int n_pairs, double s_max, double total)
 }  // namespace
 
 cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                int max_t, int pages_max, int64_t pages_sum, bool pdl,
+                                int max_t, int pages_max, int64_t pages_sum, bool early,
                                 cudaStream_t s, const void* new_k, const void* new_v) {
   if (d.esz == 2) {
     static thread_local const TcLimits lim;
@@ -158,12 +158,12 @@ cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* ou
     const int k = prefill_slices(lim, n_pairs, (pages_max + 3) / 4,
                                  (double)d.kv_heads * (pages_sum / 4.0 + n_seq));
     // Each CTA of the stream-K split may write two partial slots.
-    const int grid = k > 0 ? n_pairs * k : std::min(lim.grid, d.max_pf_items / 2);
-    return launch_attn_prefill_tc(d, layer, lo, hi, q, out, grid, k, max_t, pdl, s, new_k, new_v);
+    const int grid = k > 0 ? n_pairs * k : std::min(lim.grid, d.pf_slots / 2);
+    return launch_attn_prefill_tc(d, layer, lo, hi, q, out, grid, k, max_t, early, s, new_k, new_v);
   }
   if (new_k != nullptr) return cudaErrorInvalidValue;  // binary32: the API writes the rows first
   static thread_local const int sms = sm_count();
-  return launch_attn_prefill_f32(d, layer, q, out, n_seq, max_t, pages_max, sms, pdl, s);
+  return launch_attn_prefill_f32(d, layer, q, out, n_seq, max_t, pages_max, sms, early, s);
 }
 
 }  // namespace kvc

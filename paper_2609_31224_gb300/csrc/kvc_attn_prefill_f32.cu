@@ -106,13 +106,17 @@ __device__ inline float4 merge_chunk(uint32_t a_ml, uint32_t a_o, int k) {
 template <int RT>
 __global__ void __launch_bounds__(THREADS, 2) attn_prefill_f32_kernel(
     Dev d, int layer, const float* __restrict__ q, float* __restrict__ out, float qk_scale,
-    int n_rb, int k) {
+    int n_rb, int k, int early) {
   using S = Shape<RT>;
   extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int slice = blockIdx.x % k, rb = blockIdx.x / k % n_rb, pair = blockIdx.x / k / n_rb;
   const int H = d.kv_heads, seq = pair / H, head = pair % H;
-  if (d.g->n_units == 0) return;  // the append failed: the whole grid has nothing to do
+  if (!early) pdl_wait();  // the first call after an append waits for it
+  if (d.g->n_units == 0) {  // the append failed: the whole grid has nothing to do
+    pdl_wait();
+    return;
+  }
   const SeqInfo si = d.seq[seq];
   pdl_launch_dependents();
   const int row0 = rb * S::ROWS, R = min(S::ROWS, si.t * G - row0);  // R <= 0: no rows here
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(THREADS, 2) attn_prefill_f32_kernel(
 
 template <int RT>
 cudaError_t launch(const Dev& d, int layer, const void* q, void* out, int n_pairs, int n_rb, int k,
-                   bool spread, bool pdl, cudaStream_t s) {
+                   bool spread, bool early, cudaStream_t s) {
   static thread_local const cudaError_t attr_err = [] {
     const void* fn = reinterpret_cast<const void*>(&attn_prefill_f32_kernel<RT>);
     const cudaError_t e =
@@ -349,21 +353,20 @@ cudaError_t launch(const Dev& d, int layer, const void* q, void* out, int n_pair
     attr[n].val.clusterDim.z = 1;
     ++n;
   }
-  if (pdl) {
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n].val.programmaticStreamSerializationAllowed = 1;
-    ++n;
-  }
+  attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[n].val.programmaticStreamSerializationAllowed = 1;
+  ++n;
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, &attn_prefill_f32_kernel<RT>, d, layer,
-                            static_cast<const float*>(q), static_cast<float*>(out), scale, n_rb, k);
+                            static_cast<const float*>(q), static_cast<float*>(out), scale, n_rb, k,
+                            (int)early);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                    int max_t, int pages_max, int sms, bool pdl, cudaStream_t s) {
+                                    int max_t, int pages_max, int sms, bool early, cudaStream_t s) {
   // Rows per CTA: 32 (chunks of up to 8 tokens) or 72 (a 17-token unit's 68).
   const int R = max_t * G, n_pairs = n_seq * d.kv_heads;
   const bool small = R <= 32;
@@ -381,8 +384,8 @@ cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void
   k = max(1, min(k, pages_max / 2));
   // A small grid's clusters are spread over the SMs (4 pairs: 13.0 against 14.6 us).
   const bool spread = 2 * blocks * k <= sms;
-  return small ? launch<4>(d, layer, q, out, n_pairs, n_rb, k, spread, pdl, s)
-               : launch<9>(d, layer, q, out, n_pairs, n_rb, k, spread, pdl, s);
+  return small ? launch<4>(d, layer, q, out, n_pairs, n_rb, k, spread, early, s)
+               : launch<9>(d, layer, q, out, n_pairs, n_rb, k, spread, early, s);
 }
 
 }  // namespace kvc

@@ -268,7 +268,7 @@ template <bool FUSED, bool CLUSTER>
 __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     Dev d, int layer, const __grid_constant__ CUtensorMap map_lo,
     const __grid_constant__ CUtensorMap map_hi, const __nv_bfloat16* __restrict__ q,
-    __nv_bfloat16* __restrict__ out, float qk_scale, int ring, int max_t, int k_slices,
+    __nv_bfloat16* __restrict__ out, float qk_scale, int ring, int max_t, int k_slices, int early,
     const __nv_bfloat16* __restrict__ new_k, const __nv_bfloat16* __restrict__ new_v) {
   extern __shared__ uint8_t smem_raw[];
   // (The same offset in every CTA, so that cluster_map() of an address finds the peer's.)
@@ -279,7 +279,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
   volatile int& s_abort = s_abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = d.kv_heads, L = d.layers;
-  if (CLUSTER && d.g->n_units == 0) return;  // the append failed: nothing to do for any CTA
+  // The first call after an append waits for it (and lets nothing else start before that).
+  if (!early) pdl_wait();
+  if (CLUSTER && d.g->n_units == 0) {  // the append failed: nothing to do for any CTA
+    pdl_wait();
+    return;
+  }
   if (tid == 0) {
     for (int s = 0; s < ring; ++s) {
       mbar_init(&bars[B_K_FULL + s], 1);
@@ -373,7 +378,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
   // Stream-K: a pair's CTAs arrive at its counter.  The first segment's partial state (of a
   // pair that ends inside the range) is published when its segment ends but nothing waits
   // for the arrival; the last one's is not even published when every other part is there.
-  const bool early = !CLUSTER && u_begin < u_end && seg.u != seg.pair_start && seg.end < u_end;
+  const bool defer = !CLUSTER && u_begin < u_end && seg.u != seg.pair_start && seg.end < u_end;
 
   if (warp < 2) {
     // ---------------- producers ----------------
@@ -389,7 +394,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     const CUtensorMap* map = (lane & 1) ? &map_hi : &map_lo;
     uint8_t* dst = smem + OFF_KV + (is_v ? 2 * KV_PANEL : 0) + (lane & 1) * KV_PANEL + pg * 2048;
     const uint64_t policy = evict_first_policy();
-    bool arrive_first = is_v && early;  // (lane 0) the first pair's arrival is still to come
+    bool arrive_first = is_v && defer;  // (lane 0) the first pair's arrival is still to come
     const int first_cf = us_first_part(us, seg), first_pair = seg.seq * H + seg.head;
     const int first_nch = cta - first_cf + 1;
     uint32_t n = 0;          // stages produced
@@ -886,7 +891,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
         // Split-K: publish this part's (O, max, sum); the last CTA to arrive for the
         // (session, head) merges every part, half a query row per thread.  Every softmax
         // warp reaches the same named barriers.
-        const bool first_early = first && early, last = u >= u_end;
+        const bool deferred = first && defer, last = u >= u_end;
         if (last) wait(&bars[B_PEEK], 0);
         const bool alone = last && !dead && s_peek;  // every other part is there
         const int cf = us.owner(cur.pair_start), nch = us.owner(cur.pair_end - 1) - cf + 1;
@@ -906,14 +911,14 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
           if (write && grp == 0) d.pf_part_ml[(size_t)slot * M + r] = make_float2(Mr, Lr);
         }
         sync_groups();
-        if (first_early) {
+        if (deferred) {
           if (ts == 0) mbar_arrive(&bars[B_PUB]);
         } else {
           if (ts == 0)
             s_last = alone || arrive_acq_rel(&d.pf_count[cur.seq * H + head], nch);
           sync_groups();
         }
-        if (!first_early && s_last) {
+        if (!deferred && s_last) {
           // This CTA's own part is still in the O columns.  Every lane takes part in the
           // tensor-memory accesses; rows that are padding (or of a warp whose wait gave up)
           // write nothing.
@@ -1029,7 +1034,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
 }
 
 using TcFn = void (*)(Dev, int, const CUtensorMap, const CUtensorMap, const __nv_bfloat16*,
-                      __nv_bfloat16*, float, int, int, int, const __nv_bfloat16*,
+                      __nv_bfloat16*, float, int, int, int, int, const __nv_bfloat16*,
                       const __nv_bfloat16*);
 TcFn tc_kernel(bool fused, bool cluster) {
   return cluster ? (fused ? &attn_prefill_tc_kernel<true, true> : &attn_prefill_tc_kernel<false, true>)
@@ -1070,7 +1075,7 @@ int prefill_tc_max_clusters(int k) {
 
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
-                                   int k, int max_t, bool pdl, cudaStream_t s, const void* new_k,
+                                   int k, int max_t, bool early, cudaStream_t s, const void* new_k,
                                    const void* new_v) {
   static thread_local const cudaError_t attr_err = set_attributes();
   if (attr_err != cudaSuccess) return attr_err;
@@ -1093,16 +1098,14 @@ cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& l
     attr[n].val.clusterDim.z = 1;
     ++n;
   }
-  if (pdl) {
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n].val.programmaticStreamSerializationAllowed = 1;
-    ++n;
-  }
+  attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[n].val.programmaticStreamSerializationAllowed = 1;
+  ++n;
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, tc_kernel(new_k != nullptr, k > 0), d, layer, lo, hi,
                             static_cast<const __nv_bfloat16*>(q),
-                            static_cast<__nv_bfloat16*>(out), scale, ring, max_t, k,
+                            static_cast<__nv_bfloat16*>(out), scale, ring, max_t, k, (int)early,
                             static_cast<const __nv_bfloat16*>(new_k),
                             static_cast<const __nv_bfloat16*>(new_v));
 }

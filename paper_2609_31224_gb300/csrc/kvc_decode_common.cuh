@@ -136,11 +136,13 @@ struct Segment {
   int pwin, pid;
   const CUtensorMap* map_lo;  // tensor maps of the pool (tensor-core page loop only)
   const CUtensorMap* map_hi;
+  uint64_t policy;
 
   __device__ void init(const Dev& d, const SeqInfo& s, int h, int b0, int nb, int warp,
                        const CUtensorMap* mlo = nullptr, const CUtensorMap* mhi = nullptr) {
     map_lo = mlo;
     map_hi = mhi;
+    policy = evict_first_policy();
     si = s;
     head = h;
     blk_begin = b0;
@@ -161,20 +163,21 @@ struct Segment {
       pid = j < n_my ? block_page(si, hrow, lrow, blk_begin + warp + j * C::WARPS) : 0;
     }
     const int page = __shfl_sync(FULL, pid, k - pwin);
-    if (lane == 0) {
-      const uint32_t n = loads + k;
-      const int st = n % C::STAGES;
-      uint8_t* dst = sm.tiles + st * 2 * C::TILE;
-      mbar_arrive_expect_tx(&sm.wbars[st], 2 * C::TILE);
-      if constexpr (C::MMA) {
-        // Pool rows of the K and V tiles, each as two swizzled 64-column boxes.
-        const int krow = (((page * d.layers + layer) * 2) * d.kv_heads + head) * PS;
-        const int vrow = krow + d.kv_heads * PS;
-        tma_load_2d(dst, map_lo, 0, krow, &sm.wbars[st]);
-        tma_load_2d(dst + C::TILE / 2, map_hi, 0, krow, &sm.wbars[st]);
-        tma_load_2d(dst + C::TILE, map_lo, 0, vrow, &sm.wbars[st]);
-        tma_load_2d(dst + C::TILE + C::TILE / 2, map_hi, 0, vrow, &sm.wbars[st]);
-      } else {
+    const uint32_t n = loads + k;
+    const int st = n % C::STAGES;
+    uint8_t* dst = sm.tiles + st * 2 * C::TILE;
+    if constexpr (C::MMA) {
+      // K and V tiles, each as two swizzled 64-column boxes, one box per lane.
+      if (lane == 0) mbar_arrive_expect_tx(&sm.wbars[st], 2 * C::TILE);
+      __syncwarp();
+      if (lane < 4) {
+        const int row = (((page * d.layers + layer) * 2 + (lane >> 1)) * d.kv_heads + head) * PS;
+        tma_load_2d_hint(dst + lane * (C::TILE / 2), (lane & 1) ? map_hi : map_lo, 0, row,
+                         &sm.wbars[st], policy);
+      }
+    } else {
+      if (lane == 0) {
+        mbar_arrive_expect_tx(&sm.wbars[st], 2 * C::TILE);
         const T* kp = reinterpret_cast<const T*>(d.pool) +
                       pool_offset_elems(d, page, layer, 0, head, 0);
         bulk_g2s(dst, kp, C::TILE, &sm.wbars[st]);

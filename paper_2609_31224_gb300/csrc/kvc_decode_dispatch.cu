@@ -6,10 +6,10 @@
 //     bfloat16 the pages run on the tensor cores;
 //   - pair split, 4-warp CTAs (three per SM, tensor-core pages for bfloat16): every
 //     other call whose pairs each get k >= 1 CTAs in one wave (with k = 1 a pair needs no
-//     merge);
+//     merge), unless one slice each would leave many slots empty for long;
 //   - stream-K over (session, KV head, page) units, tensor-core pages for bfloat16:
-//     the rest (more pairs than the 4-warp shape's resident CTAs, e.g. the full-batch
-//     rounds of 64 sessions).
+//     the rest (e.g. rounds of 30-50 long sessions, and calls of more pairs than the
+//     4-warp shape's resident CTAs, like the full-batch rounds of 64 sessions).
 #include <cstring>
 
 #include "kvc_launch.cuh"
@@ -25,17 +25,22 @@ constexpr int DEC_MIN_UNITS = 12;
 // The pair-split kernel takes calls whose pairs each get at least this many CTAs
 // in one wave: with 16-warp CTAs (one per SM) first, else with stream-K's 4-warp
 // CTAs (three per SM).  Only the 16-warp shape uses tagged partial states: with
-// 4-warp CTAs the fenced arrival measured faster.  Against stream-K (CUDA-core
-// pages), the 4-warp tensor-core split measured faster at 20-28 sessions with two
-// slices per pair (56.1 against 60.8 us at 20, 71.1 against 79.0 at 28) and, with one,
-// at 29-57 sessions except near 36 (73.2 against 81.7 at 29, 99.6 against 97.7 at
-// 36, 138.4 against 148.2 at 57).  Against the 16-warp shape, the 4-warp one measured
-// faster from 4 sessions on (15.4 against 16.7 us at 4, 26.4 against 28.1 at 9) and
-// slower below (11.7 against 8.1 at 1).
+// 4-warp CTAs the fenced arrival measured faster.  Against the 16-warp shape, the 4-warp
+// one measured faster from 4 sessions on (15.4 against 16.7 us at 4, 26.4 against 28.1 at
+// 9) and slower below (11.7 against 8.1 at 1).
 constexpr int SPLIT_MIN_K = 5, SPLIT4_MIN_K = 1;
 // Below this many pages the 16-warp shape leaves most of its warps without one
 // (64 pages, 8 pairs: 6.8 us against 6.4-6.7 with 4 warps; 20 pages: 6.7 against 5.2).
 constexpr int WIDE_MIN_PAGES = 100;
+
+// One slice per pair against stream-K, 257 pages, 8 KV heads: 92.9 against 77.5 us at 30
+// sessions (a slice's CTA takes 63 us by itself), 104.7 against 100.7 at 40, 121.4 against
+// 119.7 at 48, but 128.3 against 129.4 at 52 and 137.8 against 139.8 at 57; with 38 pages
+// one slice is faster throughout (14.9 against 18.1 at 30, 17.7 against 20.8 at 40).
+constexpr int STREAM_K_MIN_PAGES = 128;
+bool one_slice_too_few(int slots, int n_pairs, int pages) {
+  return pages >= STREAM_K_MIN_PAGES && n_pairs <= slots * 7 / 8;
+}
 
 // Slices per pair of the 16-warp shape: no more than give each warp a page (257 pages, 8
 // pairs: 7.6 us at 17 slices, 7.9 at 19, 8.9 at 15; 4 pairs: 7.2 at 19, 8.4 at 38).
@@ -63,7 +68,7 @@ int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
 }  // namespace
 
 cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               int pages, bool pdl, cudaStream_t s, uint32_t epoch,
+                               int pages, bool early, cudaStream_t s, uint32_t epoch,
                                const void* new_k, const void* new_v) {
   const int esz = d.esz;
   // Grid sizes of the three shapes, per element type (their CTA shapes differ), worked
@@ -83,7 +88,9 @@ cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out
   const int n_pairs = n_seq * d.kv_heads;
   const int k = n_pairs * SPLIT_MIN_K <= slots && pages >= WIDE_MIN_PAGES
                     ? wide_slices(slots, n_pairs, pages) : 0;
-  const int k4 = k == 0 && n_pairs * SPLIT4_MIN_K <= slots4 ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
+  int k4 = k == 0 && n_pairs * SPLIT4_MIN_K <= slots4
+               ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
+  if (k4 == 1 && one_slice_too_few(slots4, n_pairs, pages)) k4 = 0;
   // Tensor maps of the pool for the tensor-core page loop (bfloat16).
   CUtensorMap map_lo, map_hi;
   memset(&map_lo, 0, sizeof(map_lo));
@@ -96,13 +103,13 @@ cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out
   if (k > 0) {
     const uint32_t tag = n_pairs * k <= d.dec_tag_slots ? epoch : 0u;
     return launch_attn_decode_split(d, true, layer, map_lo, map_hi, q, out, scale, k, tag, new_k,
-                                    new_v, n_pairs, pdl, s);
+                                    new_v, n_pairs, early, s);
   }
   if (k4 > 0)
     return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale, k4, 0u, new_k,
-                                    new_v, n_pairs, pdl, s);
+                                    new_v, n_pairs, early, s);
   return launch_attn_decode_streamk(d, layer, map_lo, map_hi, q, out, scale, grid, DEC_MIN_UNITS,
-                                    new_k, new_v, pdl, s);
+                                    new_k, new_v, early, s);
 }
 
 }  // namespace kvc

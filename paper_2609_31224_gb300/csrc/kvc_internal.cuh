@@ -47,26 +47,16 @@ struct SeqInfo {
   int32_t n_blocks;     // n_hist_pages + n_live_pages
   int32_t pad0;
   int32_t unit_base;    // first (session, kv head, page) unit of this session
-  int32_t pf_chunks;
-  int32_t pf_base;
-  int32_t pad[3];
+  int32_t pad[5];
 };
 static_assert(sizeof(SeqInfo) == 64, "SeqInfo size");
-
-// One split-K work item: blocks [blk_begin, blk_end) of one session.
-struct Item {
-  int32_t seq;
-  int32_t chunk;
-  int32_t blk_begin;
-  int32_t blk_end;
-};
 
 struct DevGlobals {
   int32_t err;
   int32_t n_seq;
   int64_t pages_used;
   int32_t n_units;
-  int32_t n_pf_items;
+  int32_t free_word;  // no page below bitmap word free_word is free
   int32_t n_moves;
   int32_t total_tokens;
   int32_t nb_max;   // largest n_blocks among the last append's sessions
@@ -86,7 +76,7 @@ struct Dev {
   int32_t bitmap_words;
   int32_t max_moves;
   int32_t dec_slots;           // decode partial slots (two per CTA of a split)
-  int32_t max_pf_items;        // prefill chunk items (binary32) / partial slots (bfloat16)
+  int32_t pf_slots;            // prefill partial slots (two per CTA of a split; bfloat16)
   // memory
   uint8_t* pool;
   SessState* sess;
@@ -99,7 +89,6 @@ struct Dev {
   DevGlobals* g;
   float2* rope;                // [max_positions][D/2] (cos, sin)
   SeqInfo* seq;                // [max_seq]
-  Item* pf_items;              // [max_pf_items]
   int32_t* tok_slot;           // [max_tokens] page * PS + slot
   int32_t* tok_pos;            // [max_tokens]
   int2* moves;                 // [max_moves] (src page*PS+slot, dst page*PS+slot)
@@ -109,14 +98,13 @@ struct Dev {
   float2* dec_part_ml;         // [dec_slots][G] (m, l) in log2 units
   unsigned long long* dec_tagged;  // [dec_tag_slots][G * D + 2 G] tagged partial states
   int32_t dec_tag_slots;
-  float* pf_part_o;            // [max_pf_items][PF_ROWS][D]
-  float2* pf_part_ml;          // [max_pf_items][PF_ROWS]
+  float* pf_part_o;            // [pf_slots][D / 4][PF_ROWS][4]
+  float2* pf_part_ml;          // [pf_slots][PF_ROWS]
   int32_t* dec_count;          // [max_seq * kv_heads] arrival counters
   int32_t* pf_count;           // [max_seq * kv_heads]
 };
 
 constexpr int PF_MAX_TOKENS = 32;  // tokens per session per prefill call
-constexpr int MAX_CHUNKS_PER_SEQ = 64;  // split-K chunks per session and call
 
 __host__ __device__ inline size_t pool_offset_elems(const Dev& d, int page, int layer, int kv,
                                                     int head, int slot) {
@@ -345,6 +333,22 @@ __device__ inline void tma_load_2d(void* dst, const CUtensorMap* map, int x, int
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// L2 cache policy for data read once per launch: replaced first, so that what is read again
+// (queries, rotary rows, partial states) stays.
+__device__ inline uint64_t evict_first_policy() {
+  uint64_t p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ inline void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y,
+                                        uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
 

@@ -33,12 +33,15 @@ cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, 
 cudaError_t launch_release(const Dev& d, const SeqArgs& a, cudaStream_t s);
 cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_out, void* k_out,
                               void* v_out, int32_t* count, cudaStream_t s);
+// Attention launches may start while the kernel before them in the stream finishes.  early:
+// they may also read what the append wrote before that (an attention launch of the same
+// append came before, so the append is complete).
 // new_k / new_v (optional): the fused per-layer write of the new tokens' K/V.
 // epoch: tag of this launch's partial states (nonzero, never reused while tags
 // of it may remain in the slots); 0 selects the fenced arrival instead.
 // pages: estimate of the longest session's pages, for the choice of the split only.
 cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               int pages, bool pdl, cudaStream_t s, uint32_t epoch,
+                               int pages, bool early, cudaStream_t s, uint32_t epoch,
                                const void* new_k = nullptr, const void* new_v = nullptr);
 // Stream-K decode kernel (kvc_attn_decode.cu): its grid (resident CTAs, capped by
 // the partial slots) and its launch.
@@ -46,7 +49,7 @@ int decode_stream_k_grid(const Dev& d);
 cudaError_t launch_attn_decode_streamk(const Dev& d, int layer, const CUtensorMap& map_lo,
                                        const CUtensorMap& map_hi, const void* q, void* out,
                                        float scale, int grid, int min_units, const void* new_k,
-                                       const void* new_v, bool pdl, cudaStream_t s);
+                                       const void* new_v, bool early, cudaStream_t s);
 // Pair-split decode kernel (kvc_attn_decode_split.cu).  wide: the 16-warp shape
 // (one CTA per SM; tensor-core pages for bfloat16), else the 4-warp shape.
 int decode_split_slots(int esz, bool wide);          // resident CTAs in one wave
@@ -54,26 +57,26 @@ bool decode_split_uses_tma(int esz, bool wide);      // needs the pool's tensor 
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
                                      float scale, int k, uint32_t epoch, const void* new_k,
-                                     const void* new_v, int n_pairs, bool pdl, cudaStream_t s);
+                                     const void* new_v, int n_pairs, bool early, cudaStream_t s);
 // new_k / new_v (optional, bfloat16 only): the chunk's rows of this layer, written
 // into the pool by the launch itself (the per-layer order).
 // pages_max, pages_sum: estimates of the sessions' resident pages (largest, sum over the
 // call), for the choice of the split only.
 cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                int max_t, int pages_max, int64_t pages_sum, bool pdl,
+                                int max_t, int pages_max, int64_t pages_sum, bool early,
                                 cudaStream_t s, const void* new_k = nullptr,
                                 const void* new_v = nullptr);
 // k = 0: stream-K over `grid` CTAs; k >= 1: pair split, grid = pairs * k CTAs.
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
-                                   int k, int max_t, bool pdl, cudaStream_t s, const void* new_k,
+                                   int k, int max_t, bool early, cudaStream_t s, const void* new_k,
                                    const void* new_v);
 int prefill_tc_max_slices();
 // Clusters of k CTAs of the pair split that fit the current device at once.
 int prefill_tc_max_clusters(int k);
 // binary32; pages_max as in launch_attn_prefill, sms: SMs of the device.
 cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                    int max_t, int pages_max, int sms, bool pdl, cudaStream_t s);
+                                    int max_t, int pages_max, int sms, bool early, cudaStream_t s);
 const void* prefill_tc_kernel_ptr();
 // Two 2-D views of the bfloat16 pool as rows of 128 elements (columns 0-63 and
 // 64-127), 16-row boxes, 128-byte swizzle; cached per pool.  False if the driver

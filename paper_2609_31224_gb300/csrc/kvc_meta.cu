@@ -79,13 +79,15 @@ __device__ int block_max(int v, int* s_warp) {
 
 // Take the k lowest free page ids, mark them used and write them, ascending,
 // to d.alloc_list[0..k).  Returns false (and marks nothing) if fewer than k
-// pages are free.  Block-uniform result.
+// pages are free.  Block-uniform result.  The search starts at the first bitmap word
+// that can hold a free page: an allocation leaves none below its last one, freeing lowers
+// the mark (free_page).
 __device__ bool block_alloc_lowest(const Dev& d, int k, int* s_warp) {
   __shared__ int s_found;
   if (k == 0) return true;
   if (threadIdx.x == 0) s_found = 0;
   __syncthreads();
-  for (int w0 = 0; w0 < d.bitmap_words; w0 += META_THREADS) {
+  for (int w0 = d.g->free_word; w0 < d.bitmap_words; w0 += META_THREADS) {
     const int w = w0 + threadIdx.x;
     uint32_t freebits = 0;
     if (w < d.bitmap_words) {
@@ -114,7 +116,10 @@ __device__ bool block_alloc_lowest(const Dev& d, int k, int* s_warp) {
     __syncthreads();
     if (threadIdx.x == 0) s_found = min(k, found + total);
     __syncthreads();
-    if (s_found >= k) return true;
+    if (s_found >= k) {
+      if (threadIdx.x == 0) d.g->free_word = d.alloc_list[k - 1] >> 5;
+      return true;
+    }
   }
   // Not enough pages: roll back what was marked.
   const int got = s_found;
@@ -124,6 +129,11 @@ __device__ bool block_alloc_lowest(const Dev& d, int k, int* s_warp) {
   }
   __syncthreads();
   return false;
+}
+
+__device__ inline void free_page(const Dev& d, int p) {
+  atomicAnd(&d.bitmap[p >> 5], ~(1u << (p & 31)));
+  atomicMin(&d.g->free_word, p >> 5);
 }
 
 __device__ inline bool evictable_type(int t) { return t == KVC_ACOUSTIC || t == KVC_ASR_DELIM; }
@@ -182,6 +192,7 @@ __global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, Append
   __shared__ int s_total_dec, s_long;
   const int i = threadIdx.x;
   const int n_seq = a.n_seq;
+  pdl_wait();
   pdl_launch_dependents();
   if (i == 0) s_bad = 0;
   __syncthreads();
@@ -363,6 +374,7 @@ __global__ void __launch_bounds__(KV_THREADS) append_kv_kernel(Dev d, int total,
   const int idx = blockIdx.x * KV_THREADS + threadIdx.x;
   const int c = idx % KC, row = idx / KC, g = row / H, h = row % H;
   const bool in = g < total;
+  pdl_launch_dependents();
   uint4 ka, kb, va, vb;
   if (in) {
     const size_t off = (((size_t)blockIdx.y * total + g) * H + h) * D + c * VEC;
@@ -394,23 +406,201 @@ __global__ void __launch_bounds__(KV_THREADS) append_kv_kernel(Dev d, int total,
 }
 
 // ---------------------------------------------------------------------------
-// Append of exactly one token per session (the decode rounds): thread i plans
-// session i of the call (page demand, lowest-free allocation in call order,
-// position, unit, slot tags, state, the attention calls' work split); when k and
-// v are given the CTA then writes the tokens' rotated K and V of every layer.
-// Same state, tags and stored bytes as the general plan kernel followed by
-// append_kv_kernel.
+// Append of exactly one token per session (the decode rounds): the same state and tags as
+// the general plan kernel.  append_few_kernel takes calls of up to 32 sessions, lane i of
+// its first warp planning session i of the call (page demand, lowest-free allocation in
+// call order, position, unit, slot tags, state, the attention calls' work split) with no
+// CTA barrier; a one-session call's other threads write its K and V rows of every layer as
+// soon as the slot is known, their inputs loaded meanwhile.  append_many_kernel takes the
+// larger calls, thread i planning session i.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(META_THREADS) append_single_kernel(Dev d, AppendArgs a,
-                                                                     const uint8_t* types,
-                                                                     const T* k, const T* v) {
+__global__ void __launch_bounds__(META_THREADS) append_few_kernel(Dev d, AppendArgs a,
+                                                                  const uint8_t* types, const T* k,
+                                                                  const T* v) {
+  using CK = Chunk16<T>;
+  constexpr int VEC = CK::N, KC = 8, HALF = KC * VEC, D = 2 * HALF;
+  constexpr int U = 2;  // K/V items (as in append_kv_kernel) in flight per thread
+  __shared__ int s_pages[32];
+  __shared__ int s_gs, s_pos;
+  const int i = threadIdx.x, lane = i & 31;
+  const int n_seq = a.n_seq, H = d.kv_heads;
+  pdl_wait();
+  pdl_launch_dependents();
+  // One session: item idx is chunk idx % 8 of row (layer, head) idx / 8.
+  const int n_items = k != nullptr ? d.layers * H * KC : 0;
+  uint4 ka[U], kb[U], va[U], vb[U];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int idx = base + u * META_THREADS;
+      if (idx < n_items) {
+        const size_t off = (size_t)(idx / KC) * D + (idx % KC) * VEC;
+        ka[u] = __ldcs(reinterpret_cast<const uint4*>(k + off));
+        kb[u] = __ldcs(reinterpret_cast<const uint4*>(k + off + HALF));
+        va[u] = __ldcs(reinterpret_cast<const uint4*>(v + off));
+        vb[u] = __ldcs(reinterpret_cast<const uint4*>(v + off + HALF));
+      }
+    }
+  };
+  load(i);
+  if (i < 32) {
+    const int mpps = d.max_pages_per_session;
+    const bool in = lane < n_seq;
+    int sid = 0, need = 0, ty = 0, page = 0, bad = 0;
+    SessState st = {};
+    if (in) {
+      sid = a.sessions[lane];
+      ty = (int)types[lane];
+      st = d.sess[sid];
+      const int tail = st.live_head + st.n_live;
+      need = (tail + PS) / PS - st.n_live_pages;
+      if (need < 0 || need > 1 || st.n_live_pages + need > mpps) bad |= KVC_DERR_PAGE_TABLE;
+      if (st.pos_next + 1 > d.max_positions) bad |= KVC_DERR_POSITION;
+      if (need == 0) page = d.live_pt[(size_t)sid * mpps + tail / PS];
+    }
+    bad = __reduce_or_sync(FULL, bad);
+    const unsigned needs = __ballot_sync(FULL, need > 0);
+    const int total_need = __popc(needs);
+    if (!bad && total_need > 0) {
+      // The total_need lowest free pages, 32 bitmap words at a time.
+      int found = 0;
+      for (int w0 = d.g->free_word; w0 < d.bitmap_words && found < total_need; w0 += 32) {
+        const int w = w0 + lane;
+        uint32_t freebits = w < d.bitmap_words ? ~d.bitmap[w] : 0u;
+        const int64_t first = (int64_t)w * 32;
+        if (freebits && first + 32 > d.n_pages) {
+          const int valid = (int)(d.n_pages - first);
+          freebits &= valid <= 0 ? 0u : (1u << valid) - 1u;
+        }
+        int base = __popc(freebits);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(FULL, base, o);
+          if (lane >= o) base += y;
+        }
+        const int sum = __shfl_sync(FULL, base, 31);
+        int idx = found + base - __popc(freebits);
+        for (uint32_t fb = freebits; fb && idx < total_need; fb &= fb - 1)
+          s_pages[idx++] = w * 32 + __ffs(fb) - 1;
+        found += sum;
+      }
+      __syncwarp();
+      if (found < total_need || total_need > d.max_alloc) {
+        bad = KVC_DERR_POOL;
+      } else if (lane < total_need) {
+        const int p = s_pages[lane];
+        atomicOr(&d.bitmap[p >> 5], 1u << (p & 31));
+        if (lane == total_need - 1) d.g->free_word = p >> 5;
+      }
+    }
+    if (bad) {
+      if (lane == 0) {
+        set_error(d, bad);
+        abandon_append(d);
+        s_gs = -1;
+      }
+    } else {
+      int nb = 0;
+      SeqInfo si = {};
+      if (in) {
+        const int tail = st.live_head + st.n_live;
+        if (need) {
+          page = s_pages[__popc(needs & lanemask_lt())];
+          d.live_pt[(size_t)sid * mpps + st.n_live_pages] = page;
+        }
+        const int gs = page * PS + tail % PS;
+        const int unit = st.unit_cur + ((ty & KVC_UNIT_BEGIN) ? 1 : 0);
+        if (lane == 0) {
+          s_gs = gs;
+          s_pos = st.pos_next;
+        }
+        d.meta_pos[gs] = st.pos_next;
+        d.meta_unit[gs] = unit;
+        d.meta_type[gs] = (uint8_t)(ty & TYPE_MASK);
+        d.tok_slot[lane] = gs;
+        d.tok_pos[lane] = st.pos_next;
+        SessState s1 = st;
+        s1.pos_next = st.pos_next + 1;
+        s1.unit_cur = unit;
+        s1.n_live = st.n_live + 1;
+        s1.last_chunk = 1;
+        s1.n_live_pages = st.n_live_pages + need;
+        s1.peak_resident = max(st.peak_resident, s1.n_hist + s1.n_live);
+        d.sess[sid] = s1;
+        nb = s1.n_hist_pages + s1.n_live_pages;
+        si.sid = sid;
+        si.t = 1;
+        si.q_row0 = lane;
+        si.pos_first = st.pos_next;
+        si.n_hist = s1.n_hist;
+        si.n_hist_pages = s1.n_hist_pages;
+        si.live_head = s1.live_head;
+        si.n_live = s1.n_live;
+        si.n_blocks = nb;
+      }
+      int units = nb * H;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, units, o);
+        if (lane >= o) units += y;
+      }
+      if (in) {
+        si.unit_base = units - nb * H;
+        d.seq[lane] = si;
+      }
+      const int total_units = __shfl_sync(FULL, units, 31);
+      const int nb_max = __reduce_max_sync(FULL, nb);
+      if (lane == 0) {
+        d.g->n_seq = n_seq;
+        d.g->total_tokens = n_seq;
+        d.g->n_units = total_units;
+        d.g->nb_max = nb_max;
+        d.g->pages_used += total_need;
+      }
+    }
+  }
+  if (n_items == 0) return;
+  __syncthreads();
+  const int gs = s_gs;
+  if (gs < 0) return;
+  T* pool = reinterpret_cast<T*>(d.pool);
+  for (int base = i; base < n_items;) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int idx = base + u * META_THREADS;
+      if (idx >= n_items) break;
+      const int c = idx % KC, h = idx / KC % H, l = idx / KC / H;
+      const float4* t4 = reinterpret_cast<const float4*>(d.rope + (size_t)s_pos * HALF + c * VEC);
+      float xa[VEC], xb[VEC], ya[VEC], yb[VEC];
+      CK::unpack(ka[u], xa);
+      CK::unpack(kb[u], xb);
+#pragma unroll
+      for (int e = 0; e < VEC; e += 2) {
+        const float4 cs = t4[e / 2];
+        rope_pair(xa[e], xb[e], make_float2(cs.x, cs.y), ya[e], yb[e]);
+        rope_pair(xa[e + 1], xb[e + 1], make_float2(cs.z, cs.w), ya[e + 1], yb[e + 1]);
+      }
+      T* dst = pool + pool_offset_elems(d, gs / PS, l, 0, h, gs % PS) + c * VEC;
+      T* dv = dst + (size_t)H * PS * D;
+      *reinterpret_cast<uint4*>(dst) = CK::pack(ya);
+      *reinterpret_cast<uint4*>(dst + HALF) = CK::pack(yb);
+      *reinterpret_cast<uint4*>(dv) = va[u];
+      *reinterpret_cast<uint4*>(dv + HALF) = vb[u];
+    }
+    base += U * META_THREADS;
+    if (base < n_items) load(base);
+  }
+}
+
+__global__ void __launch_bounds__(META_THREADS) append_many_kernel(Dev d, AppendArgs a,
+                                                                   const uint8_t* types) {
   __shared__ int s_warp[33];
   __shared__ int s_bad;
-  __shared__ int s_gs[MAX_SEQ], s_pos[MAX_SEQ];
   const int i = threadIdx.x;
   const int n_seq = a.n_seq;
   const int mpps = d.max_pages_per_session;
+  pdl_wait();
   pdl_launch_dependents();
   if (i == 0) s_bad = 0;
   __syncthreads();
@@ -460,8 +650,6 @@ __global__ void __launch_bounds__(META_THREADS) append_single_kernel(Dev d, Appe
     d.meta_type[gs] = (uint8_t)(ty & TYPE_MASK);
     d.tok_slot[i] = gs;
     d.tok_pos[i] = st.pos_next;
-    s_gs[i] = gs;
-    s_pos[i] = st.pos_next;
     SessState s1 = st;
     s1.pos_next = st.pos_next + 1;
     s1.unit_cur = unit;
@@ -496,75 +684,6 @@ __global__ void __launch_bounds__(META_THREADS) append_single_kernel(Dev d, Appe
     d.g->n_units = total_units;
     d.g->nb_max = nb_max;
     d.g->pages_used += total_need;
-  }
-  if (k == nullptr) return;
-  __syncthreads();
-  // K rotated at the token's position and V, every layer and head: one 16-byte chunk
-  // of the first half of a K row with its rotate-half partner per K item, one 16-byte
-  // chunk of V per V item; K/V input layout [L][n_seq][Hkv][D].  Each thread loads
-  // its items of a pass before it stores any, so their loads are in flight together.
-  using CK = Chunk16<T>;
-  constexpr int VEC = CK::N, UK = sizeof(T) == 2 ? 1 : 2, UV = 4;
-  const int D = d.head_dim, half = D / 2, H = d.kv_heads, L = d.layers;
-  T* pool = reinterpret_cast<T*>(d.pool);
-  const int kc = half / VEC, vc = D / VEC;
-  const int n_k = n_seq * L * H * kc, n_v = n_seq * L * H * vc;
-  for (int base = i; base < n_k; base += UK * META_THREADS) {
-    uint4 wa[UK], wb[UK];
-    float2 cs[UK][VEC];
-    int64_t dst_off[UK];
-#pragma unroll
-    for (int u = 0; u < UK; ++u) {
-      const int idx = base + u * META_THREADS;
-      dst_off[u] = -1;
-      if (idx < n_k) {
-        const int c = idx % kc, r = idx / kc, h = r % H, q = (r / H) % n_seq, l = r / H / n_seq;
-        const T* kin = k + (((size_t)l * n_seq + q) * H + h) * D + c * VEC;
-        wa[u] = *reinterpret_cast<const uint4*>(kin);
-        wb[u] = *reinterpret_cast<const uint4*>(kin + half);
-        const float2* t2 = d.rope + (size_t)s_pos[q] * half + c * VEC;
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) cs[u][e] = t2[e];
-        const int gs = s_gs[q];
-        dst_off[u] = (int64_t)(pool_offset_elems(d, gs / PS, l, 0, h, gs % PS) + c * VEC);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < UK; ++u) {
-      if (dst_off[u] < 0) break;
-      float xa[VEC], xb[VEC], ya[VEC], yb[VEC];
-      CK::unpack(wa[u], xa);
-      CK::unpack(wb[u], xb);
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) {
-        float y1, y2;
-        rope_pair(xa[e], xb[e], cs[u][e], y1, y2);
-        ya[e] = y1;
-        yb[e] = y2;
-      }
-      *reinterpret_cast<uint4*>(pool + dst_off[u]) = CK::pack(ya);
-      *reinterpret_cast<uint4*>(pool + dst_off[u] + half) = CK::pack(yb);
-    }
-  }
-  for (int base = i; base < n_v; base += UV * META_THREADS) {
-    uint4 x[UV];
-    int64_t dst_off[UV];
-#pragma unroll
-    for (int u = 0; u < UV; ++u) {
-      const int idx = base + u * META_THREADS;
-      dst_off[u] = -1;
-      if (idx < n_v) {
-        const int c = idx % vc, r = idx / vc, h = r % H, q = (r / H) % n_seq, l = r / H / n_seq;
-        x[u] = *reinterpret_cast<const uint4*>(v + (((size_t)l * n_seq + q) * H + h) * D + c * VEC);
-        const int gs = s_gs[q];
-        dst_off[u] = (int64_t)(pool_offset_elems(d, gs / PS, l, 1, h, gs % PS) + c * VEC);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < UV; ++u) {
-      if (dst_off[u] < 0) break;
-      *reinterpret_cast<uint4*>(pool + dst_off[u]) = x[u];
-    }
   }
 }
 
@@ -649,6 +768,8 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
   __shared__ int s_bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_seq = a.n_seq;
+  pdl_wait();
+  pdl_launch_dependents();
   if (tid == 0) s_bad = 0;
 
   // Phase 1: plan.  For live slot j with unit u >= 0 the unit-level test is
@@ -801,17 +922,25 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
     const int consumed = st.live_head + end;
     const int nfree = consumed / PS;
     for (int j = lane; j < nfree; j += 32) {
-      const int p = lrow[j];
-      atomicAnd(&d.bitmap[p >> 5], ~(1u << (p & 31)));
+      free_page(d, lrow[j]);
     }
     __syncwarp();
     const int remain = st.n_live_pages - nfree;
     if (nfree > 0) {
-      for (int j0 = 0; j0 < remain; j0 += 32) {
-        const int j = j0 + lane;
-        const int v = (j < remain) ? lrow[j + nfree] : 0;
+      constexpr int U = 8;  // loads in flight per lane
+      for (int j0 = 0; j0 < remain; j0 += 32 * U) {
+        int v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = j0 + 32 * u + lane;
+          v[u] = j < remain ? lrow[j + nfree] : 0;
+        }
         __syncwarp();
-        if (j < remain) lrow[j] = v;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = j0 + 32 * u + lane;
+          if (j < remain) lrow[j] = v[u];
+        }
         __syncwarp();
       }
     }
@@ -838,6 +967,8 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
 // Evict, part 2: move survivors' K/V for every layer, kv slot and head.
 // Work unit: 16 bytes; grid-stride over moves x L x 2 x Hkv x (D*esz/16).
 __global__ void __launch_bounds__(256) evict_copy_kernel(Dev d) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int n_moves = d.g->n_moves;
   const int vec_per_row = d.head_dim * d.esz / 16;
   const int rows_per_move = d.layers * 2 * d.kv_heads;
@@ -940,14 +1071,8 @@ __global__ void __launch_bounds__(META_THREADS) release_kernel(Dev d, SeqArgs a)
     const SessState st = d.sess[sid];
     const int32_t* hrow = d.hist_pt + (size_t)sid * d.max_pages_per_session;
     const int32_t* lrow = d.live_pt + (size_t)sid * d.max_pages_per_session;
-    for (int j = lane; j < st.n_hist_pages; j += 32) {
-      const int p = hrow[j];
-      atomicAnd(&d.bitmap[p >> 5], ~(1u << (p & 31)));
-    }
-    for (int j = lane; j < st.n_live_pages; j += 32) {
-      const int p = lrow[j];
-      atomicAnd(&d.bitmap[p >> 5], ~(1u << (p & 31)));
-    }
+    for (int j = lane; j < st.n_hist_pages; j += 32) free_page(d, hrow[j]);
+    for (int j = lane; j < st.n_live_pages; j += 32) free_page(d, lrow[j]);
     __syncwarp();
     if (lane == 0) {
       SessState s = {};
@@ -969,26 +1094,32 @@ cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Every kernel below may start while the one before it in the stream finishes (it waits for
+// that one before it reads anything but the caller's inputs), so that a chain of short
+// kernels does not pay a full launch each.
 cudaError_t launch_append(const Dev& d, const AppendArgs& a, const uint8_t* types, const void* k,
                           const void* v, bool single, cudaStream_t s) {
-  if (single) {
+  cudaError_t e;
+  if (single && a.n_seq <= 32) {
     // One CTA writes the K/V rows only for a one-session call (a few hundred KiB at
-    // most); larger calls keep the plan in one CTA and spread the rows over
-    // append_kv_kernel's grid.
-    const bool fuse_kv = a.n_seq == 1;
+    // most); larger calls spread the rows over append_kv_kernel's grid.
+    const bool fuse_kv = a.n_seq == 1 && k != nullptr;
+    const dim3 block(fuse_kv ? META_THREADS : 32);
     if (d.esz == 2)
-      append_single_kernel<__nv_bfloat16><<<1, META_THREADS, 0, s>>>(
-          d, a, types, static_cast<const __nv_bfloat16*>(fuse_kv ? k : nullptr),
-          static_cast<const __nv_bfloat16*>(fuse_kv ? v : nullptr));
+      e = launch_ex(&append_few_kernel<__nv_bfloat16>, dim3(1), block, 0, s, true, d, a, types,
+                    static_cast<const __nv_bfloat16*>(fuse_kv ? k : nullptr),
+                    static_cast<const __nv_bfloat16*>(fuse_kv ? v : nullptr));
     else
-      append_single_kernel<float><<<1, META_THREADS, 0, s>>>(
-          d, a, types, static_cast<const float*>(fuse_kv ? k : nullptr),
-          static_cast<const float*>(fuse_kv ? v : nullptr));
-    if (fuse_kv || k == nullptr) return cudaGetLastError();
-    return launch_append_layers(d, a.total, 0, d.layers, k, v, true, s);
+      e = launch_ex(&append_few_kernel<float>, dim3(1), block, 0, s, true, d, a, types,
+                    static_cast<const float*>(fuse_kv ? k : nullptr),
+                    static_cast<const float*>(fuse_kv ? v : nullptr));
+    if (fuse_kv) return e;
+  } else if (single) {
+    e = launch_ex(&append_many_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a, types);
+  } else {
+    e = launch_ex(&append_plan_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a, types);
   }
-  append_plan_kernel<<<1, META_THREADS, 0, s>>>(d, a, types);
-  if (k == nullptr) return cudaGetLastError();  // plan only: layers follow one by one
+  if (e != cudaSuccess || k == nullptr) return e;  // plan only: layers follow one by one
   return launch_append_layers(d, a.total, 0, d.layers, k, v, true, s);
 }
 
@@ -1006,12 +1137,13 @@ cudaError_t launch_append_layers(const Dev& d, int total, int layer0, int n_laye
 }
 
 cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, cudaStream_t s) {
-  evict_plan_kernel<<<1, META_THREADS, 0, s>>>(d, a, resident_out);
+  const cudaError_t e = launch_ex(&evict_plan_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a,
+                                  resident_out);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  evict_copy_kernel<<<sms * 4, 256, 0, s>>>(d);
-  return cudaGetLastError();
+  return launch_ex(&evict_copy_kernel, dim3(sms * 4), dim3(256), 0, s, true, d);
 }
 
 cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_out, void* k_out,

@@ -19,22 +19,6 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float RESCALE_LOG2 = 8.f;          // rescale O only when the max grows by > 2^8
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// L2 cache policy for data read once per launch: replaced first, so that what is read again
-// (queries, rotary rows, partial states) stays.
-__device__ inline uint64_t evict_first_policy() {
-  uint64_t p;
-  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ inline void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y,
-                                        uint64_t* bar, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy)
-      : "memory");
-}
-
 // -- tcgen05 helpers ------------------------------------------------------------------
 __device__ inline void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
