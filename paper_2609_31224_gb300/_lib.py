@@ -77,16 +77,17 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
                                vp, ctypes.c_size_t, vp]
     lib.kvc_destroy.argtypes = [vp]
     lib.kvc_destroy.restype = None
-    lib.kvc_append_chunk.argtypes = [vp, ctypes.c_int, p_i32, p_i32, vp, vp, vp, vp]
+    # (Host int32 lists as addresses: an int, or a pointer from host_i32().)
+    lib.kvc_append_chunk.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp, vp]
     lib.kvc_append_kv_layer.argtypes = [vp, ctypes.c_int, vp, vp, vp]
-    lib.kvc_evict.argtypes = [vp, ctypes.c_int, p_i32, vp, vp]
+    lib.kvc_evict.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_attn_prefill_chunk.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_attn_decode.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_attn_decode_kv.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp]
     lib.kvc_attn_prefill_chunk_kv.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp]
     lib.kvc_attn_decode_noalloc.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_resident_size.argtypes = [vp, ctypes.c_int, ctypes.POINTER(i64)]
-    lib.kvc_release.argtypes = [vp, ctypes.c_int, p_i32, vp]
+    lib.kvc_release.argtypes = [vp, ctypes.c_int, vp, vp]
     lib.kvc_export_state.argtypes = [vp, ctypes.c_int, ctypes.POINTER(SessionInfo), p_i32, p_i32,
                                      p_i32, ctypes.POINTER(ctypes.c_uint8), p_i32, i64]
     lib.kvc_export_kv.argtypes = [vp, ctypes.c_int, ctypes.c_int, vp, vp, i64]
@@ -106,6 +107,8 @@ def _check(rc: int) -> None:
 
 
 def _i32(a) -> np.ndarray:
+    if type(a) is np.ndarray and a.dtype == np.int32 and a.flags.c_contiguous:
+        return a
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
 
@@ -120,12 +123,11 @@ def host_i32(a):
 
 
 def _stream(stream):
-    import torch
+    """cudaStream_t of a stream argument, as an int (the current stream for None)."""
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        import torch
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def query_sizes(cfg: Config) -> tuple[int, int]:
@@ -205,7 +207,7 @@ class KVCache:
     # -- hot path -------------------------------------------------------------------
     def append_chunk(self, sessions, cu_tokens, types, k, v, stream=None) -> None:
         s, cu = _i32(sessions), _i32(cu_tokens)
-        _check(self.lib.kvc_append_chunk(self.ctx, len(s), _ptr_i32(s), _ptr_i32(cu),
+        _check(self.lib.kvc_append_chunk(self.ctx, len(s), s.ctypes.data, cu.ctypes.data,
                                          types.data_ptr(), None if k is None else k.data_ptr(),
                                          None if v is None else v.data_ptr(), _stream(stream)))
 
@@ -221,7 +223,7 @@ class KVCache:
 
     def evict(self, sessions, resident_out=None, stream=None) -> None:
         s = _i32(sessions)
-        _check(self.lib.kvc_evict(self.ctx, len(s), _ptr_i32(s),
+        _check(self.lib.kvc_evict(self.ctx, len(s), s.ctypes.data,
                                   None if resident_out is None else resident_out.data_ptr(),
                                   _stream(stream)))
 
@@ -235,7 +237,7 @@ class KVCache:
 
     def release(self, sessions, stream=None) -> None:
         s = _i32(sessions)
-        _check(self.lib.kvc_release(self.ctx, len(s), _ptr_i32(s), _stream(stream)))
+        _check(self.lib.kvc_release(self.ctx, len(s), s.ctypes.data, _stream(stream)))
 
     # -- synchronising queries -------------------------------------------------------
     def resident_size(self, session: int) -> int:

@@ -163,7 +163,8 @@ struct kvc_ctx {
   int64_t delta_since_readback = 0;
   bool readback_pending = false;
   cudaEvent_t ev = nullptr;
-  int64_t* h_readback = nullptr;  // pinned
+  int64_t* h_readback = nullptr;  // pinned, written by evict and release
+  int sms = 0;
   // Last append (queries of the following attention calls).
   bool attn_valid = false;
   int last_n_seq = 0, last_total = 0, last_max_t = 0;
@@ -218,9 +219,9 @@ cudaError_t next_decode_epoch(kvc_ctx* ctx, cudaStream_t s, uint32_t* epoch) {
   return cudaSuccess;
 }
 
+// The launch just enqueued writes the pages in use to h_readback itself: a copy in the stream
+// would cost 6 us of submission and keep the next append from starting early.
 void enqueue_readback(kvc_ctx* ctx, cudaStream_t s) {
-  cudaMemcpyAsync(ctx->h_readback, &ctx->d.g->pages_used, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                  s);
   cudaEventRecord(ctx->ev, s);
   ctx->readback_pending = true;
   ctx->delta_since_readback = 0;
@@ -306,13 +307,21 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
       launch_init(d, cfg->rope_base, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return cleanup(fail(KVC_ECUDA, "initialisation failed: %s",
                         cudaGetErrorString(cudaGetLastError())));
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return cleanup(fail(KVC_ECUDA, "device query failed"));
   *out = ctx;
   return KVC_OK;
 }
 
 void kvc_destroy(kvc_ctx* ctx) {
   if (!ctx) return;
-  if (ctx->ev) cudaEventDestroy(ctx->ev);
+  // The last evict or release may still have to write h_readback.
+  if (ctx->ev) {
+    cudaEventSynchronize(ctx->ev);
+    cudaEventDestroy(ctx->ev);
+  }
   if (ctx->h_readback) cudaFreeHost(ctx->h_readback);
   delete ctx;
 }
@@ -419,7 +428,7 @@ int kvc_evict(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, int64_t* d_res
   a.n_seq = n_seq;
   for (int i = 0; i < n_seq; ++i) a.sessions[i] = h_sessions[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, s));
+  KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, ctx->h_readback, ctx->sms, s));
   ctx->used_ub += n_seq;  // an evict adds at most one page per session, net
   enqueue_readback(ctx, s);
   ctx->attn_valid = false;
@@ -435,7 +444,7 @@ int kvc_release(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, void* stream
   a.n_seq = n_seq;
   for (int i = 0; i < n_seq; ++i) a.sessions[i] = h_sessions[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  KVC_CUDA(launch_release(ctx->d, a, s));
+  KVC_CUDA(launch_release(ctx->d, a, ctx->h_readback, s));
   for (int i = 0; i < n_seq; ++i) {
     ctx->tail_mod[h_sessions[i]] = 0;
     ctx->pos_next[h_sessions[i]] = 0;

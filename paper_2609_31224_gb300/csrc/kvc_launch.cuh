@@ -9,17 +9,24 @@ namespace kvc {
 // ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files).
 // ---------------------------------------------------------------------------
-struct AppendArgs {
+// Session lists of a call, by value.  Calls of up to FEW sessions pass the small block: the
+// driver copies a launch's arguments, and 4 KB of them cost more than the rest of a launch.
+constexpr int FEW = 32;
+template <int N>
+struct AppendArgsT {
   int32_t n_seq;
   int32_t total;
-  int32_t sessions[MAX_SEQ];
-  int32_t cu[MAX_SEQ + 1];
+  int32_t sessions[N];
+  int32_t cu[N + 1];
 };
+using AppendArgs = AppendArgsT<MAX_SEQ>;
 
-struct SeqArgs {
+template <int N>
+struct SeqArgsT {
   int32_t n_seq;
-  int32_t sessions[MAX_SEQ];
+  int32_t sessions[N];
 };
+using SeqArgs = SeqArgsT<MAX_SEQ>;
 
 cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s);
 // single: every session of the call gets exactly one token (plan and K/V write in
@@ -29,8 +36,9 @@ cudaError_t launch_append(const Dev& d, const AppendArgs& a, const uint8_t* type
 // after_plan: launched right behind the plan kernel of the same append.
 cudaError_t launch_append_layers(const Dev& d, int total, int layer0, int n_layers, const void* k,
                                  const void* v, bool after_plan, cudaStream_t s);
-cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, cudaStream_t s);
-cudaError_t launch_release(const Dev& d, const SeqArgs& a, cudaStream_t s);
+cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, int64_t* used_out,
+                         int sms, cudaStream_t s);
+cudaError_t launch_release(const Dev& d, const SeqArgs& a, int64_t* used_out, cudaStream_t s);
 cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_out, void* k_out,
                               void* v_out, int32_t* count, cudaStream_t s);
 // Attention launches may start while the kernel before them in the stream finishes.  early:

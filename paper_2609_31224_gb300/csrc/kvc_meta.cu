@@ -185,7 +185,8 @@ __device__ void abandon_append(const Dev& d) {
   d.g->n_units = 0;
 }
 
-__global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, AppendArgs a,
+template <int N>
+__global__ void __launch_bounds__(META_THREADS) append_plan_kernel(Dev d, AppendArgsT<N> a,
                                                                    const uint8_t* types) {
   __shared__ int s_warp[33];
   __shared__ int s_bad;
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(KV_THREADS) append_kv_kernel(Dev d, int total,
 // larger calls, thread i planning session i.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(META_THREADS) append_few_kernel(Dev d, AppendArgs a,
+__global__ void __launch_bounds__(META_THREADS) append_few_kernel(Dev d, SeqArgsT<FEW> a,
                                                                   const uint8_t* types, const T* k,
                                                                   const T* v) {
   using CK = Chunk16<T>;
@@ -760,8 +761,10 @@ __device__ int sink_recent_end(const Dev& d, const SessState& st, const int32_t*
   return end;
 }
 
-__global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs a,
-                                                                  int64_t* resident_out) {
+template <int N>
+__global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgsT<N> a,
+                                                                  int64_t* resident_out,
+                                                                  int64_t* used_out) {
   __shared__ int s_warp[33];
   __shared__ int s_end[MAX_SEQ], s_surv[MAX_SEQ], s_nev[MAX_SEQ];
   __shared__ int s_hneed[MAX_SEQ], s_hoff[MAX_SEQ], s_moff[MAX_SEQ];
@@ -875,6 +878,7 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
     if (tid == 0) {
       set_error(d, s_bad);
       d.g->n_moves = 0;
+      *used_out = d.g->pages_used;
     }
     return;
   }
@@ -882,6 +886,7 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
     if (tid == 0) {
       set_error(d, KVC_DERR_POOL);
       d.g->n_moves = 0;
+      *used_out = d.g->pages_used;
     }
     return;
   }
@@ -960,7 +965,7 @@ __global__ void __launch_bounds__(META_THREADS) evict_plan_kernel(Dev d, SeqArgs
   __syncthreads();
   if (tid == 0) {
     d.g->n_moves = total_moves;
-    d.g->pages_used += total_h - s_freed;
+    *used_out = d.g->pages_used += total_h - s_freed;
   }
 }
 
@@ -1061,7 +1066,8 @@ __global__ void __launch_bounds__(256) transcript_copy_kernel(Dev d, int cap, ui
 }
 
 // Release (one CTA): free every page of the listed sessions and reset them.
-__global__ void __launch_bounds__(META_THREADS) release_kernel(Dev d, SeqArgs a) {
+__global__ void __launch_bounds__(META_THREADS) release_kernel(Dev d, SeqArgs a,
+                                                               int64_t* used_out) {
   __shared__ int s_freed;
   if (threadIdx.x == 0) s_freed = 0;
   __syncthreads();
@@ -1082,7 +1088,7 @@ __global__ void __launch_bounds__(META_THREADS) release_kernel(Dev d, SeqArgs a)
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) d.g->pages_used -= s_freed;
+  if (threadIdx.x == 0) *used_out = d.g->pages_used -= s_freed;
 }
 
 }  // namespace
@@ -1100,24 +1106,34 @@ cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s) {
 cudaError_t launch_append(const Dev& d, const AppendArgs& a, const uint8_t* types, const void* k,
                           const void* v, bool single, cudaStream_t s) {
   cudaError_t e;
-  if (single && a.n_seq <= 32) {
+  if (single && a.n_seq <= FEW) {
     // One CTA writes the K/V rows only for a one-session call (a few hundred KiB at
     // most); larger calls spread the rows over append_kv_kernel's grid.
     const bool fuse_kv = a.n_seq == 1 && k != nullptr;
     const dim3 block(fuse_kv ? META_THREADS : 32);
+    SeqArgsT<FEW> few;
+    few.n_seq = a.n_seq;
+    for (int i = 0; i < a.n_seq; ++i) few.sessions[i] = a.sessions[i];
     if (d.esz == 2)
-      e = launch_ex(&append_few_kernel<__nv_bfloat16>, dim3(1), block, 0, s, true, d, a, types,
+      e = launch_ex(&append_few_kernel<__nv_bfloat16>, dim3(1), block, 0, s, true, d, few, types,
                     static_cast<const __nv_bfloat16*>(fuse_kv ? k : nullptr),
                     static_cast<const __nv_bfloat16*>(fuse_kv ? v : nullptr));
     else
-      e = launch_ex(&append_few_kernel<float>, dim3(1), block, 0, s, true, d, a, types,
+      e = launch_ex(&append_few_kernel<float>, dim3(1), block, 0, s, true, d, few, types,
                     static_cast<const float*>(fuse_kv ? k : nullptr),
                     static_cast<const float*>(fuse_kv ? v : nullptr));
     if (fuse_kv) return e;
   } else if (single) {
     e = launch_ex(&append_many_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a, types);
+  } else if (a.n_seq <= FEW) {
+    AppendArgsT<FEW> few;
+    few.n_seq = a.n_seq;
+    few.total = a.total;
+    for (int i = 0; i < a.n_seq; ++i) few.sessions[i] = a.sessions[i];
+    for (int i = 0; i <= a.n_seq; ++i) few.cu[i] = a.cu[i];
+    e = launch_ex(&append_plan_kernel<FEW>, dim3(1), dim3(META_THREADS), 0, s, true, d, few, types);
   } else {
-    e = launch_ex(&append_plan_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a, types);
+    e = launch_ex(&append_plan_kernel<MAX_SEQ>, dim3(1), dim3(META_THREADS), 0, s, true, d, a, types);
   }
   if (e != cudaSuccess || k == nullptr) return e;  // plan only: layers follow one by one
   return launch_append_layers(d, a.total, 0, d.layers, k, v, true, s);
@@ -1136,13 +1152,21 @@ cudaError_t launch_append_layers(const Dev& d, int total, int layer0, int n_laye
                    layer0, static_cast<const float*>(k), static_cast<const float*>(v));
 }
 
-cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, cudaStream_t s) {
-  const cudaError_t e = launch_ex(&evict_plan_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d, a,
-                                  resident_out);
+// used_out: the pages in use afterwards are written there (pinned host memory).
+cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, int64_t* used_out,
+                         int sms, cudaStream_t s) {
+  cudaError_t e;
+  if (a.n_seq <= FEW) {
+    SeqArgsT<FEW> few;
+    few.n_seq = a.n_seq;
+    for (int i = 0; i < a.n_seq; ++i) few.sessions[i] = a.sessions[i];
+    e = launch_ex(&evict_plan_kernel<FEW>, dim3(1), dim3(META_THREADS), 0, s, true, d, few,
+                  resident_out, used_out);
+  } else {
+    e = launch_ex(&evict_plan_kernel<MAX_SEQ>, dim3(1), dim3(META_THREADS), 0, s, true, d, a,
+                  resident_out, used_out);
+  }
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return launch_ex(&evict_copy_kernel, dim3(sms * 4), dim3(256), 0, s, true, d);
 }
 
@@ -1157,8 +1181,8 @@ cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_o
   return cudaGetLastError();
 }
 
-cudaError_t launch_release(const Dev& d, const SeqArgs& a, cudaStream_t s) {
-  release_kernel<<<1, META_THREADS, 0, s>>>(d, a);
+cudaError_t launch_release(const Dev& d, const SeqArgs& a, int64_t* used_out, cudaStream_t s) {
+  release_kernel<<<1, META_THREADS, 0, s>>>(d, a, used_out);
   return cudaGetLastError();
 }
 
