@@ -32,8 +32,9 @@
 // a stage's boxes issued by one lane and a thread per row for q, partial states and outputs
 // took 193); below that, a stage of a lone CTA takes 0.6 us, the issue of S = Q K^T (10
 // instructions of about 70 cycles; one softmax group: 0.8 us), and a launch about 7 us beside
-// its stages (1 session: 48.1 -> 12.7 us, most of it the merge of 16 parts by one CTA;
-// 9 sessions: 48.6 -> 31 us).  Under load every access that misses L2 waits behind the K/V
+// its stages (1 session: 48.1 -> 12.5 us, most of it the merge of 16 parts by one CTA;
+// 9 sessions: 48.6 -> 30.1 us; merging the parts that exist instead of 8, own rows in
+// place, took the last 2-3 %).  Under load every access that misses L2 waits behind the K/V
 // bytes in flight (about 4 us with a full ring on every SM).  So the queries and rotary rows
 // of the next segment are copied while the current one runs, K and V carry an evict-first
 // hint that keeps them, the rotary table and the partial states in L2, and in the stream-K
@@ -258,6 +259,44 @@ __device__ inline void merge_parts(const Dev& d, const UnitSplit& us, const PSeg
   }
 }
 
+// Merge of this CTA's n_rows rows from the k <= K parts of the cluster, a 4-element chunk per
+// thread and pass: part p's rows in slot p of the received ones (`per` rows apart), this
+// CTA's own (p = slice) where it left them.
+template <int K, typename RowFn>
+__device__ inline void merge_rows(const uint8_t* recv, const uint8_t* own, int slice, int k,
+                                  int per, int n_rows, int tid, RowFn out_row) {
+  for (int i = tid; i < n_rows * (D / 4); i += THREADS) {
+    const int rl = i / (D / 4), c = i % (D / 4);
+    float2 ml[K];
+    float4 o[K];
+#pragma unroll
+    for (int p = 0; p < K; ++p) {
+      const int pp = min(p, k - 1);
+      const uint8_t* pr = (pp == slice ? own : recv + pp * per * ROW_PITCH) + rl * ROW_PITCH;
+      ml[p] = p < k ? *reinterpret_cast<const float2*>(pr + D * 4) : make_float2(-INFINITY, 0.f);
+      o[p] = *reinterpret_cast<const float4*>(pr + c * 16);
+    }
+    float mx = -INFINITY;
+#pragma unroll
+    for (int p = 0; p < K; ++p) mx = fmaxf(mx, ml[p].x);
+    float L = 0.f;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < K; ++p) {
+      if (ml[p].x == -INFINITY) continue;  // a part without a key of this row
+      const float w = exp2f(ml[p].x - mx);
+      L += ml[p].y * w;
+      a.x = fmaf(o[p].x, w, a.x);
+      a.y = fmaf(o[p].y, w, a.y);
+      a.z = fmaf(o[p].z, w, a.z);
+      a.w = fmaf(o[p].w, w, a.w);
+    }
+    const float inv = 1.f / L;
+    *reinterpret_cast<uint2*>(out_row(rl) + c * 4) =
+        make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
+  }
+}
+
 // FUSED (the per-layer order): the chunk's K (rotated at each token's position) and
 // V of this layer are not in the pool yet; new_k / new_v hold them ([total][Hkv][D],
 // the append's token order).  The softmax warps write the rows of a segment's chunk
@@ -334,10 +373,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
   };
   if (CLUSTER && k_slices > 1) {
     // Rows [rank R / k, (rank + 1) R / k) of the pair are CTA rank's to merge and write: it
-    // receives k parts of each.  Arrival: this CTA has started and its barrier expects them.
+    // receives the other k - 1 parts of each.  Arrival: this CTA has started and its barrier expects them.
     if (tid == 0) {
       const int R = d.seq[seg.seq].t * G, k = k_slices, slice = cta % k;
-      mbar_arrive_expect_tx(&bars[B_RECV], k * ((slice + 1) * R / k - slice * R / k) * ROW_PITCH);
+      mbar_arrive_expect_tx(&bars[B_RECV], (k - 1) * ((slice + 1) * R / k - slice * R / k) * ROW_PITCH);
     }
     __syncwarp();
     cluster_arrive();
@@ -526,8 +565,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
           ok = mbar_wait(d, &bars[B_Q], segs & 1);
           for (int k = 0; k < n_st && ok; ++k, ++n) {
             const int g = n & 1;
-            ok = mbar_wait(d, &bars[B_K_FULL + st], pass & 1) &&
-                 mbar_wait(d, &bars[B_S_EMPTY + g], ((n >> 1) & 1) ^ 1);
+            ok = mbar_wait2(d, &bars[B_K_FULL + st], pass & 1, &bars[B_S_EMPTY + g],
+                            ((n >> 1) & 1) ^ 1);
             if (!ok) break;
             tc_fence_after();
             const uint64_t kdesc = smem_desc(sKV + st * STAGE, 0, 1024);
@@ -553,8 +592,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
           const int n_st = seg.n_st();
           for (int k = 0; k < n_st && ok; ++k, ++n) {
             const int g = n & 1;
-            ok = mbar_wait(d, &bars[B_V_FULL + st], pass & 1) &&
-                 mbar_wait(d, &bars[B_P_FULL + g], (n >> 1) & 1);
+            ok = mbar_wait2(d, &bars[B_V_FULL + st], pass & 1, &bars[B_P_FULL + g], (n >> 1) & 1);
             if (!ok) break;
             tc_fence_after();
             const uint64_t vdesc = smem_desc(sKV + st * STAGE + 2 * KV_PANEL, KV_PANEL, 1024);
@@ -977,7 +1015,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     const int R = si.t * G, per = (R + k - 1) / k;
     const int r0 = slice * R / k, n_rows = (slice + 1) * R / k - r0;
     const uint32_t s_recv = smem_u32(smem + off_out(ring, max_t));
-    // Every part goes to slot `slice` of the owner's received rows.
+    // Every part of another CTA's rows goes to slot `slice` of its received rows.
     for (int i = tid; u_begin == u_end && i < R; i += THREADS)  // no page: weighs nothing
       *reinterpret_cast<float2*>(smem + OFF_KV + i * ROW_PITCH + D * 4) = make_float2(-INFINITY, 0.f);
     fence_proxy_async_smem();
@@ -985,7 +1023,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     cluster_wait();  // every CTA of the cluster has started
     if (tid < k) {
       const int f = tid * R / k, nf = (tid + 1) * R / k - f;
-      if (nf > 0)
+      if (nf > 0 && tid != slice)
         bulk_s2cluster(cluster_map(s_recv + slice * per * ROW_PITCH, tid), sKV + f * ROW_PITCH,
                        nf * ROW_PITCH, cluster_map(smem_u32(&bars[B_RECV]), tid));
     }
@@ -994,39 +1032,20 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     const bool got = mbar_wait(d, &bars[B_RECV], 0);
     __syncwarp();
     cluster_arrive();
-    // Merge and write this CTA's rows, a 4-element chunk per thread and pass.
+    // Merge and write this CTA's rows.
     const uint8_t* rows = smem + off_out(ring, max_t);
-    for (int i = tid; i < n_rows * (D / 4) && got; i += THREADS) {
-      const int rl = i / (D / 4), c = i % (D / 4), row = r0 + rl;
-      const uint8_t* p0 = rows + rl * ROW_PITCH;
-      float2 ml[MAX_K];
-      float4 o[MAX_K];
-#pragma unroll
-      for (int p = 0; p < MAX_K; ++p) {
-        const uint8_t* pr = p0 + min(p, k - 1) * per * ROW_PITCH;
-        ml[p] = p < k ? *reinterpret_cast<const float2*>(pr + D * 4) : make_float2(-INFINITY, 0.f);
-        o[p] = *reinterpret_cast<const float4*>(pr + c * 16);
-      }
-      float mx = -INFINITY;
-#pragma unroll
-      for (int p = 0; p < MAX_K; ++p) mx = fmaxf(mx, ml[p].x);
-      float Ls = 0.f;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int p = 0; p < MAX_K; ++p) {
-        if (ml[p].x == -INFINITY) continue;  // a part without a key of this row
-        const float w = exp2f(ml[p].x - mx);
-        Ls += ml[p].y * w;
-        a.x = fmaf(o[p].x, w, a.x);
-        a.y = fmaf(o[p].y, w, a.y);
-        a.z = fmaf(o[p].z, w, a.z);
-        a.w = fmaf(o[p].w, w, a.w);
-      }
-      const float inv = 1.f / Ls;
-      __nv_bfloat16* orow = out + ((size_t)(si.q_row0 + row / G) * d.q_heads + seg.head * G +
-                                   row % G) * D + c * 4;
-      *reinterpret_cast<uint2*>(orow) =
-          make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
+    const uint8_t* own = smem + OFF_KV + r0 * ROW_PITCH;
+    auto out_row = [&](int rl) {
+      const int row = r0 + rl;
+      return out + ((size_t)(si.q_row0 + row / G) * d.q_heads + seg.head * G + row % G) * D;
+    };
+    if (got) {
+      if (k <= 2)
+        merge_rows<2>(rows, own, slice, k, per, n_rows, tid, out_row);
+      else if (k <= 4)
+        merge_rows<4>(rows, own, slice, k, per, n_rows, tid, out_row);
+      else
+        merge_rows<MAX_K>(rows, own, slice, k, per, n_rows, tid, out_row);
     }
     __syncwarp();
     cluster_wait();  // every part was received: no copy still reads this CTA's rows

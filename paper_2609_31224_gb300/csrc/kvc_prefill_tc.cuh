@@ -19,6 +19,24 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float RESCALE_LOG2 = 8.f;          // rescale O only when the max grows by > 2^8
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
+// Bounded wait for two barriers: both are tested first, back to back, so that their latencies
+// overlap when both are ready.
+__device__ inline bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ inline bool mbar_wait2(const Dev& d, uint64_t* a, uint32_t pa, uint64_t* b, uint32_t pb) {
+  const bool ra = mbar_test(a, pa), rb = mbar_test(b, pb);
+  return (ra || mbar_wait(d, a, pa)) && (rb || mbar_wait(d, b, pb));
+}
+
 // -- tcgen05 helpers ------------------------------------------------------------------
 __device__ inline void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
