@@ -10,8 +10,9 @@
 // maximum takes four shuffles and P needs no CTA barrier.
 // The k slices of a pair are a thread-block cluster: each CTA leaves its partial rows
 // (O, max, sum) in shared memory and merges its share of them from all k.
-// Measured per launch with 17-token chunks: 4 sessions x 8 heads x 1,040 positions 27.3 us
-// (0.29 GFMA; 7.5 us at the FMA peak), one session x 1 head x 520 positions 9.7 us; before,
+// Measured per launch with 17-token chunks: 4 sessions x 8 heads x 1,040 positions 26.5 us
+// (0.29 GFMA; 7.5 us at the FMA peak: with two warps per scheduler the FMA pipe is busy half
+// of the time), one session x 1 head x 520 positions 9.7 us; before,
 // with a thread per row and chunks merged through global memory by one CTA, 96.7 and 55 us.
 #include <type_traits>
 
@@ -190,21 +191,26 @@ __global__ void __launch_bounds__(THREADS, 2) attn_prefill_f32_kernel(
     for (int i = 0; i < RT; ++i)
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[i][c] = make_float2(0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < D; j += 4) {
       float4 kv[NC];
 #pragma unroll
       for (int c = 0; c < NC; ++c)
         kv[c] = *reinterpret_cast<const float4*>(kt + (tx + 16 * c) * PITCH + j);
+      // Rows innermost, so that an accumulator's updates lie RT NC instructions apart.
+      float4 x[RT];
 #pragma unroll
-      for (int i = 0; i < RT; ++i) {
-        const float4 x = *reinterpret_cast<const float4*>(s_q + i * PITCH + j);
+      for (int i = 0; i < RT; ++i) x[i] = *reinterpret_cast<const float4*>(s_q + i * PITCH + j);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          acc[i][c] = __ffma2_rn(make_float2(x.x, x.y), make_float2(kv[c].x, kv[c].y), acc[i][c]);
-          acc[i][c] = __ffma2_rn(make_float2(x.z, x.w), make_float2(kv[c].z, kv[c].w), acc[i][c]);
-        }
-      }
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+          acc[i][c] = __ffma2_rn(make_float2(x[i].x, x[i].y), make_float2(kv[c].x, kv[c].y), acc[i][c]);
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+          acc[i][c] = __ffma2_rn(make_float2(x[i].z, x[i].w), make_float2(kv[c].z, kv[c].w), acc[i][c]);
     }
     // Key tx of page c: resident slot, and its logical index for the causal limit.
     float al[RT];
@@ -241,33 +247,34 @@ __global__ void __launch_bounds__(THREADS, 2) attn_prefill_f32_kernel(
     }
     __syncwarp();
     // The tile's P V by itself first: one long chain over all keys would round more.
-    float4 ot[RT];
+    float2 ot[RT][2];
 #pragma unroll
-    for (int i = 0; i < RT; ++i) ot[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
+    for (int i = 0; i < RT; ++i) ot[i][0] = ot[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
     for (int j = 0; j < 16 * NC; j += 4) {
       float4 v[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) v[c] = *reinterpret_cast<const float4*>(vt + (j + c) * PITCH + tx * 4);
+      float4 p[RT];
 #pragma unroll
-      for (int i = 0; i < RT; ++i) {
-        const float4 p = *reinterpret_cast<const float4*>(s_p + i * PITCH + j);
-        const float pc[4] = {p.x, p.y, p.z, p.w};
+      for (int i = 0; i < RT; ++i) p[i] = *reinterpret_cast<const float4*>(s_p + i * PITCH + j);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          ot[i].x = fmaf(pc[c], v[c].x, ot[i].x);
-          ot[i].y = fmaf(pc[c], v[c].y, ot[i].y);
-          ot[i].z = fmaf(pc[c], v[c].z, ot[i].z);
-          ot[i].w = fmaf(pc[c], v[c].w, ot[i].w);
+      for (int c = 0; c < 4; ++c) {
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          const float x = c == 0 ? p[i].x : c == 1 ? p[i].y : c == 2 ? p[i].z : p[i].w;
+          const float2 pp = make_float2(x, x);
+          ot[i][0] = __ffma2_rn(pp, make_float2(v[c].x, v[c].y), ot[i][0]);
+          ot[i][1] = __ffma2_rn(pp, make_float2(v[c].z, v[c].w), ot[i][1]);
         }
       }
     }
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
-      o[i].x = fmaf(o[i].x, al[i], ot[i].x);
-      o[i].y = fmaf(o[i].y, al[i], ot[i].y);
-      o[i].z = fmaf(o[i].z, al[i], ot[i].z);
-      o[i].w = fmaf(o[i].w, al[i], ot[i].w);
+      o[i].x = fmaf(o[i].x, al[i], ot[i][0].x);
+      o[i].y = fmaf(o[i].y, al[i], ot[i][0].y);
+      o[i].z = fmaf(o[i].z, al[i], ot[i][1].x);
+      o[i].w = fmaf(o[i].w, al[i], ot[i][1].y);
     }
   };
   for (int b0 = blk0, buf = 0; b0 < blk1; b0 += 4, buf ^= 1) {
