@@ -78,13 +78,13 @@ def decode_traffic(alg_bytes_per_launch):
 
 def decode_kernel_label(w) -> str:
     """Kernel that the library's dispatch gives a full-batch decode call of `w` (sessions
-    at full budget): the 16-warp pair split while every (session, KV head) pair gets five
+    at full budget): the 16-warp pair split while every (session, KV head) pair gets six
     one-CTA-per-SM slices, the 4-warp pair split while it gets two of the three CTAs per
     SM, or one with at least 7/8 of them taken, else stream-K."""
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     pairs = w.n_sessions * w.kv_heads
-    if 5 * pairs <= sms:
+    if 6 * pairs <= sms:
         return "attn_decode_split_kernel (16 warps)"
     if 2 * pairs <= 3 * sms or 3 * sms * 7 // 8 < pairs <= 3 * sms:
         return "attn_decode_split_kernel (4 warps)"

@@ -1,9 +1,10 @@
 // Dispatch of a decode attention call (one token per session) between the three
 // kernel shapes, by the number of (session, KV head) pairs it has and the pages of its
 // longest session (estimated on the host):
-//   - pair split, 16-warp CTAs (one per SM): sessions of 100 pages or more when every
-//     pair gets k >= 5 CTAs in one wave (at most 3 sessions of 8 KV heads on 152 SMs); for
-//     bfloat16 the pages run on the tensor cores;
+//   - pair split, 16-warp CTAs (one per SM): sessions of 55 pages or more of which each
+//     warp gets one at most, and long bfloat16 sessions when every pair gets 6 CTAs in one
+//     wave (at most 3 sessions of 8 KV heads on 152 SMs); for bfloat16 the pages run on the
+//     tensor cores;
 //   - pair split, 4-warp CTAs (three per SM, tensor-core pages for bfloat16): every
 //     other call whose pairs each get k >= 1 CTAs in one wave (with k = 1 a pair needs no
 //     merge), unless one slice each would leave many slots empty for long;
@@ -22,16 +23,32 @@ constexpr int MAX_PARTS = 64;      // partial states per pair (both pair-split s
 constexpr float LOG2E = 1.4426950408889634f;
 // Minimum (session, kv head, page) units per CTA of the stream-K split.
 constexpr int DEC_MIN_UNITS = 12;
-// The pair-split kernel takes calls whose pairs each get at least this many CTAs
-// in one wave: with 16-warp CTAs (one per SM) first, else with stream-K's 4-warp
-// CTAs (three per SM).  Only the 16-warp shape uses tagged partial states: with
-// 4-warp CTAs the fenced arrival measured faster.  Against the 16-warp shape, the 4-warp
-// one measured faster from 4 sessions on (15.4 against 16.7 us at 4, 26.4 against 28.1 at
-// 9) and slower below (11.7 against 8.1 at 1).
-constexpr int SPLIT_MIN_K = 5, SPLIT4_MIN_K = 1;
-// Below this many pages the 16-warp shape leaves most of its warps without one
-// (64 pages, 8 pairs: 6.8 us against 6.4-6.7 with 4 warps; 20 pages: 6.7 against 5.2).
-constexpr int WIDE_MIN_PAGES = 100;
+// The pair-split kernel takes calls whose pairs each get a CTA in one wave: the 16-warp CTAs
+// (one per SM) where they are the better shape, else stream-K's 4-warp CTAs (three per SM).
+// Only the 16-warp shape uses tagged partial states: with 4-warp CTAs the fenced arrival
+// measured faster.
+//
+// The 16-warp shape is the better one while each of its warps has one page at most and most
+// of them have one (us, bfloat16, 16-warp against the best slices of the 4-warp one):
+//   pages       8 pairs       16 pairs      20 pairs      24 pairs
+//   52          6.5 / 5.8     6.5 / 6.3     6.5 / 6.5     6.7 / 6.6
+//   63          6.6 / 6.4     6.5 / 6.6     6.6 / 6.8     6.8 / 6.8
+//   76          6.7 / 6.5     6.7 / 6.9     6.8 / 7.1     7.2 / 7.2
+//   101         6.9 / 7.0     6.9 / 7.1     7.3 / 7.3     8.6 / 7.5
+//   157         6.9 / 7.5     9.4 / 8.5     9.5 / 8.6    10.0 / 8.9
+//   257         7.5 / 9.5    10.5 / 10.5   12.0 / 11.1   12.6 / 11.9
+// Long sessions leave both shapes' warps many pages each.  Of 257 and 501 binary32 pages, 8
+// pairs take 7.9 and 11.1 us against 10.8 and 15.8, 16 pairs 11.2 and 16.7 against 11.2 and
+// 16.6, 24 pairs 13.9 and 22.3 against 12.4 and 19.0: the 16-warp shape up to a ninth of the
+// SMs.  bfloat16 stays with it up to a sixth, at up to 6 % more for 24 pairs, so that calls
+// of one to three long sessions run one kernel; at 28 pairs the 4-warp shape is 7-12 % faster.
+constexpr int WIDE_WARPS = 16, WIDE_MIN_PAGES = 55;
+constexpr int WIDE_LONG_K = 6, WIDE_LONG_K_F32 = 9, WIDE_LONG_PAGES = 256;
+bool use_wide(int slots, int n_pairs, int pages, int esz) {
+  if (pages >= WIDE_LONG_PAGES)
+    return n_pairs * (esz == 2 ? WIDE_LONG_K : WIDE_LONG_K_F32) <= slots;
+  return pages >= WIDE_MIN_PAGES && pages + 2 <= slots / n_pairs * WIDE_WARPS;
+}
 
 // One slice per pair against stream-K, 257 pages, 8 KV heads: 92.9 against 77.5 us at 30
 // sessions (a slice's CTA takes 63 us by itself), 104.7 against 100.7 at 40, 121.4 against
@@ -42,27 +59,42 @@ bool one_slice_too_few(int slots, int n_pairs, int pages) {
   return pages >= STREAM_K_MIN_PAGES && n_pairs <= slots * 7 / 8;
 }
 
-// Slices per pair of the 16-warp shape: no more than give each warp a page (257 pages, 8
-// pairs: 7.6 us at 17 slices, 7.9 at 19, 8.9 at 15; 4 pairs: 7.2 at 19, 8.4 at 38).
+// Slices per pair of the 16-warp shape: 17, which gives 272 pages a warp each, and more for
+// longer sessions (8 pairs of 257 pages: 7.5 us at 17 slices, 8.2 at 19, 8.8 at 15; of 157:
+// 6.9 at 17, 7.1 at 11; 4 pairs of 257: 7.2 at 19, 8.4 at 38).
 int wide_slices(int slots, int n_pairs, int pages) {
-  return min(MAX_PARTS, min(slots / n_pairs, (pages + 15) / 16));
+  return min(MAX_PARTS, min(slots / n_pairs, max(17, (pages + 2 + 15) / WIDE_WARPS)));
 }
 
-// ... and of the 4-warp shape: up to 5/6 of the slots for as long as that leaves 6 slices or
-// more, all of them beyond (257 pages: 14.5 us at 12 slices of 32 pairs, 15.0 at 14; 18.9 at 8
-// of 48, 19.6 at 9; but 26.0 at 6 of 72, 26.5 at 5), and about three pages per slice at least
-// (33 pages, one binary32 pair: 4.7 us at 12 slices, 9.9 at 64; 20 pages, 8 pairs: 5.2 at 8,
-// 6.1 at 12; 17 pages: 4.5 at 6, 9.3 at 64).  The CUDA-core pages of binary32 are bound by
-// the pages of a warp: there more slices are taken if they save a warp one (48 pairs of 130
+// ... and of the 4-warp shape (two more pages than estimated: the partly filled ones of both
+// regions).  Up to 5/6 of the slots for as long as that leaves 6 slices or more, all of them
+// beyond (257 pages: 14.5 us at 12 slices of 32 pairs, 15.0 at 14; 18.9 at 8 of 48, 19.6 at 9;
+// but 26.0 at 6 of 72, 26.5 at 5), from 300 pages on as long as it leaves 8 (64 pairs: 39.9 us
+// at 7 slices of 501 pages, 41.4 at 6, but 24.0 and 23.1 of 257); and no more than 14, as the
+// merge is the dearer part beyond (8 pairs of 52 pages: 5.8 us at 14 slices, 6.3 at 16, 6.7 at
+// 18; of 76: 6.5, 7.1, 7.2).
+// bfloat16 takes a page per warp at least, and the fewest slices that leave a warp as few
+// pages (72 pairs of 76 pages: 9.9 us at 5 slices, 10.7 at 6; 32 of 157: 10.2 at 10, 10.7 at
+// 12; 16 of 29: 5.7 at 8, 6.3 at 10).  The CUDA-core pages of binary32 are bound by the pages
+// of a warp: about two pages per slice at least (20 pages, 16 pairs: 4.9 us at 11 slices, 5.2
+// at 8; 24 pairs: 5.0 and 5.2), and more slices if they save a warp one (48 pairs of 130
 // pages: 12.0 us at 9 slices, 12.5 at 8).
+constexpr int NARROW_MAX = 14, NARROW_WARPS = 4, ALL_MIN_PAGES = 300;
 int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
-  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs;
-  int fit = five_sixths >= 6 ? five_sixths : slots / n_pairs;
-  // (Two more pages than estimated: the partly filled ones of both regions.)
-  auto warp_pages = [&](int k) { return ((pages + 2 + k - 1) / k + 3) / 4; };
-  for (int k = fit + 1; cuda_cores && k <= slots / n_pairs; ++k)
-    if (warp_pages(k) < warp_pages(fit)) fit = k;
-  return max(1, min(MAX_PARTS, min(fit, (pages + 2) / 3)));
+  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs, all = slots / n_pairs;
+  auto warp_pages = [&](int k) {
+    return ((pages + 2 + k - 1) / k + NARROW_WARPS - 1) / NARROW_WARPS;
+  };
+  const int fit = five_sixths >= (pages < ALL_MIN_PAGES ? 6 : 8) ? five_sixths : all;
+  int k = min(NARROW_MAX, fit);
+  if (cuda_cores) {
+    for (int more = k + 1; more <= min(NARROW_MAX, all); ++more)
+      if (warp_pages(more) < warp_pages(k)) k = more;
+    return max(1, min(k, (pages + 2) / 2));
+  }
+  k = max(1, min(k, (pages + 2 + NARROW_WARPS - 1) / NARROW_WARPS));
+  while (k > 5 && warp_pages(k - 1) == warp_pages(k)) --k;
+  return k;
 }
 
 }  // namespace
@@ -86,10 +118,8 @@ cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out
   const int grid = sh.grid, slots = sh.slots, slots4 = sh.slots4;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   const int n_pairs = n_seq * d.kv_heads;
-  const int k = n_pairs * SPLIT_MIN_K <= slots && pages >= WIDE_MIN_PAGES
-                    ? wide_slices(slots, n_pairs, pages) : 0;
-  int k4 = k == 0 && n_pairs * SPLIT4_MIN_K <= slots4
-               ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
+  const int k = use_wide(slots, n_pairs, pages, esz) ? wide_slices(slots, n_pairs, pages) : 0;
+  int k4 = k == 0 && n_pairs <= slots4 ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
   if (k4 == 1 && one_slice_too_few(slots4, n_pairs, pages)) k4 = 0;
   // Tensor maps of the pool for the tensor-core page loop (bfloat16).
   CUtensorMap map_lo, map_hi;

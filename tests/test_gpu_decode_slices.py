@@ -35,6 +35,12 @@ CASES = {
     "8 pairs, 64 pages": (8, [1023], -1),
     "8 pairs, 101 pages": (8, [1610], -1),
     "16 pairs, 7 and 110 pages": (8, [100, 1760], -1),
+    "8 pairs, 54 pages": (8, [863], -1),
+    "8 pairs, 55 pages": (8, [864], -1),
+    "8 pairs, 300 pages": (8, [4800], -1),
+    "12 pairs, 190 pages": (4, [3030, 70, 3000], -1),
+    "24 pairs, 94 pages": (8, [40, 1490, 16], -1),
+    "24 pairs, 96 pages": (8, [40, 1530, 16], -1),
     "24 pairs": (8, [500, 501, 33], 300),
     "48 pairs": (8, [340, 1, 64, 1030, 335, 500], -1),
     "72 pairs": (8, [200 + 16 * i for i in range(9)], 180),
