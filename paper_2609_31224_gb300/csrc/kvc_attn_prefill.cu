@@ -3,11 +3,11 @@
 // For each session of the last append (T <= 32 tokens, e.g. the 17 acoustic
 // positions of a one-second unit), each KV head and its G = 4 query heads, the
 // T*G query rows attend to every resident key at or before their own position
-// (causal inside the chunk).  Split-K work items as in decode.
+// (causal inside the chunk).
 //
-// bfloat16 runs on the tcgen05 tensor cores (kvc_attn_prefill_tc.cu); this
-// file holds the launcher, the TMA tensor maps over the pool and the binary32
-// CUDA-core kernel (one thread per query row).
+// bfloat16 runs on the tcgen05 tensor cores (kvc_attn_prefill_tc.cu), binary32
+// on CUDA cores (kvc_attn_prefill_f32.cu); this file holds the launcher, the
+// choice of split and the TMA tensor maps over the pool.
 #include <cuda.h>
 
 #include <algorithm>
