@@ -1002,37 +1002,52 @@ __global__ void __launch_bounds__(256) evict_copy_kernel(Dev d) {
 // retained (= position) order.  Part 1 (one CTA): compaction of the retained
 // slots by type (block scan); the global slots go to the move list, used as
 // scratch, and the positions to pos_out.  Part 2: K and V rows of every layer.
+//
+// Part 1 is bound by its rounds of dependent loads (page list, type, position)
+// and scans: a thread takes GATHER slots in a row, so that a round covers
+// GATHER * META_THREADS slots with its loads in flight together.
+// An export of 4,100 slots of one bfloat16 layer: 14.1 -> 6.6 us, of 13,700 slots 26.7 -> 12.7,
+// against a slot per thread and round and each kernel waiting for the end of the one before.
 // ---------------------------------------------------------------------------
+constexpr int GATHER = 8;
+
 __global__ void __launch_bounds__(META_THREADS) transcript_gather_kernel(Dev d, int sid, int cap,
                                                                          int32_t* pos_out,
                                                                          int32_t* count) {
+  pdl_wait();
+  pdl_launch_dependents();
   __shared__ int s_warp[33];
   const SessState st = d.sess[sid];
   const int n = st.n_hist + st.n_live;
   const int32_t* hrow = d.hist_pt + (size_t)sid * d.max_pages_per_session;
   const int32_t* lrow = d.live_pt + (size_t)sid * d.max_pages_per_session;
   int done = 0;
-  for (int b0 = 0; b0 < n; b0 += META_THREADS) {
-    const int i = b0 + threadIdx.x;
-    int gs = 0;
-    bool tr = false;
-    if (i < n) {
-      if (i < st.n_hist) {
-        gs = hrow[i / PS] * PS + i % PS;
-      } else {
-        const int j = st.live_head + i - st.n_hist;
-        gs = lrow[j / PS] * PS + j % PS;
-      }
-      tr = d.meta_type[gs] == KVC_TRANSCRIPT;
+  for (int b0 = 0; b0 < n; b0 += GATHER * META_THREADS) {
+    int gs[GATHER];
+#pragma unroll
+    for (int e = 0; e < GATHER; ++e) {
+      const int i = b0 + GATHER * (int)threadIdx.x + e;
+      const int j = st.live_head + i - st.n_hist;
+      gs[e] = i >= n          ? -1
+              : i < st.n_hist ? hrow[i / PS] * PS + i % PS
+                              : lrow[j / PS] * PS + j % PS;
     }
+    unsigned tr = 0;
+#pragma unroll
+    for (int e = 0; e < GATHER; ++e)
+      tr |= (unsigned)(gs[e] >= 0 && d.meta_type[gs[e]] == KVC_TRANSCRIPT) << e;
     int total;
-    const int idx = done + block_exclusive_scan(tr ? 1 : 0, &total, s_warp);
-    if (tr && idx < cap) {
-      pos_out[idx] = d.meta_pos[gs];
-      d.moves[idx] = make_int2(gs, 0);
+    int idx = done + block_exclusive_scan(__popc(tr), &total, s_warp);
+#pragma unroll
+    for (int e = 0; e < GATHER; ++e) {
+      if (!(tr >> e & 1)) continue;
+      if (idx < cap) {
+        pos_out[idx] = d.meta_pos[gs[e]];
+        d.moves[idx] = make_int2(gs[e], 0);
+      }
+      ++idx;
     }
     done += total;
-    __syncthreads();  // s_warp is reused by the next scan
   }
   if (threadIdx.x == 0) {
     *count = done;
@@ -1040,28 +1055,40 @@ __global__ void __launch_bounds__(META_THREADS) transcript_gather_kernel(Dev d, 
   }
 }
 
-// Rows [L][cap][Hkv][D] of K and V; 16-byte units, grid-stride.
+// Rows [L][cap][Hkv][D] of K and V.  A warp takes the K or V rows of all heads of one
+// position of one layer, four 16-byte loads of a lane in flight before their stores.
+// 615 positions of 32 bfloat16 layers (161 MB read and written, 24 us at 6.8 TB/s): 48.5 ->
+// 32.1 us with part 1, against one load in flight per thread.
 __global__ void __launch_bounds__(256) transcript_copy_kernel(Dev d, int cap, uint8_t* k_out,
                                                               uint8_t* v_out) {
-  const int n = d.g->n_moves;
-  const int vec_per_row = d.head_dim * d.esz / 16;
-  const int64_t total = (int64_t)n * d.layers * 2 * d.kv_heads * vec_per_row;
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < total;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const int v = (int)(u % vec_per_row);
-    int64_t r = u / vec_per_row;
-    const int h = (int)(r % d.kv_heads);
-    r /= d.kv_heads;
-    const int kv = (int)(r % 2);
-    r /= 2;
-    const int i = (int)(r % n);
-    const int l = (int)(r / n);
+  pdl_wait();
+  pdl_launch_dependents();
+  constexpr int BATCH = 4;
+  const int n = d.g->n_moves, lane = threadIdx.x & 31;
+  const int vec_per_row = d.head_dim * d.esz / 16, n_vec = d.kv_heads * vec_per_row;
+  const int64_t total = (int64_t)n * d.layers * 2;
+  const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x / 32);
+  for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; u < total; u += n_warps) {
+    const int lk = (int)(u / n), i = (int)(u - (int64_t)lk * n), l = lk / 2, kv = lk % 2;
     const int gs = d.moves[i].x;
-    const size_t src = pool_offset_elems(d, gs / PS, l, kv, h, gs % PS) * d.esz + (size_t)v * 16;
-    const size_t dst =
-        (((size_t)l * cap + i) * d.kv_heads + h) * d.head_dim * d.esz + (size_t)v * 16;
-    *reinterpret_cast<uint4*>((kv ? v_out : k_out) + dst) =
-        *reinterpret_cast<const uint4*>(d.pool + src);
+    const uint8_t* src = d.pool + pool_offset_elems(d, gs / PS, l, kv, 0, gs % PS) * d.esz;
+    uint8_t* dst = (kv ? v_out : k_out) + ((size_t)l * cap + i) * n_vec * 16;
+    for (int v0 = lane; v0 < n_vec; v0 += 32 * BATCH) {
+      uint4 x[BATCH];
+#pragma unroll
+      for (int e = 0; e < BATCH; ++e) {
+        const int v = v0 + 32 * e, h = v / vec_per_row;
+        // (A head's rows are PS rows apart in a page.)
+        if (v < n_vec)
+          x[e] = *reinterpret_cast<const uint4*>(
+              src + ((size_t)h * PS * vec_per_row + (v - h * vec_per_row)) * 16);
+      }
+#pragma unroll
+      for (int e = 0; e < BATCH; ++e) {
+        const int v = v0 + 32 * e;
+        if (v < n_vec) *reinterpret_cast<uint4*>(dst + (size_t)v * 16) = x[e];
+      }
+    }
   }
 }
 
@@ -1172,13 +1199,14 @@ cudaError_t launch_evict(const Dev& d, const SeqArgs& a, int64_t* resident_out, 
 
 cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_out, void* k_out,
                               void* v_out, int32_t* count, cudaStream_t s) {
-  transcript_gather_kernel<<<1, META_THREADS, 0, s>>>(d, session, cap, pos_out, count);
+  cudaError_t e = launch_ex(&transcript_gather_kernel, dim3(1), dim3(META_THREADS), 0, s, true, d,
+                            session, cap, pos_out, count);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  transcript_copy_kernel<<<sms * 4, 256, 0, s>>>(d, cap, static_cast<uint8_t*>(k_out),
-                                                 static_cast<uint8_t*>(v_out));
-  return cudaGetLastError();
+  return launch_ex(&transcript_copy_kernel, dim3(sms * 4), dim3(256), 0, s, true, d, cap,
+                   static_cast<uint8_t*>(k_out), static_cast<uint8_t*>(v_out));
 }
 
 cudaError_t launch_release(const Dev& d, const SeqArgs& a, int64_t* used_out, cudaStream_t s) {
