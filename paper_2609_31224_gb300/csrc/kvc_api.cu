@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "kvc_launch.cuh"
+#include "kvc_order.h"
 
 using namespace kvc;
 
@@ -172,8 +173,7 @@ struct kvc_ctx {
   // eviction policy is to keep.  They guide the choice of the attention's split only.
   int est_pages_max = 0;
   int64_t est_pages_sum = 0;
-  int attn_since_append = 0;  // attention launches since the last append (or layer write)
-  uint64_t layers_written = 0;  // layers whose K/V of the last append are in the pool
+  LaunchOrder order;       // of the attention launches since the last append
   bool last_single = false;
   uint32_t dec_epoch = 0;  // tag of the last decode launch's partial states
 };
@@ -391,8 +391,7 @@ int kvc_append_chunk(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, const i
   ctx->used_ub += need;
   ctx->delta_since_readback += need;
   ctx->attn_valid = true;
-  ctx->attn_since_append = 0;
-  ctx->layers_written = d_k ? (ctx->cfg.layers == 64 ? ~0ull : (1ull << ctx->cfg.layers) - 1) : 0;
+  ctx->order.append(d_k != nullptr, ctx->cfg.layers);
   ctx->last_n_seq = n_seq;
   ctx->last_total = total;
   ctx->last_max_t = max_t;
@@ -411,10 +410,9 @@ int kvc_append_kv_layer(kvc_ctx* ctx, int layer, const void* d_k, const void* d_
     return fail(KVC_ESTATE, "kvc_append_kv_layer needs a preceding kvc_append_chunk (no evict/release after it)");
   KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false,
                                 static_cast<cudaStream_t>(stream)));
-  ctx->layers_written |= 1ull << layer;
-  // The next attention launch must not start early: its prologue loads pages
+  // The next attention launch must not read early: its prologue loads pages
   // this write may still be filling.
-  ctx->attn_since_append = 0;
+  ctx->order.layer_write(layer);
   return KVC_OK;
 }
 
@@ -463,7 +461,7 @@ static int check_attn(kvc_ctx* ctx, int layer, const void* d_q, void* d_out,
   if (!aligned16(d_q) || !aligned16(d_out)) return fail(KVC_EINVAL, "d_q / d_out must be 16-byte aligned");
   if (!ctx->attn_valid)
     return fail(KVC_ESTATE, "attention needs a preceding kvc_append_chunk (no evict/release after it)");
-  if (!writes_layer && !((ctx->layers_written >> layer) & 1))
+  if (!writes_layer && !ctx->order.layer_written(layer))
     return fail(KVC_ESTATE, "layer %d's K/V of the last append are not written (kvc_append_kv_layer)",
                 layer);
   return KVC_OK;
@@ -475,14 +473,12 @@ int kvc_attn_decode(kvc_ctx* ctx, int layer, const void* d_q, void* d_out, void*
   if (rc) return rc;
   if (!ctx->last_single)
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
-  // The first attention launch after an append follows the kernel that wrote the new
-  // token's K/V, so it reads nothing before that is complete; later ones may.
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
   KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
-                              ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream),
+                              ctx->order.early(layer, false), static_cast<cudaStream_t>(stream),
                               epoch));
-  ++ctx->attn_since_append;
+  ctx->order.launched(layer, false);
   return KVC_OK;
 }
 
@@ -495,15 +491,14 @@ int kvc_attn_decode_kv(kvc_ctx* ctx, int layer, const void* d_k, const void* d_v
   if (!aligned16(d_k) || !aligned16(d_v)) return fail(KVC_EINVAL, "d_k / d_v must be 16-byte aligned");
   if (!ctx->last_single)
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
-  // Launches after the append may start early: the new rows go into the tiles
-  // after their loads, and the previous launch writes another layer's rows only.
+  // (An early launch may load the page while a launch before it writes the new row's slot:
+  // the row goes into the tile after its load.)
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
   KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
-                              ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream),
+                              ctx->order.early(layer, true), static_cast<cudaStream_t>(stream),
                               epoch, d_k, d_v));
-  ctx->layers_written |= 1ull << layer;
-  ++ctx->attn_since_append;
+  ctx->order.launched(layer, true);
   return KVC_OK;
 }
 
@@ -533,11 +528,11 @@ int kvc_attn_prefill_chunk(kvc_ctx* ctx, int layer, const void* d_q, void* d_out
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
   KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
                                ctx->est_pages_max, ctx->est_pages_sum,
-                               ctx->attn_since_append > 0, static_cast<cudaStream_t>(stream)));
-  ++ctx->attn_since_append;
+                               ctx->order.early(layer, false),
+                               static_cast<cudaStream_t>(stream)));
+  ctx->order.launched(layer, false);
   return KVC_OK;
 }
-
 
 int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const void* d_v,
                               const void* d_q, void* d_out, void* stream) {
@@ -550,21 +545,20 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (ctx->d.esz == 2) {
-    // Launches after the append may start early: a stage holding chunk slots is
-    // copied only after its rows are written, and the previous launch writes
-    // another layer's rows only.
+    // (A stage holding chunk slots is copied only after this launch has written its rows.)
     KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
-                               ctx->est_pages_max, ctx->est_pages_sum,
-                                 ctx->attn_since_append > 0, s, d_k, d_v));
+                                 ctx->est_pages_max, ctx->est_pages_sum,
+                                 ctx->order.early(layer, true), s, d_k, d_v));
+    ctx->order.launched(layer, true);
   } else {
     // Binary32 (CUDA-core prefill): the rows first, then the attention, unoverlapped.
     KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false, s));
+    ctx->order.layer_write(layer);
     KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
-                               ctx->est_pages_max, ctx->est_pages_sum,
-                                 false, s));
+                                 ctx->est_pages_max, ctx->est_pages_sum,
+                                 ctx->order.early(layer, false), s));
+    ctx->order.launched(layer, false);
   }
-  ctx->layers_written |= 1ull << layer;
-  ++ctx->attn_since_append;
   return KVC_OK;
 }
 
