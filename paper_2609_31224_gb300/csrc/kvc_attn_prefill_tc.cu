@@ -392,6 +392,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
     }
     fence_proxy_async_smem();
   }
+  __syncwarp();  // (lanes took the branches above apart; the allocation wants them together)
   if (warp == 2) tmem_alloc(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
@@ -637,7 +638,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       dead = !__all_sync(FULL, mbar_wait(d, bar, parity));
       if (dead && lane == 0) s_abort = 1;
     };
-    auto sync_groups = [] { asm volatile("bar.sync 1, %0;" ::"n"(SM_THREADS) : "memory"); };
+    // (bar.sync and the tensor-memory accesses want the warp converged.)
+    auto sync_groups = [] {
+      __syncwarp();
+      asm volatile("bar.sync 1, %0;" ::"n"(SM_THREADS) : "memory");
+    };
     uint8_t* st_q = smem + off_q(ring);
     uint8_t* st_rope = smem + off_rope(ring, max_t);
     uint8_t* st_out = smem + off_out(ring, max_t);
@@ -834,6 +839,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
         }
         const float2 r2 = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
         l += r2.x + r2.y;
+        __syncwarp();
         tmem_st32(trow + P_COL + grp * (NK / 2), pw);
         tc_fence_before();
         __syncwarp();
@@ -859,6 +865,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       const float Lr = (has0 ? ml0.y * f0 : 0.f) + (has1 ? ml1.y * f1 : 0.f);
       // Columns [64 grp + 32 c, + 32) of this row, both groups' parts summed.
       auto own = [&](int c, float sc, float (&o)[32]) {
+        __syncwarp();  // (rows that are not live skip the stores of the columns before)
         const uint32_t col = trow + O_COL + 64 * grp + 32 * c;
         const float a0 = f0 * sc, a1 = f1 * sc;
         if (has0) {
@@ -998,6 +1005,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
                 make_uint4(pack_bf16(o[i], o[i + 1]), pack_bf16(o[i + 2], o[i + 3]),
                            pack_bf16(o[i + 4], o[i + 5]), pack_bf16(o[i + 6], o[i + 7]));
         });
+    __syncwarp();
     asm volatile("bar.sync 1, %0;" ::"n"(SM_THREADS) : "memory");
     for (int i = ts; i < R * 16; i += SM_THREADS) {
       const int row = i >> 4, c = i & 15;

@@ -1,0 +1,36 @@
+"""Rules of the kernels that a run cannot show to be broken, read off their sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2609_31224_gb300", "csrc")
+
+
+def code(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def statement_before(text, at):
+    """The statement that ends before offset `at`."""
+    head = text[:at].rstrip().rstrip("{").rstrip()
+    return head[max(head[:-1].rfind(";"), head[:-1].rfind("}"), head[:-1].rfind("{")) + 1:].strip()
+
+
+@pytest.mark.parametrize("name,calls", [
+    ("kvc_attn_prefill_f32.cu", [r'asm volatile\("barrier\.cluster\.arrive']),
+    ("kvc_attn_prefill_tc.cu", [r"cluster_arrive\(\);", r"cluster_wait\(\);",
+                                r'asm volatile\("bar\.sync', r"if \(warp == 2\) tmem_alloc"]),
+])
+def test_aligned_barriers_follow_a_reconvergence(name, calls):
+    """Warp-aligned instructions behind code that lanes run apart (rows of their own, loops of
+    different lengths) come right after a __syncwarp() or a barrier of the whole CTA."""
+    text = code(name)
+    for call in calls:
+        found = list(re.finditer(call, text))
+        assert found, call
+        for m in found:
+            assert re.match(r"__sync(warp|threads)\(\);", statement_before(text, m.start())), \
+                text[m.start() - 200:m.end()]
