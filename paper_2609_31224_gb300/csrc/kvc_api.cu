@@ -165,7 +165,7 @@ struct kvc_ctx {
   bool readback_pending = false;
   cudaEvent_t ev = nullptr;
   int64_t* h_readback = nullptr;  // pinned, written by evict and release
-  int sms = 0;
+  Limits lim = {};  // of the device that it was created on
   // Last append (queries of the following attention calls).
   bool attn_valid = false;
   int last_n_seq = 0, last_total = 0, last_max_t = 0;
@@ -307,10 +307,9 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
       launch_init(d, cfg->rope_base, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return cleanup(fail(KVC_ECUDA, "initialisation failed: %s",
                         cudaGetErrorString(cudaGetLastError())));
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return cleanup(fail(KVC_ECUDA, "device query failed"));
+  const cudaError_t le = query_limits(d, &ctx->lim);
+  if (le != cudaSuccess)
+    return cleanup(fail(KVC_ECUDA, "device query failed: %s", cudaGetErrorString(le)));
   *out = ctx;
   return KVC_OK;
 }
@@ -426,7 +425,7 @@ int kvc_evict(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, int64_t* d_res
   a.n_seq = n_seq;
   for (int i = 0; i < n_seq; ++i) a.sessions[i] = h_sessions[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, ctx->h_readback, ctx->sms, s));
+  KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, ctx->h_readback, ctx->lim.sms, s));
   ctx->used_ub += n_seq;  // an evict adds at most one page per session, net
   enqueue_readback(ctx, s);
   ctx->attn_valid = false;
@@ -475,9 +474,9 @@ int kvc_attn_decode(kvc_ctx* ctx, int layer, const void* d_q, void* d_out, void*
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
-  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
-                              ctx->order.early(layer, false), static_cast<cudaStream_t>(stream),
-                              epoch));
+  KVC_CUDA(launch_attn_decode(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
+                              ctx->est_pages_max, ctx->order.early(layer, false),
+                              static_cast<cudaStream_t>(stream), epoch));
   ctx->order.launched(layer, false);
   return KVC_OK;
 }
@@ -495,9 +494,9 @@ int kvc_attn_decode_kv(kvc_ctx* ctx, int layer, const void* d_k, const void* d_v
   // the row goes into the tile after its load.)
   uint32_t epoch = 0;
   KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
-  KVC_CUDA(launch_attn_decode(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->est_pages_max,
-                              ctx->order.early(layer, true), static_cast<cudaStream_t>(stream),
-                              epoch, d_k, d_v));
+  KVC_CUDA(launch_attn_decode(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
+                              ctx->est_pages_max, ctx->order.early(layer, true),
+                              static_cast<cudaStream_t>(stream), epoch, d_k, d_v));
   ctx->order.launched(layer, true);
   return KVC_OK;
 }
@@ -526,8 +525,8 @@ int kvc_attn_prefill_chunk(kvc_ctx* ctx, int layer, const void* d_q, void* d_out
   if (rc) return rc;
   if (ctx->last_max_t > PF_MAX_TOKENS)
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
-  KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
-                               ctx->est_pages_max, ctx->est_pages_sum,
+  KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
+                               ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
                                ctx->order.early(layer, false),
                                static_cast<cudaStream_t>(stream)));
   ctx->order.launched(layer, false);
@@ -546,16 +545,16 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (ctx->d.esz == 2) {
     // (A stage holding chunk slots is copied only after this launch has written its rows.)
-    KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
-                                 ctx->est_pages_max, ctx->est_pages_sum,
+    KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
+                                 ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
                                  ctx->order.early(layer, true), s, d_k, d_v));
     ctx->order.launched(layer, true);
   } else {
     // Binary32 (CUDA-core prefill): the rows first, then the attention, unoverlapped.
     KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false, s));
     ctx->order.layer_write(layer);
-    KVC_CUDA(launch_attn_prefill(ctx->d, layer, d_q, d_out, ctx->last_n_seq, ctx->last_max_t,
-                                 ctx->est_pages_max, ctx->est_pages_sum,
+    KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
+                                 ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
                                  ctx->order.early(layer, false), s));
     ctx->order.launched(layer, false);
   }

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
 
 // Resident CTAs of the pair-split kernel with CTA shape C (one wave).
 template <typename T, int D, class C>
-int split_slots() {
+int split_slots(int sms) {
   const void* fn = reinterpret_cast<const void*>(&attn_decode_split_kernel<T, D, false, C>);
   const int smem = C::SMEM;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -262,9 +262,6 @@ int split_slots() {
                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, C::THREADS, smem);
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return max(0, per_sm) * sms;
 }
 
@@ -283,11 +280,12 @@ cudaError_t launch_split(const Dev& d, int layer, const CUtensorMap& map_lo,
 
 }  // namespace
 
-int decode_split_slots(int esz, bool wide) {
+int decode_split_slots(int esz, bool wide, int sms) {
   if (esz == 2)
-    return wide ? split_slots<__nv_bfloat16, 128, SpCfg<__nv_bfloat16, 128>>()
-                : split_slots<__nv_bfloat16, 128, Sp4Cfg<__nv_bfloat16, 128>>();
-  return wide ? split_slots<float, 64, SpCfg<float, 64>>() : split_slots<float, 64, Sp4Cfg<float, 64>>();
+    return wide ? split_slots<__nv_bfloat16, 128, SpCfg<__nv_bfloat16, 128>>(sms)
+                : split_slots<__nv_bfloat16, 128, Sp4Cfg<__nv_bfloat16, 128>>(sms);
+  return wide ? split_slots<float, 64, SpCfg<float, 64>>(sms)
+              : split_slots<float, 64, Sp4Cfg<float, 64>>(sms);
 }
 
 bool decode_split_uses_tma(int esz, bool wide) {

@@ -89,36 +89,6 @@ bool pool_tensor_maps(const Dev& d, CUtensorMap* lo, CUtensorMap* hi) {
 
 namespace {
 
-int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
-// CTAs of the bfloat16 kernel resident at once.
-int pf_grid(const void* fn, int threads, int smem) {
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-  return max(1, per_sm) * sm_count();
-}
-
-}  // namespace
-
-namespace {
-
-// Grid limits of the bfloat16 kernel on the current device: CTAs of the stream-K split
-// (resident at once), clusters of k CTAs of the pair split.
-struct TcLimits {
-  int grid = 0;
-  int clusters[17] = {};
-  TcLimits() {
-    grid = pf_grid(prefill_tc_kernel_ptr(), prefill_tc_threads(), prefill_tc_smem());
-    for (int k = 1; k <= prefill_tc_max_slices(); ++k) clusters[k] = prefill_tc_max_clusters(k);
-  }
-};
-
 // Slices per pair of the pair split, or 0 for stream-K, whichever is expected to take less.
 // n_pairs pairs, the longest of `s_max` stages (4 pages), `total` stages in all.  Times in
 // us, fitted to 32-layer runs of 1-20 sessions of 8 KV heads at 200-10,600 positions:
@@ -130,12 +100,12 @@ struct TcLimits {
 // Measured at 4,100 positions (pair split with the k chosen / stream-K): 12.6 / 33.4 at one
 // session, 14.4 / 28.5 at 2, 19.6 / 27.7 at 4, 31.1 / 35.6 at 9, 43.9 / 37.1 at 10 (k = 1),
 // 45.5 / 49.4 at 16; at 250 positions 7.6 / 14.9 at one session, 8.9 / 18.9 at 16.
-int prefill_slices(const TcLimits& lim, int n_pairs, double s_max, double total) {
-  const double per = std::max(1.0, total / lim.grid);
+int prefill_slices(const Limits& lim, int n_pairs, double s_max, double total) {
+  const double per = std::max(1.0, total / lim.pf_stream_k);
   double best = 13.0 + 0.68 * per + 0.9 * std::max(1.0, s_max / per);
   int best_k = 0;
-  for (int k = 1; k <= prefill_tc_max_slices(); ++k) {
-    if (n_pairs > lim.clusters[k]) continue;
+  for (int k = 1; k <= PF_MAX_SLICES; ++k) {
+    if (n_pairs > lim.pf_clusters[k]) continue;
     const double t = std::max(0.0048 * total, 5.0 + 0.6 * std::ceil(s_max / k) + (k > 1 ? 2.5 : 0.0));
     if (t < best) {
       best = t;
@@ -147,23 +117,22 @@ int prefill_slices(const TcLimits& lim, int n_pairs, double s_max, double total)
 
 }  // namespace
 
-cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                int max_t, int pages_max, int64_t pages_sum, bool early,
-                                cudaStream_t s, const void* new_k, const void* new_v) {
+cudaError_t launch_attn_prefill(const Dev& d, const Limits& lim, int layer, const void* q,
+                                void* out, int n_seq, int max_t, int pages_max,
+                                int64_t pages_sum, bool early, cudaStream_t s, const void* new_k,
+                                const void* new_v) {
   if (d.esz == 2) {
-    static thread_local const TcLimits lim;
     CUtensorMap lo, hi;
     if (!pool_tensor_maps(d, &lo, &hi)) return cudaErrorInvalidValue;
     const int n_pairs = n_seq * d.kv_heads;
     const int k = prefill_slices(lim, n_pairs, (pages_max + 3) / 4,
                                  (double)d.kv_heads * (pages_sum / 4.0 + n_seq));
     // Each CTA of the stream-K split may write two partial slots.
-    const int grid = k > 0 ? n_pairs * k : std::min(lim.grid, d.pf_slots / 2);
+    const int grid = k > 0 ? n_pairs * k : std::min(lim.pf_stream_k, d.pf_slots / 2);
     return launch_attn_prefill_tc(d, layer, lo, hi, q, out, grid, k, max_t, early, s, new_k, new_v);
   }
   if (new_k != nullptr) return cudaErrorInvalidValue;  // binary32: the API writes the rows first
-  static thread_local const int sms = sm_count();
-  return launch_attn_prefill_f32(d, layer, q, out, n_seq, max_t, pages_max, sms, early, s);
+  return launch_attn_prefill_f32(d, lim, layer, q, out, n_seq, max_t, pages_max, early, s);
 }
 
 }  // namespace kvc

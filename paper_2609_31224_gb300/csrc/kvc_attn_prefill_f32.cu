@@ -339,14 +339,6 @@ __global__ void __launch_bounds__(THREADS, 2) attn_prefill_f32_kernel(
 template <int RT>
 cudaError_t launch(const Dev& d, int layer, const void* q, void* out, int n_pairs, int n_rb, int k,
                    bool spread, bool early, cudaStream_t s) {
-  static thread_local const cudaError_t attr_err = [] {
-    const void* fn = reinterpret_cast<const void*>(&attn_prefill_f32_kernel<RT>);
-    const cudaError_t e =
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ONE_PER_SM);
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  }();
-  if (attr_err != cudaSuccess) return attr_err;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_pairs * n_rb * k);
@@ -372,10 +364,49 @@ cudaError_t launch(const Dev& d, int layer, const void* q, void* out, int n_pair
                             (int)early);
 }
 
+// Attributes of the kernel, and the largest cluster of it that the device takes, without and
+// with the shared memory that spreads its CTAs over the SMs.
+template <int RT>
+cudaError_t limits(int (&largest)[2]) {
+  const void* fn = reinterpret_cast<const void*>(&attn_prefill_f32_kernel<RT>);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ONE_PER_SM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  for (int spread = 0; spread < 2; ++spread) {
+    largest[spread] = 1;
+    for (int k = MAX_K; k > 1 && largest[spread] == 1; --k) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(k);
+      cfg.blockDim = dim3(THREADS);
+      cfg.dynamicSmemBytes = spread ? ONE_PER_SM : Shape<RT>::SMEM;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = k;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      e = cudaOccupancyMaxActiveClusters(&n, &attn_prefill_f32_kernel<RT>, &cfg);
+      if (e == cudaSuccess && n > 0) largest[spread] = k;
+      if (e != cudaSuccess) cudaGetLastError();  // (a size that the device does not take: no error)
+    }
+  }
+  return cudaSuccess;
+}
+
 }  // namespace
 
-cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                    int max_t, int pages_max, int sms, bool early, cudaStream_t s) {
+cudaError_t prefill_f32_limits(Limits* lim) {
+  const cudaError_t e = limits<4>(lim->f32_cluster[0]);
+  return e != cudaSuccess ? e : limits<9>(lim->f32_cluster[1]);
+}
+
+cudaError_t launch_attn_prefill_f32(const Dev& d, const Limits& lim, int layer, const void* q,
+                                    void* out, int n_seq, int max_t, int pages_max, bool early,
+                                    cudaStream_t s) {
+  const int sms = lim.sms;
   // Rows per CTA: 32 (chunks of up to 8 tokens) or 72 (a 17-token unit's 68).
   const int R = max_t * G, n_pairs = n_seq * d.kv_heads;
   const bool small = R <= 32;
@@ -390,9 +421,10 @@ cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void
   const int fit = sms * 27 / 16 / blocks;
   int k = min(blocks <= 8 ? MAX_K : blocks <= 21 ? 12 : 8, fit);
   if (k < 2) k = blocks <= 3 * sms ? 3 : 1;
-  k = max(1, min(k, pages_max / 2));
+  const int* largest = lim.f32_cluster[small ? 0 : 1];  // (that the device takes at all)
+  k = max(1, min(min(k, largest[0]), pages_max / 2));
   // A small grid's clusters are spread over the SMs (4 pairs: 13.0 against 14.6 us).
-  const bool spread = 2 * blocks * k <= sms;
+  const bool spread = 2 * blocks * k <= sms && k <= largest[1];
   return small ? launch<4>(d, layer, q, out, n_pairs, n_rb, k, spread, early, s)
                : launch<9>(d, layer, q, out, n_pairs, n_rb, k, spread, early, s);
 }

@@ -59,7 +59,6 @@ constexpr int SM_THREADS = 8 * 32;           // softmax threads
 constexpr int PF_MIN_UNITS = 16;             // pages per CTA of the stream-K split, at least
 constexpr int PF_MAX_PARTS = 1 << 16;        // no limit on CTAs per pair (merged row by row)
 constexpr int MAX_RING = 6;                  // K/V stages of the ring, at most
-constexpr int MAX_K = 8;                     // slices of a pair (cluster size), at most
 
 // Shared memory map (offsets from a 1024-aligned base): barriers and (max, sum) pairs
 // first, then the K/V ring, then (CLUSTER) the partial rows sent to this CTA.
@@ -1053,7 +1052,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
       else if (k <= 4)
         merge_rows<4>(rows, own, slice, k, per, n_rows, tid, out_row);
       else
-        merge_rows<MAX_K>(rows, own, slice, k, per, n_rows, tid, out_row);
+        merge_rows<PF_MAX_SLICES>(rows, own, slice, k, per, n_rows, tid, out_row);
     }
     __syncwarp();
     cluster_wait();  // every part was received: no copy still reads this CTA's rows
@@ -1078,34 +1077,38 @@ cudaError_t set_attributes() {
 
 }  // namespace
 
-const void* prefill_tc_kernel_ptr() { return reinterpret_cast<const void*>(tc_kernel(false, false)); }
-int prefill_tc_smem() { return SMEM_MAX; }
-int prefill_tc_threads() { return THREADS; }
-int prefill_tc_max_slices() { return MAX_K; }
-
-int prefill_tc_max_clusters(int k) {
-  if (set_attributes() != cudaSuccess) return 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(k);
-  cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = SMEM_MAX;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = k;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  return cudaOccupancyMaxActiveClusters(&n, tc_kernel(false, true), &cfg) == cudaSuccess ? n : 0;
+cudaError_t prefill_tc_limits(Limits* lim) {
+  cudaError_t e = set_attributes();
+  if (e != cudaSuccess) return e;
+  const void* fn = reinterpret_cast<const void*>(tc_kernel(false, false));
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, THREADS, SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  lim->pf_stream_k = max(1, per_sm) * lim->sms;
+  for (int k = 1; k <= PF_MAX_SLICES; ++k) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(k);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_MAX;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = k;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, tc_kernel(false, true), &cfg);
+    lim->pf_clusters[k] = e == cudaSuccess ? n : 0;
+    if (e != cudaSuccess) cudaGetLastError();  // (a size that the device does not take: no error)
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
                                    int k, int max_t, bool early, cudaStream_t s, const void* new_k,
                                    const void* new_v) {
-  static thread_local const cudaError_t attr_err = set_attributes();
-  if (attr_err != cudaSuccess) return attr_err;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   // The deepest ring that leaves room for the rows sent to a CTA (k parts of its share).
   const int recv = k > 1 ? (max_t * G + k - 1) / k * k : 0;

@@ -99,23 +99,10 @@ int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
 
 }  // namespace
 
-cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               int pages, bool early, cudaStream_t s, uint32_t epoch,
-                               const void* new_k, const void* new_v) {
-  const int esz = d.esz;
-  // Grid sizes of the three shapes, per element type (their CTA shapes differ), worked
-  // out on a thread's first call with that type.
-  struct Shapes {
-    int grid = 0, slots = 0, slots4 = 0;
-  };
-  static thread_local Shapes shapes[2];
-  Shapes& sh = shapes[esz == 2 ? 1 : 0];
-  if (sh.grid == 0) {
-    sh.grid = decode_stream_k_grid(d);
-    sh.slots = decode_split_slots(esz, true);
-    sh.slots4 = decode_split_slots(esz, false);
-  }
-  const int grid = sh.grid, slots = sh.slots, slots4 = sh.slots4;
+cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const void* q,
+                               void* out, int n_seq, int pages, bool early, cudaStream_t s,
+                               uint32_t epoch, const void* new_k, const void* new_v) {
+  const int esz = d.esz, slots = lim.dec_wide, slots4 = lim.dec_narrow;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   const int n_pairs = n_seq * d.kv_heads;
   const int k = use_wide(slots, n_pairs, pages, esz) ? wide_slices(slots, n_pairs, pages) : 0;
@@ -138,8 +125,20 @@ cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out
   if (k4 > 0)
     return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale, k4, 0u, new_k,
                                     new_v, n_pairs, early, s);
-  return launch_attn_decode_streamk(d, layer, map_lo, map_hi, q, out, scale, grid, DEC_MIN_UNITS,
-                                    new_k, new_v, early, s);
+  return launch_attn_decode_streamk(d, layer, map_lo, map_hi, q, out, scale, lim.dec_stream_k,
+                                    DEC_MIN_UNITS, new_k, new_v, early, s);
+}
+
+cudaError_t query_limits(const Dev& d, Limits* lim) {
+  memset(lim, 0, sizeof(*lim));
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim->sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  lim->dec_stream_k = decode_stream_k_grid(d);
+  lim->dec_wide = decode_split_slots(d.esz, true, lim->sms);
+  lim->dec_narrow = decode_split_slots(d.esz, false, lim->sms);
+  return d.esz == 2 ? prefill_tc_limits(lim) : prefill_f32_limits(lim);
 }
 
 }  // namespace kvc

@@ -28,6 +28,21 @@ struct SeqArgsT {
 };
 using SeqArgs = SeqArgsT<MAX_SEQ>;
 
+// What the device runs at once, for each kernel whose launch shape follows from it.  Worked out
+// for the current device when a context is created, which also sets the kernels' attributes
+// there: nothing is kept per thread or process, so that contexts of several devices, and
+// several threads, do not meet one another's.
+constexpr int PF_MAX_SLICES = 8;  // CTAs of a bfloat16 prefill cluster, at most
+struct Limits {
+  int sms;                         // SMs
+  int dec_stream_k;                // CTAs of the stream-K decode's grid
+  int dec_wide, dec_narrow;        // CTAs of the 16-warp and 4-warp pair split in one wave
+  int pf_stream_k;                 // CTAs of the stream-K prefill (bfloat16)
+  int pf_clusters[PF_MAX_SLICES + 1];  // [k] clusters of k CTAs of the prefill's pair split
+  int f32_cluster[2][2];           // largest cluster of the binary32 prefill: [rows][spread]
+};
+cudaError_t query_limits(const Dev& d, Limits* lim);
+
 cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s);
 // single: every session of the call gets exactly one token (plan and K/V write in
 // one launch).
@@ -48,11 +63,12 @@ cudaError_t launch_transcript(const Dev& d, int session, int cap, int32_t* pos_o
 // epoch: tag of this launch's partial states (nonzero, never reused while tags
 // of it may remain in the slots); 0 selects the fenced arrival instead.
 // pages: estimate of the longest session's pages, for the choice of the split only.
-cudaError_t launch_attn_decode(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                               int pages, bool early, cudaStream_t s, uint32_t epoch,
-                               const void* new_k = nullptr, const void* new_v = nullptr);
+cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const void* q,
+                               void* out, int n_seq, int pages, bool early, cudaStream_t s,
+                               uint32_t epoch, const void* new_k = nullptr,
+                               const void* new_v = nullptr);
 // Stream-K decode kernel (kvc_attn_decode.cu): its grid (resident CTAs, capped by
-// the partial slots) and its launch.
+// the partial slots; sets its attributes) and its launch.
 int decode_stream_k_grid(const Dev& d);
 cudaError_t launch_attn_decode_streamk(const Dev& d, int layer, const CUtensorMap& map_lo,
                                        const CUtensorMap& map_hi, const void* q, void* out,
@@ -60,7 +76,8 @@ cudaError_t launch_attn_decode_streamk(const Dev& d, int layer, const CUtensorMa
                                        const void* new_v, bool early, cudaStream_t s);
 // Pair-split decode kernel (kvc_attn_decode_split.cu).  wide: the 16-warp shape
 // (one CTA per SM; tensor-core pages for bfloat16), else the 4-warp shape.
-int decode_split_slots(int esz, bool wide);          // resident CTAs in one wave
+// Resident CTAs in one wave (sets its attributes).
+int decode_split_slots(int esz, bool wide, int sms);
 bool decode_split_uses_tma(int esz, bool wide);      // needs the pool's tensor maps
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
@@ -70,28 +87,26 @@ cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const C
 // into the pool by the launch itself (the per-layer order).
 // pages_max, pages_sum: estimates of the sessions' resident pages (largest, sum over the
 // call), for the choice of the split only.
-cudaError_t launch_attn_prefill(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                int max_t, int pages_max, int64_t pages_sum, bool early,
-                                cudaStream_t s, const void* new_k = nullptr,
-                                const void* new_v = nullptr);
+cudaError_t launch_attn_prefill(const Dev& d, const Limits& lim, int layer, const void* q,
+                                void* out, int n_seq, int max_t, int pages_max,
+                                int64_t pages_sum, bool early, cudaStream_t s,
+                                const void* new_k = nullptr, const void* new_v = nullptr);
 // k = 0: stream-K over `grid` CTAs; k >= 1: pair split, grid = pairs * k CTAs.
 cudaError_t launch_attn_prefill_tc(const Dev& d, int layer, const CUtensorMap& lo,
                                    const CUtensorMap& hi, const void* q, void* out, int grid,
                                    int k, int max_t, bool early, cudaStream_t s, const void* new_k,
                                    const void* new_v);
-int prefill_tc_max_slices();
-// Clusters of k CTAs of the pair split that fit the current device at once.
-int prefill_tc_max_clusters(int k);
-// binary32; pages_max as in launch_attn_prefill, sms: SMs of the device.
-cudaError_t launch_attn_prefill_f32(const Dev& d, int layer, const void* q, void* out, int n_seq,
-                                    int max_t, int pages_max, int sms, bool early, cudaStream_t s);
-const void* prefill_tc_kernel_ptr();
+// Sets its attributes; CTAs of the stream-K split and clusters of the pair split at once.
+cudaError_t prefill_tc_limits(Limits* lim);
+// binary32; pages_max as in launch_attn_prefill.
+cudaError_t prefill_f32_limits(Limits* lim);
+cudaError_t launch_attn_prefill_f32(const Dev& d, const Limits& lim, int layer, const void* q,
+                                    void* out, int n_seq, int max_t, int pages_max, bool early,
+                                    cudaStream_t s);
 // Two 2-D views of the bfloat16 pool as rows of 128 elements (columns 0-63 and
 // 64-127), 16-row boxes, 128-byte swizzle; cached per pool.  False if the driver
 // entry point is missing or the encoding fails.
 bool pool_tensor_maps(const Dev& d, CUtensorMap* lo, CUtensorMap* hi);
-int prefill_tc_smem();
-int prefill_tc_threads();
 int noalloc_max_pairs();
 cudaError_t launch_attn_decode_noalloc(const Dev& d, int layer, const void* q, void* out,
                                        int n_seq, cudaStream_t s);
