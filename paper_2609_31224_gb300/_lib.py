@@ -77,17 +77,16 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
                                vp, ctypes.c_size_t, vp]
     lib.kvc_destroy.argtypes = [vp]
     lib.kvc_destroy.restype = None
-    # (Host int32 lists as addresses: an int, or a pointer from host_i32().)
-    lib.kvc_append_chunk.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp, vp]
+    lib.kvc_append_chunk.argtypes = [vp, ctypes.c_int, p_i32, p_i32, vp, vp, vp, vp]
     lib.kvc_append_kv_layer.argtypes = [vp, ctypes.c_int, vp, vp, vp]
-    lib.kvc_evict.argtypes = [vp, ctypes.c_int, vp, vp, vp]
+    lib.kvc_evict.argtypes = [vp, ctypes.c_int, p_i32, vp, vp]
     lib.kvc_attn_prefill_chunk.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_attn_decode.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_attn_decode_kv.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp]
     lib.kvc_attn_prefill_chunk_kv.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp]
     lib.kvc_attn_decode_noalloc.argtypes = [vp, ctypes.c_int, vp, vp, vp]
     lib.kvc_resident_size.argtypes = [vp, ctypes.c_int, ctypes.POINTER(i64)]
-    lib.kvc_release.argtypes = [vp, ctypes.c_int, vp, vp]
+    lib.kvc_release.argtypes = [vp, ctypes.c_int, p_i32, vp]
     lib.kvc_export_state.argtypes = [vp, ctypes.c_int, ctypes.POINTER(SessionInfo), p_i32, p_i32,
                                      p_i32, ctypes.POINTER(ctypes.c_uint8), p_i32, i64]
     lib.kvc_export_kv.argtypes = [vp, ctypes.c_int, ctypes.c_int, vp, vp, i64]
@@ -97,6 +96,13 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     for name in EXPORTED:
         if name not in ("kvc_destroy", "kvc_last_error"):
             getattr(lib, name).restype = ctypes.c_int
+    # The same entry points with the host int32 lists as addresses, for the methods that make
+    # the lists themselves (_i32): a typed pointer to an array costs more than the call.
+    lib.append_addr, lib.evict_addr, lib.release_addr = (
+        lib["kvc_append_chunk"], lib["kvc_evict"], lib["kvc_release"])
+    lib.append_addr.argtypes = [vp, ctypes.c_int, vp, vp, vp, vp, vp, vp]
+    lib.evict_addr.argtypes = [vp, ctypes.c_int, vp, vp, vp]
+    lib.release_addr.argtypes = [vp, ctypes.c_int, vp, vp]
     _lib = lib
     return lib
 
@@ -107,7 +113,7 @@ def _check(rc: int) -> None:
 
 
 def _i32(a) -> np.ndarray:
-    if type(a) is np.ndarray and a.dtype == np.int32 and a.flags.c_contiguous:
+    if type(a) is np.ndarray and a.dtype == np.int32 and a.ndim == 1 and a.flags.c_contiguous:
         return a
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
@@ -207,9 +213,9 @@ class KVCache:
     # -- hot path -------------------------------------------------------------------
     def append_chunk(self, sessions, cu_tokens, types, k, v, stream=None) -> None:
         s, cu = _i32(sessions), _i32(cu_tokens)
-        _check(self.lib.kvc_append_chunk(self.ctx, len(s), s.ctypes.data, cu.ctypes.data,
-                                         types.data_ptr(), None if k is None else k.data_ptr(),
-                                         None if v is None else v.data_ptr(), _stream(stream)))
+        _check(self.lib.append_addr(self.ctx, len(s), s.ctypes.data, cu.ctypes.data,
+                                    types.data_ptr(), None if k is None else k.data_ptr(),
+                                    None if v is None else v.data_ptr(), _stream(stream)))
 
     def append_kv_layer(self, layer: int, k, v, stream=None) -> None:
         """One layer's K/V [total][Hkv][D] of the last append (after an append without K/V)."""
@@ -223,9 +229,9 @@ class KVCache:
 
     def evict(self, sessions, resident_out=None, stream=None) -> None:
         s = _i32(sessions)
-        _check(self.lib.kvc_evict(self.ctx, len(s), s.ctypes.data,
-                                  None if resident_out is None else resident_out.data_ptr(),
-                                  _stream(stream)))
+        _check(self.lib.evict_addr(self.ctx, len(s), s.ctypes.data,
+                                   None if resident_out is None else resident_out.data_ptr(),
+                                   _stream(stream)))
 
     def attn_prefill_chunk(self, layer: int, q, out, stream=None) -> None:
         _check(self.lib.kvc_attn_prefill_chunk(self.ctx, layer, q.data_ptr(), out.data_ptr(),
@@ -237,7 +243,7 @@ class KVCache:
 
     def release(self, sessions, stream=None) -> None:
         s = _i32(sessions)
-        _check(self.lib.kvc_release(self.ctx, len(s), s.ctypes.data, _stream(stream)))
+        _check(self.lib.release_addr(self.ctx, len(s), s.ctypes.data, _stream(stream)))
 
     # -- synchronising queries -------------------------------------------------------
     def resident_size(self, session: int) -> int:
