@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_prefill_tc_kernel(
           pid_next = page_at(4 * k + 32 + lane);
         }
         const int page = __shfl_sync(FULL, pid, 4 * (k & 7) + pg);
-        if (arrive_first && lane == 0 && mbar_try_wait(&bars[B_PUB], 0)) {
+        if (arrive_first && lane == 0 && mbar_test(&bars[B_PUB], 0)) {
           s_first_last = arrive_acq_rel(&d.pf_count[first_pair], first_nch);
           arrive_first = false;
         }

@@ -19,8 +19,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float RESCALE_LOG2 = 8.f;          // rescale O only when the max grows by > 2^8
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// Bounded wait for two barriers: both are tested first, back to back, so that their latencies
-// overlap when both are ready.
+// Whether a phase is complete, without waiting (mbarrier.try_wait may suspend the thread).
 __device__ inline bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -32,6 +31,8 @@ __device__ inline bool mbar_test(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// Bounded wait for two barriers: both are tested first, back to back, so that their latencies
+// overlap when both are ready.
 __device__ inline bool mbar_wait2(const Dev& d, uint64_t* a, uint32_t pa, uint64_t* b, uint32_t pb) {
   const bool ra = mbar_test(a, pa), rb = mbar_test(b, pb);
   return (ra || mbar_wait(d, a, pa)) && (rb || mbar_wait(d, b, pb));

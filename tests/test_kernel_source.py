@@ -56,3 +56,11 @@ def test_launch_state_is_kept_by_the_context():
             code("kvc_decode_dispatch.cu")
     assert "cudaOccupancyMaxActiveClusters" in code("kvc_attn_prefill_f32.cu")
     assert "query_limits(" in code("kvc_api.cu")
+
+
+def test_only_waits_suspend():
+    """mbarrier.try_wait may suspend the thread for a while, so it stands in bounded waits alone;
+    a look at a phase on the way past it is mbarrier.test_wait."""
+    for name in sorted(os.listdir(CSRC)):
+        for m in re.finditer(r"(.*)mbar_try_wait\(", code(name)):
+            assert re.search(r"if \($|while \(!$|inline bool $", m.group(1)), (name, m.group(0))
