@@ -12,6 +12,7 @@
 //     the rest (e.g. rounds of 30-50 long sessions, and calls of more pairs than the
 //     4-warp shape's resident CTAs, like the full-batch rounds of 64 sessions).
 #include <cstring>
+#include <mutex>
 
 #include "kvc_launch.cuh"
 
@@ -129,16 +130,42 @@ cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const
                                     DEC_MIN_UNITS, new_k, new_v, early, s);
 }
 
+namespace {
+
+struct KnownLimits {
+  unsigned long long ctx_id;
+  int esz;
+  Limits lim;
+};
+constexpr int MAX_KNOWN = 64;
+KnownLimits g_known[MAX_KNOWN];
+int g_n_known = 0;
+std::mutex g_known_mu;
+
+}  // namespace
+
 cudaError_t query_limits(const Dev& d, Limits* lim) {
+  std::lock_guard<std::mutex> lock(g_known_mu);
+  unsigned long long id = 0;
+  cudaError_t e = current_context_id(&id);
+  if (e != cudaSuccess) return e;
+  for (int i = 0; i < g_n_known; ++i)
+    if (g_known[i].ctx_id == id && g_known[i].esz == d.esz) {
+      *lim = g_known[i].lim;
+      return cudaSuccess;
+    }
   memset(lim, 0, sizeof(*lim));
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim->sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   lim->dec_stream_k = decode_stream_k_grid(d);
   lim->dec_wide = decode_split_slots(d.esz, true, lim->sms);
   lim->dec_narrow = decode_split_slots(d.esz, false, lim->sms);
-  return d.esz == 2 ? prefill_tc_limits(lim) : prefill_f32_limits(lim);
+  e = d.esz == 2 ? prefill_tc_limits(lim) : prefill_f32_limits(lim);
+  // A full table only means that later contexts repeat this for every kvc_create.
+  if (e == cudaSuccess && g_n_known < MAX_KNOWN) g_known[g_n_known++] = {id, d.esz, *lim};
+  return e;
 }
 
 }  // namespace kvc

@@ -28,10 +28,9 @@ struct SeqArgsT {
 };
 using SeqArgs = SeqArgsT<MAX_SEQ>;
 
-// What the device runs at once, for each kernel whose launch shape follows from it.  Worked out
-// for the current device when a context is created, which also sets the kernels' attributes
-// there: nothing is kept per thread or process, so that contexts of several devices, and
-// several threads, do not meet one another's.
+// What the device runs at once, for each kernel whose launch shape follows from it.  kvc_create
+// looks it up for the current CUDA context; the first time for a context and element type (about
+// 3 ms) that also sets the kernels' attributes, which belong to the CUDA context too.
 constexpr int PF_MAX_SLICES = 8;  // CTAs of a bfloat16 prefill cluster, at most
 struct Limits {
   int sms;                         // SMs
@@ -42,6 +41,9 @@ struct Limits {
   int f32_cluster[2][2];           // largest cluster of the binary32 prefill: [rows][spread]
 };
 cudaError_t query_limits(const Dev& d, Limits* lim);
+// Id of the current CUDA context (never reused: a context that replaces a destroyed one at the
+// same address has another).
+cudaError_t current_context_id(unsigned long long* id);
 
 cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s);
 // single: every session of the call gets exactly one token (plan and K/V write in

@@ -387,10 +387,13 @@ cudaError_t kernel_per_sm(int* per_sm) {
   return *per_sm > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-cudaError_t setup_for_current_context(NaSetup* out) {
+}  // namespace
+
+cudaError_t current_context_id(unsigned long long* id) {
   static PfnCtxGetCurrent get_current = nullptr;
   static PfnCtxGetId get_id = nullptr;
-  std::lock_guard<std::mutex> lock(g_setup_mu);
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
   cudaError_t e;
   if (!get_current || !get_id) {
     void* f1 = nullptr;
@@ -402,15 +405,24 @@ cudaError_t setup_for_current_context(NaSetup* out) {
   }
   CUcontext ctx = nullptr;
   if (get_current(&ctx) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
-  void* p = nullptr;
   if (!ctx) {
     // No context current on this thread yet: the runtime makes the device's
     // primary context current on this lookup.
+    void* p = nullptr;
     if ((e = cudaGetSymbolAddress(&p, g_noalloc_scratch)) != cudaSuccess) return e;
     if (get_current(&ctx) != CUDA_SUCCESS || !ctx) return cudaErrorDeviceUninitialized;
   }
+  return get_id(ctx, id) == CUDA_SUCCESS ? cudaSuccess : cudaErrorDeviceUninitialized;
+}
+
+namespace {
+
+cudaError_t setup_for_current_context(NaSetup* out) {
+  std::lock_guard<std::mutex> lock(g_setup_mu);
   unsigned long long id = 0;
-  if (get_id(ctx, &id) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
+  cudaError_t e = current_context_id(&id);
+  if (e != cudaSuccess) return e;
+  void* p = nullptr;
   for (int i = 0; i < g_n_setup; ++i)
     if (g_setup[i].ctx_id == id) {
       *out = g_setup[i];

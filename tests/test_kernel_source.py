@@ -37,10 +37,10 @@ def test_aligned_barriers_follow_a_reconvergence(name, calls):
 
 
 def test_launch_state_is_kept_by_the_context():
-    """Kernel attributes, grid and cluster limits belong to a device: nothing of them is kept per
-    thread or process, where a context on another device would find the first one's.  (What is
-    kept: the driver's entry points, the tensor maps of a pool by its address and extent, and the
-    last error's text.)"""
+    """Kernel attributes, grid and cluster limits belong to a CUDA context: nothing of them is kept
+    per thread or process, where a context on another device would find the first one's, but in
+    tables by the CUDA context's id.  (What else is kept: the driver's entry points, the tensor
+    maps of a pool by its address and extent, and the last error's text.)"""
     kept = []
     for name in sorted(os.listdir(CSRC)):
         for line in code(name).splitlines():
@@ -49,13 +49,15 @@ def test_launch_state_is_kept_by_the_context():
                 kept.append((name, m.group(1).strip().split()[0]))
     assert sorted(set(kept)) == [("kvc_api.cu", "std::string"), ("kvc_attn_prefill.cu", "EncodeTiledFn"),
                                  ("kvc_attn_prefill.cu", "PoolMaps"), ("kvc_noalloc.cu", "PfnCtxGetCurrent"),
-                                 ("kvc_noalloc.cu", "PfnCtxGetId")]
+                                 ("kvc_noalloc.cu", "PfnCtxGetId"), ("kvc_noalloc.cu", "std::mutex")]
     for name, setter in (("kvc_attn_prefill_f32.cu", "prefill_f32_limits"),
                          ("kvc_attn_prefill_tc.cu", "prefill_tc_limits")):
         assert "cudaFuncSetAttribute" in code(name) and setter in code("kvc_attn_prefill.cu") + \
             code("kvc_decode_dispatch.cu")
     assert "cudaOccupancyMaxActiveClusters" in code("kvc_attn_prefill_f32.cu")
     assert "query_limits(" in code("kvc_api.cu")
+    table = code("kvc_decode_dispatch.cu")
+    assert "current_context_id(&id)" in table and "g_known[i].ctx_id == id" in table
 
 
 def test_only_waits_suspend():
