@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "kvc_estimate.h"
 #include "kvc_launch.cuh"
 #include "kvc_order.h"
 
@@ -160,6 +161,7 @@ struct kvc_ctx {
   // Host mirrors.
   std::vector<int32_t> tail_mod;  // (live_head + n_live) % PS, exact
   std::vector<int32_t> pos_next;  // exact
+  std::vector<ResidentEstimate> resident;
   int64_t used_ub = 0;            // upper bound of pages in use after enqueued work
   int64_t delta_since_readback = 0;
   bool readback_pending = false;
@@ -169,8 +171,8 @@ struct kvc_ctx {
   // Last append (queries of the following attention calls).
   bool attn_valid = false;
   int last_n_seq = 0, last_total = 0, last_max_t = 0;
-  // Estimates of its sessions' resident pages (largest, sum): what was fed, capped at what the
-  // eviction policy is to keep.  They guide the choice of the attention's split only.
+  // Estimates of its sessions' resident pages (largest, sum), for the choice of the attention's
+  // split only.
   int est_pages_max = 0;
   int64_t est_pages_sum = 0;
   LaunchOrder order;       // of the attention launches since the last append
@@ -293,6 +295,7 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
   layout_meta(*cfg, static_cast<uint8_t*>(d_meta), &d);
   ctx->tail_mod.assign(cfg->n_sessions, 0);
   ctx->pos_next.assign(cfg->n_sessions, 0);
+  ctx->resident.assign(cfg->n_sessions, ResidentEstimate());
   auto cleanup = [&](int code) {
     if (ctx->ev) cudaEventDestroy(ctx->ev);
     if (ctx->h_readback) cudaFreeHost(ctx->h_readback);
@@ -375,15 +378,12 @@ int kvc_append_chunk(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, const i
     const int t = h_cu_tokens[i + 1] - h_cu_tokens[i];
     ctx->tail_mod[sid] = (ctx->tail_mod[sid] + t) % PS;
     ctx->pos_next[sid] += t;
+    ctx->resident[sid].append(t);
   }
-  const int64_t keep = ctx->cfg.policy == KVC_POLICY_SINK_RECENT
-                           ? (int64_t)ctx->cfg.sink + ctx->cfg.recent
-                           : (ctx->cfg.budget >= 0 ? ctx->cfg.budget : INT64_MAX / 2);
   ctx->est_pages_max = 0;
   ctx->est_pages_sum = 0;
   for (int i = 0; i < n_seq; ++i) {
-    const int64_t fed = ctx->pos_next[h_sessions[i]], t = h_cu_tokens[i + 1] - h_cu_tokens[i];
-    const int pages = (int)(std::min(fed, keep + t) / PS + 1);
+    const int pages = (int)(ctx->resident[h_sessions[i]].positions() / PS + 1);
     ctx->est_pages_max = std::max(ctx->est_pages_max, pages);
     ctx->est_pages_sum += pages;
   }
@@ -426,6 +426,7 @@ int kvc_evict(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, int64_t* d_res
   for (int i = 0; i < n_seq; ++i) a.sessions[i] = h_sessions[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, ctx->h_readback, ctx->lim.sms, s));
+  for (int i = 0; i < n_seq; ++i) ctx->resident[h_sessions[i]].evict(ctx->cfg);
   ctx->used_ub += n_seq;  // an evict adds at most one page per session, net
   enqueue_readback(ctx, s);
   ctx->attn_valid = false;
@@ -445,6 +446,7 @@ int kvc_release(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, void* stream
   for (int i = 0; i < n_seq; ++i) {
     ctx->tail_mod[h_sessions[i]] = 0;
     ctx->pos_next[h_sessions[i]] = 0;
+    ctx->resident[h_sessions[i]].release();
   }
   enqueue_readback(ctx, s);
   ctx->attn_valid = false;
