@@ -39,15 +39,15 @@ UNIT = "audio-s/s"
 
 # DRAM bytes per algorithmic byte of the roofline kernel (reads + writes), from one
 # ncu capture of the stream-K kernel on the 64-session, two-layer case (the bench's
-# launch shape; smaller calls may run the pair-split kernel): 1,085.39 MB of traffic
-# (1,082.53 MB read, 2.86 MB written) for a 1,077.10 MB launch.  Valid only while the
+# launch shape; smaller calls may run the pair-split kernel): 1,085.54 MB of traffic
+# (1,082.56 MB read, 2.98 MB written) for a 1,077.10 MB launch.  Valid only while the
 # decode sources hash to the version it was taken on; the roofline's traffic is null
 # otherwise.
-DECODE_TRAFFIC_RATIO = 1085.39 / 1077.10
+DECODE_TRAFFIC_RATIO = 1085.54 / 1077.10
 DECODE_TRAFFIC_SOURCES = ("paper_2609_31224_gb300/csrc/kvc_attn_decode.cu",
                           "paper_2609_31224_gb300/csrc/kvc_decode_common.cuh",
                           "paper_2609_31224_gb300/csrc/kvc_internal.cuh")
-DECODE_TRAFFIC_SHA256 = "3d10ae39fc6f95d5358d2fd8671f631631448302659143c429b91f1c8aff59d7"
+DECODE_TRAFFIC_SHA256 = "9af6bc26c31df9e2d348017e9b6956adf2fc32ab191acb94d7a3413729e4ee93"
 
 
 def code_only(text: str) -> str:

@@ -198,21 +198,44 @@ int check_sessions(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+cudaError_t is_capturing(cudaStream_t s, bool* capturing) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &st);
+  *capturing = e == cudaSuccess && st != cudaStreamCaptureStatusNone;
+  return e;
+}
+
+// Estimates of the pages of the last append's sessions (largest, sum), for the choice of a
+// launch's shape.  A captured launch is replayed when they have grown, so it is shaped for the
+// pages that they come to hold.
+struct PageHint {
+  int max;
+  int64_t sum;
+};
+PageHint page_hint(const kvc_ctx* ctx, bool capturing) {
+  PageHint h = {ctx->est_pages_max, ctx->est_pages_sum};
+  if (capturing) {
+    const kvc_config& c = ctx->cfg;
+    const int64_t most = std::min<int64_t>(ResidentEstimate::kept(c, c.max_positions), c.max_positions);
+    const int settled = std::min<int>(c.max_pages_per_session, (int)(most / PS + 2));
+    h.max = std::max(h.max, settled);
+    h.sum = std::max<int64_t>(h.sum, (int64_t)settled * ctx->last_n_seq);
+  }
+  return h;
+}
+
 // Tag for the next decode launch's partial states, or 0 (fenced arrival) while
 // the stream is being captured: a graph replays a launch with the tag it was
 // captured with, which older words in the slots may carry.  When the counter
 // wraps the slots are cleared first, so no word keeps a tag that comes round again.
-cudaError_t next_decode_epoch(kvc_ctx* ctx, cudaStream_t s, uint32_t* epoch) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(s, &st);
-  if (e != cudaSuccess) return e;
-  if (st != cudaStreamCaptureStatusNone) {
+cudaError_t next_decode_epoch(kvc_ctx* ctx, cudaStream_t s, bool capturing, uint32_t* epoch) {
+  if (capturing) {
     *epoch = 0;
     return cudaSuccess;
   }
   if (++ctx->dec_epoch == 0) {
     const int G = ctx->cfg.q_heads / ctx->cfg.kv_heads;
-    e = cudaMemsetAsync(ctx->d.dec_tagged, 0,
+    const cudaError_t e = cudaMemsetAsync(ctx->d.dec_tagged, 0,
                         (size_t)ctx->d.dec_tag_slots * (G * ctx->cfg.head_dim + 2 * G) * 8, s);
     if (e != cudaSuccess) return e;
     ctx->dec_epoch = 1;
@@ -313,6 +336,7 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
   const cudaError_t le = query_limits(d, &ctx->lim);
   if (le != cudaSuccess)
     return cleanup(fail(KVC_ECUDA, "device query failed: %s", cudaGetErrorString(le)));
+  d.dec_narrow = ctx->lim.dec_narrow;
   *out = ctx;
   return KVC_OK;
 }
@@ -474,10 +498,12 @@ int kvc_attn_decode(kvc_ctx* ctx, int layer, const void* d_q, void* d_out, void*
   if (rc) return rc;
   if (!ctx->last_single)
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
+  bool capturing = false;
+  KVC_CUDA(is_capturing(static_cast<cudaStream_t>(stream), &capturing));
   uint32_t epoch = 0;
-  KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
+  KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), capturing, &epoch));
   KVC_CUDA(launch_attn_decode(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
-                              ctx->est_pages_max, ctx->order.early(layer, false),
+                              page_hint(ctx, capturing).max, ctx->order.early(layer, false),
                               static_cast<cudaStream_t>(stream), epoch));
   ctx->order.launched(layer, false);
   return KVC_OK;
@@ -494,10 +520,12 @@ int kvc_attn_decode_kv(kvc_ctx* ctx, int layer, const void* d_k, const void* d_v
     return fail(KVC_ESTATE, "decode needs exactly one appended token per session");
   // (An early launch may load the page while a launch before it writes the new row's slot:
   // the row goes into the tile after its load.)
+  bool capturing = false;
+  KVC_CUDA(is_capturing(static_cast<cudaStream_t>(stream), &capturing));
   uint32_t epoch = 0;
-  KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), &epoch));
+  KVC_CUDA(next_decode_epoch(ctx, static_cast<cudaStream_t>(stream), capturing, &epoch));
   KVC_CUDA(launch_attn_decode(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
-                              ctx->est_pages_max, ctx->order.early(layer, true),
+                              page_hint(ctx, capturing).max, ctx->order.early(layer, true),
                               static_cast<cudaStream_t>(stream), epoch, d_k, d_v));
   ctx->order.launched(layer, true);
   return KVC_OK;
@@ -527,10 +555,13 @@ int kvc_attn_prefill_chunk(kvc_ctx* ctx, int layer, const void* d_q, void* d_out
   if (rc) return rc;
   if (ctx->last_max_t > PF_MAX_TOKENS)
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  bool capturing = false;
+  KVC_CUDA(is_capturing(s, &capturing));
+  const PageHint pages = page_hint(ctx, capturing);
   KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
-                               ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
-                               ctx->order.early(layer, false),
-                               static_cast<cudaStream_t>(stream)));
+                               ctx->last_max_t, pages.max, pages.sum,
+                               ctx->order.early(layer, false), s));
   ctx->order.launched(layer, false);
   return KVC_OK;
 }
@@ -545,10 +576,13 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
   if (ctx->last_max_t > PF_MAX_TOKENS)
     return fail(KVC_EINVAL, "prefill chunks are limited to %d tokens per session", PF_MAX_TOKENS);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  bool capturing = false;
+  KVC_CUDA(is_capturing(s, &capturing));
+  const PageHint pages = page_hint(ctx, capturing);
   if (ctx->d.esz == 2) {
     // (A stage holding chunk slots is copied only after this launch has written its rows.)
     KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
-                                 ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
+                                 ctx->last_max_t, pages.max, pages.sum,
                                  ctx->order.early(layer, true), s, d_k, d_v));
     ctx->order.launched(layer, true);
   } else {
@@ -556,7 +590,7 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
     KVC_CUDA(launch_append_layers(ctx->d, ctx->last_total, layer, 1, d_k, d_v, false, s));
     ctx->order.layer_write(layer);
     KVC_CUDA(launch_attn_prefill(ctx->d, ctx->lim, layer, d_q, d_out, ctx->last_n_seq,
-                                 ctx->last_max_t, ctx->est_pages_max, ctx->est_pages_sum,
+                                 ctx->last_max_t, pages.max, pages.sum,
                                  ctx->order.early(layer, false), s));
     ctx->order.launched(layer, false);
   }

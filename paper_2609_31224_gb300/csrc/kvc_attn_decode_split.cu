@@ -1,11 +1,12 @@
 // Single-token decode attention, pair-split kernel (calls of few sessions): CTA
-// c takes slice c % k of (session, KV head) pair c / k, the pair's pages cut into
-// k equal slices, so that every page of a small call is in flight at once.  The
+// c takes one slice of one (session, KV head) pair, the pair's pages cut into equal
+// slices, so that every page of a small call is in flight at once.  The
 // bfloat16 pages run on the tensor cores (mma.sync) in both CTA shapes.  With 16
 // warps (one CTA per SM) the partial states are tagged 64-bit words merged after a
 // relaxed arrival; with 4 warps (three CTAs per SM) the acquire-release arrival of
 // stream-K is used.
 #include "kvc_decode_common.cuh"
+#include "kvc_decode_slices.h"
 
 // Shape constants of the CUDA-core loop are unused by the tensor-core shapes.
 #pragma nv_diag_suppress 177
@@ -13,6 +14,8 @@
 namespace kvc {
 
 namespace {
+
+static_assert(SLICES_MAX <= MAX_PARTS, "a merge takes every slice");
 
 // Tagged partial state of slot `slot`: G * D output words, then (m, l) per row.
 template <class C>
@@ -156,21 +159,25 @@ __device__ inline void drain_after_failure(const Dev& d, const Smem<C>& sm, cons
 }
 
 // ---------------------------------------------------------------------------
-// Pair-split kernel (few sessions): CTA c takes slice c % k of pair c / k, the
-// pair's pages cut into k equal slices.  Each CTA's pages are issued before it
-// waits on the previous kernel; the k partial states of a pair are merged by
-// the last of its CTAs to finish.
+// Pair-split kernel (few sessions): a CTA takes one of the k <= k_most equal slices of a pair's
+// pages.  16 warps: k = k_most, the grid is flat.  4 warps: k is the append's count, the grid is
+// (k_most, pairs), so that k's latency is not followed by a division of the block index, and
+// CTAs past k leave at once.  Each CTA's pages are issued before it waits on the previous
+// kernel; the k partial states of
+// a pair are merged by the last of its CTAs to finish.
 // ---------------------------------------------------------------------------
 template <typename T, int D, bool FUSED, class C>
 __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
     Dev d, int layer, const __grid_constant__ CUtensorMap map_lo,
     const __grid_constant__ CUtensorMap map_hi, const T* __restrict__ q, T* __restrict__ out,
-    float qk_scale, int k, uint32_t epoch, int early, const T* new_k, const T* new_v) {
+    float qk_scale, int k_most, uint32_t epoch, int early, const T* new_k, const T* new_v) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Smem<C> sm(smem, warp);
   __shared__ int s_last;
-  const int pair = blockIdx.x / k, slice = blockIdx.x % k;
+  constexpr bool WIDE = C::WARPS == WIDE_WARPS;
+  const int pair = WIDE ? blockIdx.x / k_most : blockIdx.y;
+  const int slice = WIDE ? blockIdx.x % k_most : blockIdx.x;
   const int seq = pair / d.kv_heads, head = pair % d.kv_heads;
   init_warp_barriers<C>(sm.wbars, lane);
   __syncthreads();
@@ -178,6 +185,9 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
   pdl_launch_dependents();
 
   const SeqInfo si = d.seq[seq];
+  // (The append's count is of this call's pairs; a failed append leaves an older call's.)
+  const int k = WIDE ? k_most : max(1, min(si.dec_slices, k_most));
+  if (!WIDE && slice >= k) return;
   const int nb = si.n_blocks;
   const int b0 = (int)((int64_t)slice * nb / k), b1 = (int)((int64_t)(slice + 1) * nb / k);
   Segment<C> sg;
@@ -224,14 +234,14 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
   __syncthreads();
   merge_warps<C>(sm, warp, lane);
   T* orow = out + ((size_t)si.q_row0 * d.q_heads + head * G) * D;
-  const int slot = blockIdx.x;
+  const int slot = WIDE ? blockIdx.x : pair * k_most + slice;
   if (k > 1 && epoch != 0) {
     publish_tagged<C>(d, sm, slot, epoch, tid);
     __syncthreads();
     if (tid == 0) s_last = arrive_relaxed(&d.dec_count[pair], k);
     __syncthreads();
     if (!s_last) return;
-    merge_tagged<C>(d, sm, k, pair * k, epoch, orow, tid, warp, lane);
+    merge_tagged<C>(d, sm, k, pair * k_most, epoch, orow, tid, warp, lane);
     if (tid == 0) d.dec_count[pair] = 0;
     return;
   }
@@ -248,7 +258,7 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
   }
   if (k == 1) return;
   if (!arrive_last(&d.dec_count[pair], k, tid, &s_last)) return;
-  merge_parts<C>(d, sm, k, [&](int ch) { return pair * k + ch; }, orow, tid, warp, lane);
+  merge_parts<C>(d, sm, k, [&](int ch) { return pair * k_most + ch; }, orow, tid, warp, lane);
   if (tid == 0) d.dec_count[pair] = 0;
 }
 
@@ -267,14 +277,15 @@ int split_slots(int sms) {
 
 template <typename T, int D, class C>
 cudaError_t launch_split(const Dev& d, int layer, const CUtensorMap& map_lo,
-                         const CUtensorMap& map_hi, const void* q, void* out, float scale, int k,
-                         uint32_t epoch, const void* new_k, const void* new_v, int n_pairs,
+                         const CUtensorMap& map_hi, const void* q, void* out, float scale,
+                         int k_most, uint32_t epoch, const void* new_k, const void* new_v, int n_pairs,
                          bool early, cudaStream_t s) {
   const bool fused = new_k != nullptr;
   return launch_ex(fused ? &attn_decode_split_kernel<T, D, true, C>
                          : &attn_decode_split_kernel<T, D, false, C>,
-                   dim3(n_pairs * k), dim3(C::THREADS), C::SMEM, s, true, d, layer, map_lo, map_hi,
-                   static_cast<const T*>(q), static_cast<T*>(out), scale, k, epoch, (int)early,
+                   C::WARPS == WIDE_WARPS ? dim3(n_pairs * k_most) : dim3(k_most, n_pairs),
+                   dim3(C::THREADS), C::SMEM, s, true, d, layer, map_lo, map_hi,
+                   static_cast<const T*>(q), static_cast<T*>(out), scale, k_most, epoch, (int)early,
                    static_cast<const T*>(new_k), static_cast<const T*>(new_v));
 }
 
@@ -295,19 +306,19 @@ bool decode_split_uses_tma(int esz, bool wide) {
 
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
-                                     float scale, int k, uint32_t epoch, const void* new_k,
+                                     float scale, int k_most, uint32_t epoch, const void* new_k,
                                      const void* new_v, int n_pairs, bool early, cudaStream_t s) {
   if (d.esz == 2) {
     if (wide)
       return launch_split<__nv_bfloat16, 128, SpCfg<__nv_bfloat16, 128>>(
-          d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, early, s);
+          d, layer, map_lo, map_hi, q, out, scale, k_most, epoch, new_k, new_v, n_pairs, early, s);
     return launch_split<__nv_bfloat16, 128, Sp4Cfg<__nv_bfloat16, 128>>(
-        d, layer, map_lo, map_hi, q, out, scale, k, epoch, new_k, new_v, n_pairs, early, s);
+        d, layer, map_lo, map_hi, q, out, scale, k_most, epoch, new_k, new_v, n_pairs, early, s);
   }
   if (wide)
-    return launch_split<float, 64, SpCfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k,
+    return launch_split<float, 64, SpCfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k_most,
                                                      epoch, new_k, new_v, n_pairs, early, s);
-  return launch_split<float, 64, Sp4Cfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k,
+  return launch_split<float, 64, Sp4Cfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k_most,
                                                     epoch, new_k, new_v, n_pairs, early, s);
 }
 

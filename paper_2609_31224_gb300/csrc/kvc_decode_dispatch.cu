@@ -14,13 +14,13 @@
 #include <cstring>
 #include <mutex>
 
+#include "kvc_decode_slices.h"
 #include "kvc_launch.cuh"
 
 namespace kvc {
 
 namespace {
 
-constexpr int MAX_PARTS = 64;      // partial states per pair (both pair-split shapes)
 constexpr float LOG2E = 1.4426950408889634f;
 // Minimum (session, kv head, page) units per CTA of the stream-K split.
 constexpr int DEC_MIN_UNITS = 12;
@@ -43,7 +43,7 @@ constexpr int DEC_MIN_UNITS = 12;
 // 16.6, 24 pairs 13.9 and 22.3 against 12.4 and 19.0: the 16-warp shape up to a ninth of the
 // SMs.  bfloat16 stays with it up to a sixth, at up to 6 % more for 24 pairs, so that calls
 // of one to three long sessions run one kernel; at 28 pairs the 4-warp shape is 7-12 % faster.
-constexpr int WIDE_WARPS = 16, WIDE_MIN_PAGES = 55;
+constexpr int WIDE_MIN_PAGES = 55;
 constexpr int WIDE_LONG_K = 6, WIDE_LONG_K_F32 = 9, WIDE_LONG_PAGES = 256;
 bool use_wide(int slots, int n_pairs, int pages, int esz) {
   if (pages >= WIDE_LONG_PAGES)
@@ -60,44 +60,6 @@ bool one_slice_too_few(int slots, int n_pairs, int pages) {
   return pages >= STREAM_K_MIN_PAGES && n_pairs <= slots * 7 / 8;
 }
 
-// Slices per pair of the 16-warp shape: 17, which gives 272 pages a warp each, and more for
-// longer sessions (8 pairs of 257 pages: 7.5 us at 17 slices, 8.2 at 19, 8.8 at 15; of 157:
-// 6.9 at 17, 7.1 at 11; 4 pairs of 257: 7.2 at 19, 8.4 at 38).
-int wide_slices(int slots, int n_pairs, int pages) {
-  return min(MAX_PARTS, min(slots / n_pairs, max(17, (pages + 2 + 15) / WIDE_WARPS)));
-}
-
-// ... and of the 4-warp shape (two more pages than estimated: the partly filled ones of both
-// regions).  Up to 5/6 of the slots for as long as that leaves 6 slices or more, all of them
-// beyond (257 pages: 14.5 us at 12 slices of 32 pairs, 15.0 at 14; 18.9 at 8 of 48, 19.6 at 9;
-// but 26.0 at 6 of 72, 26.5 at 5), from 300 pages on as long as it leaves 8 (64 pairs: 39.9 us
-// at 7 slices of 501 pages, 41.4 at 6, but 24.0 and 23.1 of 257); and no more than 14, as the
-// merge is the dearer part beyond (8 pairs of 52 pages: 5.8 us at 14 slices, 6.3 at 16, 6.7 at
-// 18; of 76: 6.5, 7.1, 7.2).
-// bfloat16 takes a page per warp at least, and the fewest slices that leave a warp as few
-// pages (72 pairs of 76 pages: 9.9 us at 5 slices, 10.7 at 6; 32 of 157: 10.2 at 10, 10.7 at
-// 12; 16 of 29: 5.7 at 8, 6.3 at 10).  The CUDA-core pages of binary32 are bound by the pages
-// of a warp: about two pages per slice at least (20 pages, 16 pairs: 4.9 us at 11 slices, 5.2
-// at 8; 24 pairs: 5.0 and 5.2), and more slices if they save a warp one (48 pairs of 130
-// pages: 12.0 us at 9 slices, 12.5 at 8).
-constexpr int NARROW_MAX = 14, NARROW_WARPS = 4, ALL_MIN_PAGES = 300;
-int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
-  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs, all = slots / n_pairs;
-  auto warp_pages = [&](int k) {
-    return ((pages + 2 + k - 1) / k + NARROW_WARPS - 1) / NARROW_WARPS;
-  };
-  const int fit = five_sixths >= (pages < ALL_MIN_PAGES ? 6 : 8) ? five_sixths : all;
-  int k = min(NARROW_MAX, fit);
-  if (cuda_cores) {
-    for (int more = k + 1; more <= min(NARROW_MAX, all); ++more)
-      if (warp_pages(more) < warp_pages(k)) k = more;
-    return max(1, min(k, (pages + 2) / 2));
-  }
-  k = max(1, min(k, (pages + 2 + NARROW_WARPS - 1) / NARROW_WARPS));
-  while (k > 5 && warp_pages(k - 1) == warp_pages(k)) --k;
-  return k;
-}
-
 }  // namespace
 
 cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const void* q,
@@ -107,7 +69,8 @@ cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   const int n_pairs = n_seq * d.kv_heads;
   const int k = use_wide(slots, n_pairs, pages, esz) ? wide_slices(slots, n_pairs, pages) : 0;
-  int k4 = k == 0 && n_pairs <= slots4 ? narrow_slices(slots4, n_pairs, pages, esz == 4) : 0;
+  // As many slices as any number of pages can want: the kernel takes the append's count.
+  int k4 = k == 0 ? narrow_most(slots4, n_pairs) : 0;
   if (k4 == 1 && one_slice_too_few(slots4, n_pairs, pages)) k4 = 0;
   // Tensor maps of the pool for the tensor-core page loop (bfloat16).
   CUtensorMap map_lo, map_hi;
