@@ -47,7 +47,7 @@ DECODE_TRAFFIC_RATIO = 1085.54 / 1077.10
 DECODE_TRAFFIC_SOURCES = ("paper_2609_31224_gb300/csrc/kvc_attn_decode.cu",
                           "paper_2609_31224_gb300/csrc/kvc_decode_common.cuh",
                           "paper_2609_31224_gb300/csrc/kvc_internal.cuh")
-DECODE_TRAFFIC_SHA256 = "9af6bc26c31df9e2d348017e9b6956adf2fc32ab191acb94d7a3413729e4ee93"
+DECODE_TRAFFIC_SHA256 = "0cff2756718fb1d29431bc56a93028e65fa157ee59d0c161bf8ac5f28209e6dd"
 
 
 def code_only(text: str) -> str:

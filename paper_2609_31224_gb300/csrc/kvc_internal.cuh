@@ -100,8 +100,8 @@ struct Dev {
   float2* dec_part_ml;         // [dec_slots][G] (m, l) in log2 units
   unsigned long long* dec_tagged;  // [dec_tag_slots][G * D + 2 G] tagged partial states
   int32_t dec_tag_slots;
-  float* pf_part_o;            // [pf_slots][D / 4][PF_ROWS][4]
-  float2* pf_part_ml;          // [pf_slots][PF_ROWS]
+  float* pf_part_o;            // [pf_slots][D / 4][128 query rows][4]
+  float2* pf_part_ml;          // [pf_slots][128]
   int32_t* dec_count;          // [max_seq * kv_heads] arrival counters
   int32_t* pf_count;           // [max_seq * kv_heads]
 };
@@ -327,17 +327,6 @@ __device__ inline void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t b
       : "memory");
 }
 
-// 2-D tensor copy (TMA engine) of the box at column x, row y of `map` into
-// shared memory, completing on `bar`.
-__device__ inline void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
-                                   uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-
 // L2 cache policy for data read once per launch: replaced first, so that what is read again
 // (queries, rotary rows, partial states) stays.
 __device__ inline uint64_t evict_first_policy() {
@@ -345,6 +334,8 @@ __device__ inline uint64_t evict_first_policy() {
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+// 2-D tensor copy (TMA engine) of the box at column x, row y of `map` into shared memory,
+// completing on `bar`, with that policy.
 __device__ inline void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y,
                                         uint64_t* bar, uint64_t policy) {
   asm volatile(

@@ -46,7 +46,7 @@ cudaError_t query_limits(const Dev& d, Limits* lim);
 cudaError_t current_context_id(unsigned long long* id);
 
 cudaError_t launch_init(const Dev& d, double rope_base, cudaStream_t s);
-// single: every session of the call gets exactly one token (plan and K/V write in
+// single: every session of the call gets exactly one token (one session: plan and K/V write in
 // one launch).
 cudaError_t launch_append(const Dev& d, const AppendArgs& a, const uint8_t* types, const void* k,
                           const void* v, bool single, cudaStream_t s);

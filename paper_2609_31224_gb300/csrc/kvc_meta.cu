@@ -981,7 +981,6 @@ __global__ void __launch_bounds__(256) evict_copy_kernel(Dev d) {
   const int vec_per_row = d.head_dim * d.esz / 16;
   const int rows_per_move = d.layers * 2 * d.kv_heads;
   const int64_t total = (int64_t)n_moves * rows_per_move * vec_per_row;
-  const size_t row_bytes = (size_t)d.head_dim * d.esz;
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < total;
        u += (int64_t)gridDim.x * blockDim.x) {
     const int v = (int)(u % vec_per_row);
@@ -996,7 +995,6 @@ __global__ void __launch_bounds__(256) evict_copy_kernel(Dev d) {
     const size_t dof = pool_offset_elems(d, mv.y / PS, l, kv, h, mv.y % PS) * d.esz;
     const uint4 x = *reinterpret_cast<const uint4*>(d.pool + so + (size_t)v * 16);
     *reinterpret_cast<uint4*>(d.pool + dof + (size_t)v * 16) = x;
-    (void)row_bytes;
   }
 }
 
