@@ -35,7 +35,7 @@ CASES = {
     "8 pairs, 64 pages": (8, [1023], -1),
     "8 pairs, 101 pages": (8, [1610], -1),
     "16 pairs, 7 and 110 pages": (8, [100, 1760], -1),
-    "8 pairs, 54 pages": (8, [863], -1),
+    "8 pairs, 54 pages": (8, [862], -1),
     "8 pairs, 55 pages": (8, [864], -1),
     "8 pairs, 300 pages": (8, [4800], -1),
     "12 pairs, 190 pages": (4, [3030, 70, 3000], -1),
