@@ -110,16 +110,15 @@ std::mutex g_known_mu;
 cudaError_t query_limits(const Dev& d, Limits* lim) {
   std::lock_guard<std::mutex> lock(g_known_mu);
   unsigned long long id = 0;
-  cudaError_t e = current_context_id(&id);
-  if (e != cudaSuccess) return e;
-  for (int i = 0; i < g_n_known; ++i)
+  const bool known = current_context_id(&id) == cudaSuccess;  // (else worked out each time)
+  for (int i = 0; known && i < g_n_known; ++i)
     if (g_known[i].ctx_id == id && g_known[i].esz == d.esz) {
       *lim = g_known[i].lim;
       return cudaSuccess;
     }
   memset(lim, 0, sizeof(*lim));
   int dev = 0;
-  e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim->sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   lim->dec_stream_k = decode_stream_k_grid(d);
@@ -127,7 +126,7 @@ cudaError_t query_limits(const Dev& d, Limits* lim) {
   lim->dec_narrow = decode_split_slots(d.esz, false, lim->sms);
   e = d.esz == 2 ? prefill_tc_limits(lim) : prefill_f32_limits(lim);
   // A full table only means that later contexts repeat this for every kvc_create.
-  if (e == cudaSuccess && g_n_known < MAX_KNOWN) g_known[g_n_known++] = {id, d.esz, *lim};
+  if (e == cudaSuccess && known && g_n_known < MAX_KNOWN) g_known[g_n_known++] = {id, d.esz, *lim};
   return e;
 }
 

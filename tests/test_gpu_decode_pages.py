@@ -1,5 +1,5 @@
-"""Decode calls whose sessions hold other numbers of pages than the host expects when it launches:
-launches captured with short sessions and replayed on long ones, and sessions of text that a
+"""Calls whose sessions hold other numbers of pages than the host expects when it launches them:
+decode and prefill captured with short sessions and replayed on long ones, and sessions of text that a
 small budget cannot shorten.  Against the same call launched anew, and on an unbounded cache.
 """
 import numpy as np
@@ -48,33 +48,36 @@ class Sessions:
                                 self.rand(1, self.n * m, HEADS, self.D),
                                 self.rand(1, self.n * m, HEADS, self.D))
 
-    def buffers(self):
-        return (self.rand(self.n, 4 * HEADS, self.D),
-                torch.full((self.n, 4 * HEADS, self.D), float("nan"), dtype=self.t, device="cuda"))
+    def buffers(self, tokens=1):
+        shape = (self.n * tokens, 4 * HEADS, self.D)
+        return (self.rand(*shape),
+                torch.full(shape, float("nan"), dtype=self.t, device="cuda"))
 
 
-@pytest.mark.parametrize("n,grown", [(1, 20), (1, 3000), (3, 900), (6, 2100), (40, 600)])
+@pytest.mark.parametrize("n,grown", [(1, 20), (1, 3000), (3, 900), (6, 2100), (20, 700), (40, 600)])
+@pytest.mark.parametrize("tokens", [1, 17])
 @pytest.mark.parametrize("budget", [-1, 256])
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
-def test_captured_short_replayed_long(n, grown, budget, dtype):
-    s = Sessions(n, dtype, budget, grown + 2)
-    q, out = s.buffers()
+def test_captured_short_replayed_long(n, grown, tokens, budget, dtype):
+    s = Sessions(n, dtype, budget, grown + 2 * tokens)
+    attend = s.cache.attn_decode if tokens == 1 else s.cache.attn_prefill_chunk
+    q, out = s.buffers(tokens)
     fresh = torch.empty_like(out)
-    s.feed(1, ACOUSTIC)
-    s.cache.attn_decode(0, q, out)
+    s.feed(tokens, ACOUSTIC)
+    attend(0, q, out)
     torch.cuda.synchronize()
     g, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
     with torch.cuda.graph(g, stream=stream):
-        s.cache.attn_decode(0, q, out, stream=stream)
+        attend(0, q, out, stream=stream)
     for m in (0, grown):
         if m:
             s.feed(m, TEXT)
             s.cache.evict(np.arange(n))
-            s.feed(1, TEXT)
+            s.feed(tokens, TEXT)
         out.fill_(float("nan"))
         g.replay()
         torch.cuda.synchronize()
-        s.cache.attn_decode(0, q, fresh)
+        attend(0, q, fresh)
         assert s.cache.device_status()[1] == 0
         assert_close(out.float().cpu().numpy(), fresh.float().cpu().numpy(), dtype, f"{m} grown")
     del g
