@@ -238,8 +238,9 @@ int kvc_attn_prefill_chunk_kv(kvc_ctx* ctx, int layer, const void* d_k, const vo
  * rounded to bfloat16 and binary32 accumulation and softmax, in every call size;
  * binary32 calls run on CUDA cores in binary32.  The split of a session's pages
  * over CTAs (and so the order of the partial sums) depends on how many sessions
- * share its call, so its output can differ in the last bits with that number;
- * both stay within the attention tolerance.
+ * share its call, on the pages they hold or are expected to hold, and on whether
+ * the launch is captured, so its output can differ in the last bits with those; all
+ * stay within the attention tolerance.
  *   d_q     device [n_seq][Hq][D] un-rotated queries (call order of the append)
  *   d_out   device [n_seq][Hq][D]
  * May be captured into a CUDA graph: a launch made while `stream` is capturing

@@ -11,8 +11,8 @@
 // The k slices of a pair are a thread-block cluster: each CTA leaves its partial rows
 // (O, max, sum) in shared memory and merges its share of them from all k.
 // Measured per launch with 17-token chunks: 4 sessions x 8 heads x 1,040 positions 26.5 us
-// (0.29 GFMA; 7.5 us at the FMA peak: with two warps per scheduler the FMA pipe is busy half
-// of the time), one session x 1 head x 520 positions 9.7 us; before,
+// (0.29 GFMA; 7.5 us at the FMA peak: the FMA pipe is busy 45 % of the time on the SMs with two
+// CTAs, two warps per scheduler, and a third of it over all), one session x 1 head x 520 positions 9.7 us; before,
 // with a thread per row and chunks merged through global memory by one CTA, 96.7 and 55 us.
 #include <type_traits>
 

@@ -7,7 +7,8 @@
 //     tensor cores;
 //   - pair split, 4-warp CTAs (three per SM, tensor-core pages for bfloat16): every
 //     other call whose pairs each get k >= 1 CTAs in one wave (with k = 1 a pair needs no
-//     merge), unless one slice each would leave many slots empty for long;
+//     merge), unless one slice each would leave many slots empty for long; k follows the
+//     pages on the device (kvc_decode_slices.h);
 //   - stream-K over (session, KV head, page) units, tensor-core pages for bfloat16:
 //     the rest (e.g. rounds of 30-50 long sessions, and calls of more pairs than the
 //     4-warp shape's resident CTAs, like the full-batch rounds of 64 sessions).
