@@ -39,15 +39,15 @@ UNIT = "audio-s/s"
 
 # DRAM bytes per algorithmic byte of the roofline kernel (reads + writes), from one
 # ncu capture of the stream-K kernel on the 64-session, two-layer case (the bench's
-# launch shape; smaller calls may run the pair-split kernel): 1,085.54 MB of traffic
-# (1,082.56 MB read, 2.98 MB written) for a 1,077.10 MB launch.  Valid only while the
+# launch shape; smaller calls may run the pair-split kernel): 1,085.39 MB of traffic
+# (1,082.53 MB read, 2.86 MB written) for a 1,077.10 MB launch.  Valid only while the
 # decode sources hash to the version it was taken on; the roofline's traffic is null
 # otherwise.
-DECODE_TRAFFIC_RATIO = 1085.54 / 1077.10
+DECODE_TRAFFIC_RATIO = 1085.39 / 1077.10
 DECODE_TRAFFIC_SOURCES = ("paper_2609_31224_gb300/csrc/kvc_attn_decode.cu",
                           "paper_2609_31224_gb300/csrc/kvc_decode_common.cuh",
                           "paper_2609_31224_gb300/csrc/kvc_internal.cuh")
-DECODE_TRAFFIC_SHA256 = "0cff2756718fb1d29431bc56a93028e65fa157ee59d0c161bf8ac5f28209e6dd"
+DECODE_TRAFFIC_SHA256 = "c9c9528b173f8ebb621008bba3afd216411902b927e36e88c54e753999b1705a"
 
 
 def code_only(text: str) -> str:

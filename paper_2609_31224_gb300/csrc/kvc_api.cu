@@ -336,7 +336,6 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
   const cudaError_t le = query_limits(d, &ctx->lim);
   if (le != cudaSuccess)
     return cleanup(fail(KVC_ECUDA, "device query failed: %s", cudaGetErrorString(le)));
-  d.dec_narrow = ctx->lim.dec_narrow;
   *out = ctx;
   return KVC_OK;
 }

@@ -15,7 +15,6 @@
 #include <cstring>
 #include <mutex>
 
-#include "kvc_decode_slices.h"
 #include "kvc_launch.cuh"
 
 namespace kvc {
@@ -69,27 +68,28 @@ cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const
   const int esz = d.esz, slots = lim.dec_wide, slots4 = lim.dec_narrow;
   const float scale = LOG2E / sqrtf((float)d.head_dim);
   const int n_pairs = n_seq * d.kv_heads;
-  const int k = use_wide(slots, n_pairs, pages, esz) ? wide_slices(slots, n_pairs, pages) : 0;
-  // As many slices as any number of pages can want: the kernel takes the append's count.
-  int k4 = k == 0 ? narrow_most(slots4, n_pairs) : 0;
-  if (k4 == 1 && one_slice_too_few(slots4, n_pairs, pages)) k4 = 0;
+  const bool wide = use_wide(slots, n_pairs, pages, esz);
+  const int most = n_pairs <= slots4 ? narrow_most(slots4, n_pairs) : 0;
+  const bool narrow = !wide && most > 0 && !(most == 1 && one_slice_too_few(slots4, n_pairs, pages));
   // Tensor maps of the pool for the tensor-core page loop (bfloat16).
   CUtensorMap map_lo, map_hi;
   memset(&map_lo, 0, sizeof(map_lo));
   memset(&map_hi, 0, sizeof(map_hi));
   // (The stream-K kernel's bfloat16 pages also run on the tensor cores.)
-  if (((k > 0 && decode_split_uses_tma(esz, true)) ||
-       (k4 > 0 && decode_split_uses_tma(esz, false)) || (k == 0 && k4 == 0 && esz == 2)) &&
+  if (((wide && decode_split_uses_tma(esz, true)) || (narrow && decode_split_uses_tma(esz, false)) ||
+       (!wide && !narrow && esz == 2)) &&
       !pool_tensor_maps(d, &map_lo, &map_hi))
     return cudaErrorInvalidValue;
-  if (k > 0) {
-    const uint32_t tag = n_pairs * k <= d.dec_tag_slots ? epoch : 0u;
-    return launch_attn_decode_split(d, true, layer, map_lo, map_hi, q, out, scale, k, tag, new_k,
+  if (wide) {
+    const SliceCut cut = wide_cut(slots, n_pairs, pages);
+    const uint32_t tag = n_pairs * cut.k <= d.dec_tag_slots ? epoch : 0u;
+    return launch_attn_decode_split(d, true, layer, map_lo, map_hi, q, out, scale, cut, tag, new_k,
                                     new_v, n_pairs, early, s);
   }
-  if (k4 > 0)
-    return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale, k4, 0u, new_k,
-                                    new_v, n_pairs, early, s);
+  if (narrow)
+    return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale,
+                                    narrow_cut(slots4, n_pairs, pages, esz == 4), 0u, new_k, new_v,
+                                    n_pairs, early, s);
   return launch_attn_decode_streamk(d, layer, map_lo, map_hi, q, out, scale, lim.dec_stream_k,
                                     DEC_MIN_UNITS, new_k, new_v, early, s);
 }

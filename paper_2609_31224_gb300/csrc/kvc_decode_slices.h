@@ -1,9 +1,11 @@
 // Slices per (session, KV head) pair of the two pair-split decode shapes, by the pages of the
-// call's longest session.  Those of the 4-warp shape range from 1 to 14, so the append kernels
-// work them out from the page lists they write; the host launches as many CTAs as any number of
-// pages can want, and those past the slices leave at once.  So a launch that was captured with
-// short sessions, or one whose sessions the host estimates wrong, is cut for the pages that are
-// there (8 pairs captured at one page and replayed at 250: 48.2 us with the host's slices).
+// call's longest session.  Those of the 4-warp shape range from 1 to 14.  The host launches as
+// many CTAs as any number of pages can want, with the count for its estimate of the pages; a
+// kernel that finds other pages (nb_max of the append) works the count out again, and CTAs past
+// it leave at once.  So a launch that was captured with short sessions, or one whose sessions the
+// host estimates wrong, is cut for the pages that are there (8 pairs captured at one page and
+// replayed at 250: 48.2 us with the host's count).  That an append kernel works the count out
+// instead costs each of them 0.3 us.
 // Those of the 16-warp shape hardly depend on the pages: they are the host's, as CTAs without a
 // slice would keep the next launch's off their SM (8 pairs of 257 pages: 7.5 us with 17 slices
 // launched, 7.9 with 19 of which 17 work).  Plain C++ beside CUDA, so that it is tested on the CPU.
@@ -23,7 +25,7 @@ constexpr int NARROW_MAX = 14, ALL_MIN_PAGES = 300;
 
 KVC_HD inline int at_most(int a, int b) { return a < b ? a : b; }
 KVC_HD inline int at_least(int a, int b) { return a > b ? a : b; }
-KVC_HD inline int div_up(int a, int b) { return (a + b - 1) / b; }
+KVC_HD inline int div_up(int a, int b) { return ((unsigned)a + b - 1) / (unsigned)b; }  // a, b > 0
 
 // The most slices of a call with n_pairs pairs, whatever its pages (slots: CTAs in one wave).
 KVC_HD inline int narrow_most(int slots, int n_pairs) { return at_most(NARROW_MAX, slots / n_pairs); }
@@ -47,20 +49,50 @@ KVC_HD inline int wide_slices(int slots, int n_pairs, int pages) {
 // of a warp: about two pages per slice at least (20 pages, 16 pairs: 4.9 us at 11 slices, 5.2
 // at 8; 24 pairs: 5.0 and 5.2), and more slices if they save a warp one (48 pairs of 130
 // pages: 12.0 us at 9 slices, 12.5 at 8).
-KVC_HD inline int narrow_slices(int slots, int n_pairs, int pages, bool cuda_cores) {
+//
+// What follows from the pairs alone is the host's part, so that a kernel is left with two divisions.
+struct NarrowFit {
+  int most;         // slices that the slots and NARROW_MAX allow
+  int below, from;  // of sessions below, and from, ALL_MIN_PAGES pages on
+};
+KVC_HD inline NarrowFit narrow_fit(int slots, int n_pairs) {
   const int most = narrow_most(slots, n_pairs);
-  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs;
+  const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs, some = at_most(most, five_sixths);
+  return {most, five_sixths >= 6 ? some : most, five_sixths >= 8 ? some : most};
+}
+KVC_HD inline int narrow_slices(const NarrowFit& fit, int pages, bool cuda_cores) {
+  if (fit.most < 1) return 1;
   const int n = pages + 2;  // (the figures above are of sessions whose first and last are partly filled)
-  int k = five_sixths >= (pages < ALL_MIN_PAGES ? 6 : 8) ? at_most(most, five_sixths) : most;
-  if (k < 1) return 1;
-  auto warp_pages = [&](int slices) { return div_up(div_up(n, slices), NARROW_WARPS); };
+  int k = pages < ALL_MIN_PAGES ? fit.below : fit.from;
+  // Pages of a warp: ceil(ceil(n / k) / NARROW_WARPS).
   if (cuda_cores) {
-    const int w = warp_pages(most);
-    if (w < warp_pages(k)) k = div_up(n, NARROW_WARPS * w);
+    const int w = div_up(n, NARROW_WARPS * fit.most);
+    if (w < div_up(n, NARROW_WARPS * k)) k = div_up(n, NARROW_WARPS * w);
     return at_least(1, at_most(k, n / 2));
   }
   k = at_least(1, at_most(k, div_up(n, NARROW_WARPS)));
-  return k > 5 ? at_least(5, div_up(n, NARROW_WARPS * warp_pages(k))) : k;
+  return k > 5 ? at_least(5, div_up(n, NARROW_WARPS * div_up(n, NARROW_WARPS * k))) : k;
+}
+
+// How a launch of a pair split is cut: `most` CTAs per pair, of which k work while the call's
+// longest session has lo to hi pages (16 warps: most = k, any number).
+struct SliceCut {
+  NarrowFit fit;
+  int most, k, lo, hi;
+};
+inline SliceCut wide_cut(int slots, int n_pairs, int pages) {
+  const int k = wide_slices(slots, n_pairs, pages);
+  return {{k, k, k}, k, k, 0, 1 << 30};
+}
+// `pages` estimated; a quarter and two pages more or less are not worth another count.
+inline SliceCut narrow_cut(int slots, int n_pairs, int pages, bool cuda_cores) {
+  const NarrowFit fit = narrow_fit(slots, n_pairs);
+  return {fit, fit.most, narrow_slices(fit, pages, cuda_cores), pages - pages / 4 - 2,
+          pages + pages / 4 + 2};
+}
+KVC_HD inline int cut_slices(const SliceCut& c, int pages, bool cuda_cores) {
+  const int k = pages < c.lo || pages > c.hi ? narrow_slices(c.fit, pages, cuda_cores) : c.k;
+  return at_least(1, at_most(k, c.most));
 }
 
 }  // namespace kvc

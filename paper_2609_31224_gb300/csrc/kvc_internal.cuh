@@ -47,8 +47,7 @@ struct SeqInfo {
   int32_t n_blocks;     // n_hist_pages + n_live_pages
   int32_t pad0;
   int32_t unit_base;    // first (session, kv head, page) unit of this session
-  int32_t dec_slices;   // slices per pair of the call in the 4-warp decode (single-token appends)
-  int32_t pad[4];
+  int32_t pad[5];
 };
 static_assert(sizeof(SeqInfo) == 64, "SeqInfo size");
 
@@ -78,7 +77,6 @@ struct Dev {
   int32_t max_moves;
   int32_t dec_slots;           // decode partial slots (two per CTA of a split)
   int32_t pf_slots;            // prefill partial slots (two per CTA of a split; bfloat16)
-  int32_t dec_narrow;          // CTAs of the 4-warp pair-split decode in one wave
   // memory
   uint8_t* pool;
   SessState* sess;

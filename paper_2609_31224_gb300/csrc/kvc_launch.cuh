@@ -2,6 +2,7 @@
 // argument blocks they pass by value.
 #pragma once
 
+#include "kvc_decode_slices.h"
 #include "kvc_internal.cuh"
 
 namespace kvc {
@@ -83,8 +84,9 @@ int decode_split_slots(int esz, bool wide, int sms);
 bool decode_split_uses_tma(int esz, bool wide);      // needs the pool's tensor maps
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
-                                     float scale, int k_most, uint32_t epoch, const void* new_k,
-                                     const void* new_v, int n_pairs, bool early, cudaStream_t s);
+                                     float scale, const SliceCut& cut, uint32_t epoch,
+                                     const void* new_k, const void* new_v, int n_pairs, bool early,
+                                     cudaStream_t s);
 // new_k / new_v (optional, bfloat16 only): the chunk's rows of this layer, written
 // into the pool by the launch itself (the per-layer order).
 // pages_max, pages_sum: estimates of the sessions' resident pages (largest, sum over the

@@ -6,7 +6,6 @@
 // session order then token order (append) or session order (evict: all
 // sessions' compacted-region pages are allocated before any live page is
 // freed).  This makes page tables a deterministic function of the calls.
-#include "kvc_decode_slices.h"
 #include "kvc_launch.cuh"
 #include "kvc_rope.cuh"
 
@@ -547,13 +546,12 @@ __global__ void __launch_bounds__(META_THREADS) append_few_kernel(Dev d, SeqArgs
         const int y = __shfl_up_sync(FULL, units, o);
         if (lane >= o) units += y;
       }
-      const int nb_max = __reduce_max_sync(FULL, nb);
       if (in) {
         si.unit_base = units - nb * H;
-        si.dec_slices = narrow_slices(d.dec_narrow, n_seq * H, nb_max, sizeof(T) == 4);
         d.seq[lane] = si;
       }
       const int total_units = __shfl_sync(FULL, units, 31);
+      const int nb_max = __reduce_max_sync(FULL, nb);
       if (lane == 0) {
         d.g->n_seq = n_seq;
         d.g->total_tokens = n_seq;
@@ -678,7 +676,6 @@ __global__ void __launch_bounds__(META_THREADS) append_many_kernel(Dev d, Append
   const int nb_max = block_max(i < n_seq ? nb : 0, s_warp);
   if (i < n_seq) {
     si.unit_base = ubase;
-    si.dec_slices = narrow_slices(d.dec_narrow, n_seq * d.kv_heads, nb_max, d.esz == 4);
     d.seq[i] = si;
   }
   __syncthreads();

@@ -1,6 +1,6 @@
 """Slices per pair of the pair-split decode (csrc/kvc_decode_slices.h), over every number of pairs
-and pages: the rule in closed form, as the append kernels evaluate it, against the rule as a
-search, and within what the host launches and the buffers hold.
+and pages: the rule in closed form, as the kernels evaluate it, against the rule as a search,
+and a launch's slices for pages other than the host's estimate within what it launches.
 """
 import os
 import subprocess
@@ -33,7 +33,7 @@ int main() {
     for (int n_pairs = 1; n_pairs <= 3 * sms; ++n_pairs)
       for (int pages = 1; pages <= 1100; ++pages) {
         for (int cc = 0; cc < 2; ++cc) {
-          const int k = narrow_slices(3 * sms, n_pairs, pages, cc);
+          const int k = narrow_slices(narrow_fit(3 * sms, n_pairs), pages, cc);
           if (k != narrow_search(3 * sms, n_pairs, pages, cc) || k < 1 ||
               k > narrow_most(3 * sms, n_pairs)) {
             std::printf("4 warps, %d SMs, %d pairs, %d pages: %d\n", sms, n_pairs, pages, k);
@@ -48,10 +48,24 @@ int main() {
           return 1;
         }
       }
-    // More pairs than slots: not launched, but every append evaluates it.
-    if (narrow_slices(3 * sms, 3 * sms + 1, 5, false) != 1) return 2;
+    for (int n_pairs : {1, 2, 8, 16, 24, 48, 72, 100, 160, 320, 456})
+      for (int est = 1; est <= 700; est += est < 40 ? 1 : 13)
+        for (int pages = 1; pages <= 700; pages += pages < 40 ? 1 : 7)
+          for (int cc = 0; cc < 2 && n_pairs <= 3 * sms; ++cc) {
+            const SliceCut c = narrow_cut(3 * sms, n_pairs, est, cc);
+            const int k = cut_slices(c, pages, cc);
+            const bool near = 4 * pages >= 3 * est - 12 && 4 * pages <= 5 * est + 8;
+            const int here = narrow_slices(c.fit, pages, cc), there = narrow_slices(c.fit, est, cc);
+            if (c.most != narrow_most(3 * sms, n_pairs) || k < 1 || k > c.most ||
+                (!near && k != here) || (pages == est && k != there) || (k != here && k != there)) {
+              std::printf("%d SMs, %d pairs, %d pages for %d: %d\n", sms, n_pairs, pages, est, k);
+              return 2;
+            }
+          }
+    const SliceCut w = wide_cut(sms, 1, 300);
+    if (w.most != w.k || cut_slices(w, 1, false) != w.k || cut_slices(w, 1 << 20, true) != w.k) return 3;
   }
-  return narrow_slices(0, 1, 1, true) == 1 ? 0 : 3;
+  return 0;
 }
 """
 
