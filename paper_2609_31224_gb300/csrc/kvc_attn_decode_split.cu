@@ -19,9 +19,9 @@ namespace {
 
 static_assert(SLICES_MAX <= MAX_PARTS, "a merge takes every slice");
 
-// What a kernel of shape C is told of its slices: 16 warps their number.
+// What a kernel of shape C is told of its slices: 16 warps their number, 4 warps how to count.
 template <class C>
-using CutOf = std::conditional_t<C::WARPS == WIDE_WARPS, int, SliceCut>;
+using CutOf = std::conditional_t<C::WARPS == WIDE_WARPS, int, NarrowFit>;
 
 // Tagged partial state of slot `slot`: G * D output words, then (m, l) per row.
 template <class C>
@@ -166,9 +166,9 @@ __device__ inline void drain_after_failure(const Dev& d, const Smem<C>& sm, cons
 
 // ---------------------------------------------------------------------------
 // Pair-split kernel (few sessions): a CTA takes one of the k <= k_most equal slices of a pair's
-// pages.  16 warps: k = k_most, the grid is flat.  4 warps: k follows the pages (SliceCut), the
-// grid is (k_most, pairs), so that k's latency is not followed by a division of the block index,
-// and CTAs past k leave at once.  Each CTA's pages are issued before it waits on the previous
+// pages.  16 warps: k = k_most, the grid is flat.  4 warps: k follows the pages, the grid
+// is (k_most, pairs), so that the count is not followed by a division of the block index, and
+// CTAs past k leave at once.  Each CTA's pages are issued before it waits on the previous
 // kernel; the k partial states of
 // a pair are merged by the last of its CTAs to finish.
 // ---------------------------------------------------------------------------
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
 
   const SeqInfo si = d.seq[seq];
   int k = k_most;
-  if constexpr (!WIDE) k = cut_slices(cut, d.g->nb_max, sizeof(T) == 4);
+  if constexpr (!WIDE) k = narrow_slices(cut, d.g->nb_max, sizeof(T) == 4);
   if (!WIDE && slice >= k) return;
   const int nb = si.n_blocks;
   const int b0 = (int)((int64_t)slice * nb / k), b1 = (int)((int64_t)(slice + 1) * nb / k);
@@ -287,15 +287,15 @@ int split_slots(int sms) {
 template <typename T, int D, class C>
 cudaError_t launch_split(const Dev& d, int layer, const CUtensorMap& map_lo,
                          const CUtensorMap& map_hi, const void* q, void* out, float scale,
-                         const SliceCut& cut, uint32_t epoch, const void* new_k,
+                         int k_most, const NarrowFit& fit, uint32_t epoch, const void* new_k,
                          const void* new_v, int n_pairs, bool early, cudaStream_t s) {
   const bool fused = new_k != nullptr;
   CutOf<C> told;
-  if constexpr (C::WARPS == WIDE_WARPS) told = cut.most;
-  else told = cut;
+  if constexpr (C::WARPS == WIDE_WARPS) told = k_most;
+  else told = fit;
   return launch_ex(fused ? &attn_decode_split_kernel<T, D, true, C>
                          : &attn_decode_split_kernel<T, D, false, C>,
-                   C::WARPS == WIDE_WARPS ? dim3(n_pairs * cut.most) : dim3(cut.most, n_pairs),
+                   C::WARPS == WIDE_WARPS ? dim3(n_pairs * k_most) : dim3(k_most, n_pairs),
                    dim3(C::THREADS), C::SMEM, s, true, d, layer, map_lo, map_hi,
                    static_cast<const T*>(q), static_cast<T*>(out), scale, told, epoch, (int)early,
                    static_cast<const T*>(new_k), static_cast<const T*>(new_v));
@@ -318,21 +318,21 @@ bool decode_split_uses_tma(int esz, bool wide) {
 
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
-                                     float scale, const SliceCut& cut, uint32_t epoch,
-                                     const void* new_k, const void* new_v, int n_pairs, bool early,
-                                     cudaStream_t s) {
+                                     float scale, int k_most, const NarrowFit& fit,
+                                     uint32_t epoch, const void* new_k, const void* new_v,
+                                     int n_pairs, bool early, cudaStream_t s) {
   if (d.esz == 2) {
     if (wide)
       return launch_split<__nv_bfloat16, 128, SpCfg<__nv_bfloat16, 128>>(
-          d, layer, map_lo, map_hi, q, out, scale, cut, epoch, new_k, new_v, n_pairs, early, s);
+          d, layer, map_lo, map_hi, q, out, scale, k_most, fit, epoch, new_k, new_v, n_pairs, early, s);
     return launch_split<__nv_bfloat16, 128, Sp4Cfg<__nv_bfloat16, 128>>(
-        d, layer, map_lo, map_hi, q, out, scale, cut, epoch, new_k, new_v, n_pairs, early, s);
+        d, layer, map_lo, map_hi, q, out, scale, k_most, fit, epoch, new_k, new_v, n_pairs, early, s);
   }
   if (wide)
-    return launch_split<float, 64, SpCfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, cut,
-                                                     epoch, new_k, new_v, n_pairs, early, s);
-  return launch_split<float, 64, Sp4Cfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, cut,
-                                                    epoch, new_k, new_v, n_pairs, early, s);
+    return launch_split<float, 64, SpCfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k_most,
+                                                     fit, epoch, new_k, new_v, n_pairs, early, s);
+  return launch_split<float, 64, Sp4Cfg<float, 64>>(d, layer, map_lo, map_hi, q, out, scale, k_most,
+                                                    fit, epoch, new_k, new_v, n_pairs, early, s);
 }
 
 }  // namespace kvc

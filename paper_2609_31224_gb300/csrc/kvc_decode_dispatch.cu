@@ -81,15 +81,14 @@ cudaError_t launch_attn_decode(const Dev& d, const Limits& lim, int layer, const
       !pool_tensor_maps(d, &map_lo, &map_hi))
     return cudaErrorInvalidValue;
   if (wide) {
-    const SliceCut cut = wide_cut(slots, n_pairs, pages);
-    const uint32_t tag = n_pairs * cut.k <= d.dec_tag_slots ? epoch : 0u;
-    return launch_attn_decode_split(d, true, layer, map_lo, map_hi, q, out, scale, cut, tag, new_k,
+    const int k = wide_slices(slots, n_pairs, pages);
+    const uint32_t tag = n_pairs * k <= d.dec_tag_slots ? epoch : 0u;
+    return launch_attn_decode_split(d, true, layer, map_lo, map_hi, q, out, scale, k, {}, tag, new_k,
                                     new_v, n_pairs, early, s);
   }
   if (narrow)
-    return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale,
-                                    narrow_cut(slots4, n_pairs, pages, esz == 4), 0u, new_k, new_v,
-                                    n_pairs, early, s);
+    return launch_attn_decode_split(d, false, layer, map_lo, map_hi, q, out, scale, most,
+                                    narrow_fit(slots4, n_pairs), 0u, new_k, new_v, n_pairs, early, s);
   return launch_attn_decode_streamk(d, layer, map_lo, map_hi, q, out, scale, lim.dec_stream_k,
                                     DEC_MIN_UNITS, new_k, new_v, early, s);
 }

@@ -1,11 +1,12 @@
 // Slices per (session, KV head) pair of the two pair-split decode shapes, by the pages of the
-// call's longest session.  Those of the 4-warp shape range from 1 to 14.  The host launches as
-// many CTAs as any number of pages can want, with the count for its estimate of the pages; a
-// kernel that finds other pages (nb_max of the append) works the count out again, and CTAs past
-// it leave at once.  So a launch that was captured with short sessions, or one whose sessions the
-// host estimates wrong, is cut for the pages that are there (8 pairs captured at one page and
-// replayed at 250: 48.2 us with the host's count).  That an append kernel works the count out
-// instead costs each of them 0.3 us.
+// call's longest session.  Those of the 4-warp shape range from 1 to 14 and follow from the pages
+// that are there (nb_max of the append): the host launches as many CTAs as any number of pages
+// can want, and CTAs past the count leave at once.  So a launch that was captured with short
+// sessions, or one whose sessions the host estimates wrong, is cut right (8 pairs captured at one
+// page and replayed at 250: 48.2 us with the host's count), and a captured launch is cut like an
+// eager one.  Each CTA counts for itself; that and the CTAs without a slice cost up to 0.1 us of
+// a launch, 0.4 where one slice in six is spare (72 pairs of 76 pages: 9.9 -> 10.3 us).  In the
+// append kernels the count cost each of them 0.3 us.
 // Those of the 16-warp shape hardly depend on the pages: they are the host's, as CTAs without a
 // slice would keep the next launch's off their SM (8 pairs of 257 pages: 7.5 us with 17 slices
 // launched, 7.9 with 19 of which 17 work).  Plain C++ beside CUDA, so that it is tested on the CPU.
@@ -62,7 +63,7 @@ KVC_HD inline NarrowFit narrow_fit(int slots, int n_pairs) {
 }
 KVC_HD inline int narrow_slices(const NarrowFit& fit, int pages, bool cuda_cores) {
   if (fit.most < 1) return 1;
-  const int n = pages + 2;  // (the figures above are of sessions whose first and last are partly filled)
+  const int n = pages + 1;  // (the figures above count whole pages)
   int k = pages < ALL_MIN_PAGES ? fit.below : fit.from;
   // Pages of a warp: ceil(ceil(n / k) / NARROW_WARPS).
   if (cuda_cores) {
@@ -72,27 +73,6 @@ KVC_HD inline int narrow_slices(const NarrowFit& fit, int pages, bool cuda_cores
   }
   k = at_least(1, at_most(k, div_up(n, NARROW_WARPS)));
   return k > 5 ? at_least(5, div_up(n, NARROW_WARPS * div_up(n, NARROW_WARPS * k))) : k;
-}
-
-// How a launch of a pair split is cut: `most` CTAs per pair, of which k work while the call's
-// longest session has lo to hi pages (16 warps: most = k, any number).
-struct SliceCut {
-  NarrowFit fit;
-  int most, k, lo, hi;
-};
-inline SliceCut wide_cut(int slots, int n_pairs, int pages) {
-  const int k = wide_slices(slots, n_pairs, pages);
-  return {{k, k, k}, k, k, 0, 1 << 30};
-}
-// `pages` estimated; a quarter and two pages more or less are not worth another count.
-inline SliceCut narrow_cut(int slots, int n_pairs, int pages, bool cuda_cores) {
-  const NarrowFit fit = narrow_fit(slots, n_pairs);
-  return {fit, fit.most, narrow_slices(fit, pages, cuda_cores), pages - pages / 4 - 2,
-          pages + pages / 4 + 2};
-}
-KVC_HD inline int cut_slices(const SliceCut& c, int pages, bool cuda_cores) {
-  const int k = pages < c.lo || pages > c.hi ? narrow_slices(c.fit, pages, cuda_cores) : c.k;
-  return at_least(1, at_most(k, c.most));
 }
 
 }  // namespace kvc

@@ -78,15 +78,16 @@ cudaError_t launch_attn_decode_streamk(const Dev& d, int layer, const CUtensorMa
                                        float scale, int grid, int min_units, const void* new_k,
                                        const void* new_v, bool early, cudaStream_t s);
 // Pair-split decode kernel (kvc_attn_decode_split.cu).  wide: the 16-warp shape
-// (one CTA per SM; tensor-core pages for bfloat16), else the 4-warp shape.
+// (one CTA per SM; tensor-core pages for bfloat16), else the 4-warp shape.  k_most: CTAs per
+// pair; fit: how the 4-warp shape counts those that work.
 // Resident CTAs in one wave (sets its attributes).
 int decode_split_slots(int esz, bool wide, int sms);
 bool decode_split_uses_tma(int esz, bool wide);      // needs the pool's tensor maps
 cudaError_t launch_attn_decode_split(const Dev& d, bool wide, int layer, const CUtensorMap& map_lo,
                                      const CUtensorMap& map_hi, const void* q, void* out,
-                                     float scale, const SliceCut& cut, uint32_t epoch,
-                                     const void* new_k, const void* new_v, int n_pairs, bool early,
-                                     cudaStream_t s);
+                                     float scale, int k_most, const NarrowFit& fit,
+                                     uint32_t epoch, const void* new_k, const void* new_v,
+                                     int n_pairs, bool early, cudaStream_t s);
 // new_k / new_v (optional, bfloat16 only): the chunk's rows of this layer, written
 // into the pool by the launch itself (the per-layer order).
 // pages_max, pages_sum: estimates of the sessions' resident pages (largest, sum over the

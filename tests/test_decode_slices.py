@@ -1,6 +1,6 @@
 """Slices per pair of the pair-split decode (csrc/kvc_decode_slices.h), over every number of pairs
 and pages: the rule in closed form, as the kernels evaluate it, against the rule as a search,
-and a launch's slices for pages other than the host's estimate within what it launches.
+and within what the host launches.
 """
 import os
 import subprocess
@@ -14,7 +14,7 @@ using namespace kvc;
 
 // The 4-warp rule by trying slice after slice.
 int narrow_search(int slots, int n_pairs, int pages, bool cuda_cores) {
-  const int all = std::min(NARROW_MAX, slots / n_pairs), x = pages + 2;
+  const int all = std::min(NARROW_MAX, slots / n_pairs), x = pages + 1;
   auto warp_pages = [&](int k) { return ((x + k - 1) / k + 3) / 4; };
   const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs;
   int k = std::min(all, five_sixths >= (pages < 300 ? 6 : 8) ? five_sixths : all);
@@ -48,22 +48,6 @@ int main() {
           return 1;
         }
       }
-    for (int n_pairs : {1, 2, 8, 16, 24, 48, 72, 100, 160, 320, 456})
-      for (int est = 1; est <= 700; est += est < 40 ? 1 : 13)
-        for (int pages = 1; pages <= 700; pages += pages < 40 ? 1 : 7)
-          for (int cc = 0; cc < 2 && n_pairs <= 3 * sms; ++cc) {
-            const SliceCut c = narrow_cut(3 * sms, n_pairs, est, cc);
-            const int k = cut_slices(c, pages, cc);
-            const bool near = 4 * pages >= 3 * est - 12 && 4 * pages <= 5 * est + 8;
-            const int here = narrow_slices(c.fit, pages, cc), there = narrow_slices(c.fit, est, cc);
-            if (c.most != narrow_most(3 * sms, n_pairs) || k < 1 || k > c.most ||
-                (!near && k != here) || (pages == est && k != there) || (k != here && k != there)) {
-              std::printf("%d SMs, %d pairs, %d pages for %d: %d\n", sms, n_pairs, pages, est, k);
-              return 2;
-            }
-          }
-    const SliceCut w = wide_cut(sms, 1, 300);
-    if (w.most != w.k || cut_slices(w, 1, false) != w.k || cut_slices(w, 1 << 20, true) != w.k) return 3;
   }
   return 0;
 }
