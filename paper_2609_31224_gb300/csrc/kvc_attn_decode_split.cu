@@ -166,8 +166,8 @@ __device__ inline void drain_after_failure(const Dev& d, const Smem<C>& sm, cons
 
 // ---------------------------------------------------------------------------
 // Pair-split kernel (few sessions): a CTA takes one of the k <= k_most equal slices of a pair's
-// pages.  16 warps: k = k_most, the grid is flat.  4 warps: k follows the pages, the grid
-// is (k_most, pairs), so that the count is not followed by a division of the block index, and
+// pages.  16 warps: k = k_most, the grid is flat.  4 warps: k follows the pair's pages, the
+// grid is (k_most, pairs), so that the count is not followed by a division of the block index, and
 // CTAs past k leave at once.  Each CTA's pages are issued before it waits on the previous
 // kernel; the k partial states of
 // a pair are merged by the last of its CTAs to finish.
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(C::THREADS) attn_decode_split_kernel(
 
   const SeqInfo si = d.seq[seq];
   int k = k_most;
-  if constexpr (!WIDE) k = narrow_slices(cut, d.g->nb_max, sizeof(T) == 4);
+  if constexpr (!WIDE) k = narrow_slices(cut, si.n_blocks, sizeof(T) == 4);
   if (!WIDE && slice >= k) return;
   const int nb = si.n_blocks;
   const int b0 = (int)((int64_t)slice * nb / k), b1 = (int)((int64_t)(slice + 1) * nb / k);

@@ -1,16 +1,17 @@
-// Slices per (session, KV head) pair of the two pair-split decode shapes, by the pages of the
-// call's longest session.  Those of the 4-warp shape range from 1 to 14 and follow from the pages
-// that are there (nb_max of the append): the host launches as many CTAs as any number of pages
-// can want, and CTAs past the count leave at once.  So a launch that was captured with short
-// sessions, or one whose sessions the host estimates wrong, is cut right (8 pairs captured at one
-// page and replayed at 250: 48.2 us with the host's count), and a captured launch is cut like an
-// eager one.  Each CTA counts for itself; that and the CTAs without a slice cost up to 0.1 us of
-// a launch, 0.4 where one slice in six is spare (72 pairs of 76 pages: 9.9 -> 10.3 us).  In the
-// append kernels the count cost each of them 0.3 us.
+// Slices per (session, KV head) pair of the two pair-split decode shapes.  Those of the 4-warp
+// shape range from 1 to 14 and follow from the pages of the pair's session: the host launches as
+// many CTAs as any number of pages can want, each counts the slices for itself, and those past
+// the count leave at once.  So a launch that was captured with short sessions, or one whose
+// sessions the host estimates wrong, is cut right (8 pairs captured at one page and replayed at
+// 250: 48.2 us with the host's count), and a captured launch is cut like an eager one.  (The count
+// in the append kernels cost each of them 0.3 us; from the call's longest session, one address
+// that every CTA reads, it cost a decode launch up to 0.3.)
 // Those of the 16-warp shape hardly depend on the pages: they are the host's, as CTAs without a
 // slice would keep the next launch's off their SM (8 pairs of 257 pages: 7.5 us with 17 slices
 // launched, 7.9 with 19 of which 17 work).  Plain C++ beside CUDA, so that it is tested on the CPU.
 #pragma once
+
+#include <stdint.h>
 
 #ifdef __CUDACC__
 #define KVC_HD __host__ __device__
@@ -51,28 +52,41 @@ KVC_HD inline int wide_slices(int slots, int n_pairs, int pages) {
 // at 8; 24 pairs: 5.0 and 5.2), and more slices if they save a warp one (48 pairs of 130
 // pages: 12.0 us at 9 slices, 12.5 at 8).
 //
-// What follows from the pairs alone is the host's part, so that a kernel is left with two divisions.
+// What follows from the pairs alone is the host's part.  A kernel is left with one division, for
+// long sessions: it comes before a CTA's first load, and three of them took 0.1-0.4 us.
+struct WarpPages {  // pages of a warp with k slices: n / (4 k) rounded up, as a product
+  int d;            // 4 k
+  uint32_t inv;     // 2^32 / d rounded up: exact up to 2^32 / d pages
+  KVC_HD int of(int n) const { return (int)(((uint64_t)(uint32_t)(n + d - 1) * inv) >> 32); }
+};
+inline WarpPages warp_pages(int k) {
+  const int d = NARROW_WARPS * (k > 0 ? k : 1);
+  return {d, (uint32_t)(((1ull << 32) + d - 1) / d)};
+}
 struct NarrowFit {
   int most;         // slices that the slots and NARROW_MAX allow
   int below, from;  // of sessions below, and from, ALL_MIN_PAGES pages on
+  WarpPages w_most, w_below, w_from;
 };
-KVC_HD inline NarrowFit narrow_fit(int slots, int n_pairs) {
+inline NarrowFit narrow_fit(int slots, int n_pairs) {
   const int most = narrow_most(slots, n_pairs);
   const int five_sixths = (slots * 5 / 6 + n_pairs / 2) / n_pairs, some = at_most(most, five_sixths);
-  return {most, five_sixths >= 6 ? some : most, five_sixths >= 8 ? some : most};
+  const int below = five_sixths >= 6 ? some : most, from = five_sixths >= 8 ? some : most;
+  return {most, below, from, warp_pages(most), warp_pages(below), warp_pages(from)};
 }
 KVC_HD inline int narrow_slices(const NarrowFit& fit, int pages, bool cuda_cores) {
-  if (fit.most < 1) return 1;
   const int n = pages + 1;  // (the figures above count whole pages)
-  int k = pages < ALL_MIN_PAGES ? fit.below : fit.from;
-  // Pages of a warp: ceil(ceil(n / k) / NARROW_WARPS).
+  const bool shorter = pages < ALL_MIN_PAGES;
+  const int k = shorter ? fit.below : fit.from;
+  const int w = (shorter ? fit.w_below : fit.w_from).of(n);
+  const int quarter = (n + NARROW_WARPS - 1) / NARROW_WARPS;  // slices with a page per warp
   if (cuda_cores) {
-    const int w = div_up(n, NARROW_WARPS * fit.most);
-    if (w < div_up(n, NARROW_WARPS * k)) k = div_up(n, NARROW_WARPS * w);
-    return at_least(1, at_most(k, n / 2));
+    const int w_most = fit.w_most.of(n);
+    const int more = w_most >= w ? k : w_most == 1 ? quarter : div_up(quarter, w_most);
+    return at_least(1, at_most(more, n / 2));
   }
-  k = at_least(1, at_most(k, div_up(n, NARROW_WARPS)));
-  return k > 5 ? at_least(5, div_up(n, NARROW_WARPS * div_up(n, NARROW_WARPS * k))) : k;
+  if (quarter <= k) return quarter;
+  return k > 5 ? at_least(5, div_up(quarter, w)) : at_least(1, k);
 }
 
 }  // namespace kvc

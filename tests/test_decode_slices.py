@@ -31,7 +31,8 @@ int narrow_search(int slots, int n_pairs, int pages, bool cuda_cores) {
 int main() {
   for (int sms : {152, 148, 132, 7}) {
     for (int n_pairs = 1; n_pairs <= 3 * sms; ++n_pairs)
-      for (int pages = 1; pages <= 1100; ++pages) {
+      for (int at = 1; at <= 1120; ++at) {
+        const int pages = at <= 1100 ? at : (1 << 20) + 3 * at - 3400;  // (a session has 2^20 and a few)
         for (int cc = 0; cc < 2; ++cc) {
           const int k = narrow_slices(narrow_fit(3 * sms, n_pairs), pages, cc);
           if (k != narrow_search(3 * sms, n_pairs, pages, cc) || k < 1 ||
