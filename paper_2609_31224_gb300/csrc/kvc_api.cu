@@ -165,6 +165,7 @@ struct kvc_ctx {
   int64_t used_ub = 0;            // upper bound of pages in use after enqueued work
   int64_t delta_since_readback = 0;
   bool readback_pending = false;
+  bool captured_readback = false;  // a graph holds a launch that writes h_readback
   cudaEvent_t ev = nullptr;
   int64_t* h_readback = nullptr;  // pinned, written by evict and release
   Limits lim = {};  // of the device that it was created on
@@ -246,7 +247,15 @@ cudaError_t next_decode_epoch(kvc_ctx* ctx, cudaStream_t s, bool capturing, uint
 
 // The launch just enqueued writes the pages in use to h_readback itself: a copy in the stream
 // would cost 6 us of submission and keep the next append from starting early.
+// A captured launch is not in the stream yet and its event cannot be waited for: the word is taken
+// behind eager launches only.  (A replay may have written it since: a later count, so that with
+// the pages added since the eager launch it is still an upper bound.)
 void enqueue_readback(kvc_ctx* ctx, cudaStream_t s) {
+  bool capturing = false;
+  if (is_capturing(s, &capturing) != cudaSuccess || capturing) {
+    ctx->captured_readback = true;
+    return;
+  }
   cudaEventRecord(ctx->ev, s);
   ctx->readback_pending = true;
   ctx->delta_since_readback = 0;
@@ -342,7 +351,8 @@ int kvc_create(kvc_ctx** out, const kvc_config* cfg, void* d_pool, size_t pool_b
 
 void kvc_destroy(kvc_ctx* ctx) {
   if (!ctx) return;
-  // The last evict or release may still have to write h_readback.
+  // The last evict or release, or a replayed one, may still have to write h_readback.
+  if (ctx->captured_readback) cudaDeviceSynchronize();
   if (ctx->ev) {
     cudaEventSynchronize(ctx->ev);
     cudaEventDestroy(ctx->ev);
@@ -451,6 +461,7 @@ int kvc_evict(kvc_ctx* ctx, int n_seq, const int32_t* h_sessions, int64_t* d_res
   KVC_CUDA(launch_evict(ctx->d, a, d_resident_out, ctx->h_readback, ctx->lim.sms, s));
   for (int i = 0; i < n_seq; ++i) ctx->resident[h_sessions[i]].evict(ctx->cfg);
   ctx->used_ub += n_seq;  // an evict adds at most one page per session, net
+  ctx->delta_since_readback += n_seq;
   enqueue_readback(ctx, s);
   ctx->attn_valid = false;
   return KVC_OK;
